@@ -11,8 +11,9 @@ Each case is one kind of call at one size, through the Python layer:
   icp         Scene.icp_poses: given poses refined against a live depth frame;
   train       a forest adapted to a room from posed frames, all leaves clustered,
               its modes read back;
-  track       the online loop: posed frames adapted one by one with a budget of
-              leaves re-clustered per frame, then a lost frame relocalised.
+  track       the online loop from empty leaves: posed frames adapted one by one
+              with a budget of leaves re-clustered per frame, then a lost frame
+              relocalised.
 
 Inputs are rendered on the GPU from the seed: an axis-aligned box room tiled
 with 8 cm cells of random colour, a training trajectory round the room, query
@@ -90,9 +91,9 @@ def listed():
         # a forest adapted to a room and clustered whole
         dict(name="train 24 frames", kind="train", **_size(640, 480, room=1),
              **_forest(depth=11, m_max=10, frames=24)),
-        # eight tracked frames of the online loop, then a lost one
-        dict(name="track 8 frames", kind="track", **_size(640, 480), **_forest(depth=13, frames=48),
-             **_reloc("default", 1), steps=8, budget=256),
+        # a room mapped online, then a lost frame
+        dict(name="track 16 frames", kind="track", **_size(640, 480), **_forest(depth=12, min_size=5, frames=16),
+             **_reloc("default", 1), budget=2048),
     ]
 
 
@@ -115,7 +116,7 @@ def draw(rng):
     if kind == "train":
         return dict(kind=kind, **size, **_forest(trees=rng.randint(1, 5), depth=rng.randint(7, 11),
                                                  kappa=_log(rng, 100, 1024), m_max=rng.randint(4, 12),
-                                                 min_size=rng.randint(2, 20), tau_c=round(rng.uniform(0.03, 0.2), 3),
+                                                 min_size=rng.randint(2, 12), tau_c=round(rng.uniform(0.05, 0.2), 3),
                                                  fp16=rng.random() < 0.7, frames=rng.randint(4, 24)))
     # frames to train on, and leaves that hold 25 to 80 of their grid pixels each: fewer leave no modes
     frames = rng.randint(30, 80)
@@ -128,17 +129,19 @@ def draw(rng):
     if kind == "serve":
         return dict(kind=kind, **size, **forest, batch=_log(rng, 2, 32), max_batch=rng.randint(2, 16))
     if kind == "track":
+        forest.update(frames=min(frames, 32), depth=max(7, min(13, depth - 1)))
         return dict(kind=kind, **size, **forest, **_reloc("default", 1, n_hyp=_log(rng, 128, 1024), loose=True),
-                    steps=rng.randint(2, 8), budget=_log(rng, 100, 2048))
+                    budget=_log(rng, 256, 4096))
     wide = rng.random() < 0.2  # most or all stored modes used
     batch = _log(rng, 1, max(1, min(64, (2 if wide else 32) * 307200 // pixels)))
     preset = rng.choice(["default", "paper", "paper", "fast", "intermediate", "slow"])
-    few = preset in ("fast", "intermediate", "slow")  # few generation iterations: the loose checks find triples
+    trees = rng.randint(1, forest["trees"])
+    # few generation iterations or few modes: only the loose checks find triples
+    few = preset in ("fast", "intermediate", "slow") or trees < 3
     return dict(kind=kind, **size, **forest, **_reloc(
-        preset, batch, n_hyp=_log(rng, 128, 2048), eta=_log(rng, 48, 512),
-        k_top=rng.randint(16, 50) if wide else rng.randint(5, 11),
-        trees_used=rng.randint(1, forest["trees"]), icp=rng.random() < 0.15, redraw=rng.random() < 0.2,
-        loose=few or rng.random() < 0.5))
+        preset, batch, n_hyp=_log(rng, 192, 2048), eta=_log(rng, 48, 512),
+        k_top=rng.randint(16, 50) if wide else rng.randint(5, 11), trees_used=trees, icp=rng.random() < 0.15,
+        redraw=rng.random() < 0.2, loose=few or rng.random() < 0.5))
 
 
 # ---- inputs ---------------------------------------------------------------
@@ -286,14 +289,16 @@ def _forest_bytes(case):
     return (case["trees"] << case["depth"]) * (case["kappa"] * 16 + case["m_max"] * 120 + 128) + (64 << 20)
 
 
-def _trained(s, stream=False):
-    """The case's forest, adapted to the room from posed frames, every leaf clustered."""
+def _random_forest(s):
     c = s.case
-    f = s.keep(rg.Forest.random(s.ctx, dict(
+    return s.keep(rg.Forest.random(s.ctx, dict(
         n_trees=c["trees"], depth=c["depth"], kappa=c["kappa"], m_max=c["m_max"], min_cluster_size=c["min_size"],
         tau_c=c["tau_c"], mode_precision=int(c["fp16"])), int(s.rng.integers(1 << 40))))
-    if stream:
-        f.set_streaming(True)
+
+
+def _trained(s):
+    """The case's forest, adapted to the room from posed frames, every leaf clustered."""
+    c, f = s.case, _random_forest(s)
     poses = _trajectory(s.room.size, c["frames"], s.rng)
     for k in range(0, len(poses), 32):
         depth, rgb = s.room.render(s.K, poses[k:k + 32], c["missing"])
@@ -315,10 +320,7 @@ def prepare(case, seed):
         return s
     if kind == "train":
         s = _State(case, seed, _forest_bytes(case) + (256 << 20))
-        s.forest = s.keep(rg.Forest.random(s.ctx, dict(
-            n_trees=case["trees"], depth=case["depth"], kappa=case["kappa"], m_max=case["m_max"],
-            min_cluster_size=case["min_size"], tau_c=case["tau_c"], mode_precision=int(case["fp16"])),
-            int(s.rng.integers(1 << 40))))
+        s.forest = _random_forest(s)
         s.poses = _trajectory(s.room.size, case["frames"], s.rng)
         s.depth, s.rgb = s.room.render(s.K, s.poses, case["missing"])
         return s
@@ -327,7 +329,11 @@ def prepare(case, seed):
     room_for = [dict(p, n_trees_used=min(p["n_trees_used"], case["trees"])) for p in room_for]
     s = _State(case, seed, int(1.1 * (_forest_bytes(case) + sum(_frame_bytes(case, p, slots) for p in room_for))) +
                (256 << 20))
-    s.forest = _trained(s, stream=kind == "track")
+    if kind == "track":
+        s.forest = _random_forest(s)
+        s.forest.set_streaming(True)
+    else:
+        s.forest = _trained(s)
     s.scene = s.keep(rg.Scene(s.ctx, np.zeros(3), s.room.size))
     s.seeds = [int(x) for x in s.rng.integers(1 << 40, size=n)]
     W, H = case["width"], case["height"]
@@ -349,9 +355,12 @@ def prepare(case, seed):
     else:
         s.reloc = s.keep(rg.Relocaliser(s.forest, s.scene, room_for[0], W, H, n))
     if kind == "track":
-        s.poses = _queries(case, case["steps"], s.rng)
+        s.poses = _trajectory(s.room.size, case["frames"], s.rng)
         s.tracked = s.room.render(s.K, s.poses, case["missing"])
-    s.depth, s.rgb = s.room.render(s.K, _queries(case, n, s.rng), case["missing"])
+        lost = _near([s.poses[case["frames"] // 2]], s.room.size, s.rng, 0.2, 10.0)
+    else:
+        lost = _queries(case, n, s.rng)
+    s.depth, s.rgb = s.room.render(s.K, lost, case["missing"])
     return s
 
 
@@ -391,6 +400,7 @@ def run(state):
         e = f.export()
         return {k: e[k] for k in ("res_count", "nmodes", "mode_pos", "mode_rgb", "mode_U", "mode_size")}
     if kind == "track":
+        state.forest.reset_leaves()
         for d, r, T in zip(*state.tracked, state.poses):
             state.forest.adapt(d, r, state.K, T)
             state.forest.update_modes(state.case["budget"])
@@ -432,11 +442,10 @@ def work(case):
         return {"bytes": pixels * 4 + case["poses"] * 264,
                 "flops": case["poses"] * pixels * (6 / 16 + 3 / 4 + 2) * ICP_PIXEL}
     if kind in ("train", "track"):
-        frames = case["frames"] if kind == "train" else case["steps"]
-        grid = (pixels + 15) // 16
+        frames, grid = case["frames"], (pixels + 15) // 16
         leaves = case["trees"] << case["depth"]
-        done = leaves if kind == "train" else min(leaves, case["budget"] * frames)
-        seen = frames if kind == "train" else case["frames"] + frames
+        done = leaves if kind == "train" else case["budget"] * frames
+        seen = frames if kind == "train" else frames / 2
         points = min(case["kappa"], seen * grid * case["trees"] / leaves)  # in a mean leaf
         byte = frames * grid * 7 + done * (points * 16 + case["m_max"] * 43)
         flops = frames * grid * case["trees"] * case["depth"] * NODE + done * points * points * 20
