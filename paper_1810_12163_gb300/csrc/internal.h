@@ -100,7 +100,9 @@ struct rl_forest {
     // adaptation scratch
     uint32_t *ex_leaf = nullptr;    // [T][grid pixels]
     float4 *ex_pt = nullptr;        // [grid pixels]
-    uint32_t *ex_rank = nullptr;    // [T][grid pixels]
+    uint32_t *ex_rank = nullptr;    // [T][grid pixels] arrival number; then the slots by list entry
+    uint32_t *ex_list = nullptr;    // [T][grid pixels] examples by leaf; then [16] entries used per tree
+    uint2 *ex_seg = nullptr;        // [L] (first entry, length) of the leaf's examples in ex_list
     uint32_t *frame_cnt = nullptr;  // [L]
     int ex_capacity = 0;
     float *stage_depth = nullptr;
