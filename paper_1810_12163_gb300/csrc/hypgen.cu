@@ -8,6 +8,8 @@
 // (FP64 from FP32 inputs) are plain IEEE operations in a fixed order, so
 // every accept/reject decision, and therefore the winning iteration of each
 // slot, is exactly reproducible.
+#include <limits.h>
+
 #include "hypgen_dev.cuh"
 #include "kernels.h"
 
@@ -133,6 +135,51 @@ __device__ __forceinline__ void stage1_bits2(const HypArgs &a, const Frame &fr, 
     sB = decide(okB, wB, rB, dB);
 }
 
+// |M(u)| of a pixel record.
+__device__ __forceinline__ int rec_modes(const uint4 &rec, int n_trees) {
+    int c = 0;
+    for (int t = 0; t < n_trees; ++t) c += rec_count(rec, t);
+    return c;
+}
+
+// The same for more modes per pixel than the masks cover: the checked
+// pixel's record gives its mode, and the mode's colour is compared with the
+// pixel's.  Only the checked pixel's record is gathered, where a general
+// attempt reads all three: 4 frames of 4096 slots and up to 250 modes per
+// pixel 1.95 ms, 3.97 by the general path.
+template <int REDRAW>
+__device__ __forceinline__ void stage1_rec2(const HypArgs &a, const Frame &fr, const uint4 *pr,
+                                            const uint32_t *s_bits, int slot, int itA, int itB, Draw &dA, Draw &dB,
+                                            bool &sA, bool &sB) {
+    auto usable = [&](int q) { return bit_set(s_bits, q); };
+    dA = draw<decltype(usable), REDRAW>(a, fr, slot, itA, usable);
+    dB = draw<decltype(usable), REDRAW>(a, fr, slot, itB, usable);
+    const int pA = dA.j == 0 ? dA.pix[0] : (dA.j == 1 ? dA.pix[1] : dA.pix[2]);
+    const int pB = dB.j == 0 ? dB.pix[0] : (dB.j == 1 ? dB.pix[1] : dB.pix[2]);
+    const uint4 wA = pr[pA], wB = pr[pB];
+    const uint8_t *cA = fr.rgb + (size_t)pA * 3, *cB = fr.rgb + (size_t)pB * 3;
+    const int3 colA = make_int3(cA[0], cA[1], cA[2]), colB = make_int3(cB[0], cB[1], cB[2]);
+    const bool okA = bit_set(s_bits, dA.pix[0]) && bit_set(s_bits, dA.pix[1]) && bit_set(s_bits, dA.pix[2]);
+    const bool okB = bit_set(s_bits, dB.pix[0]) && bit_set(s_bits, dB.pix[1]) && bit_set(s_bits, dB.pix[2]);
+    const uint32_t ctr1 = (TAG_HYP << 16) | (uint32_t)a.p.level;
+    const uint4 rA = philox(make_uint4(slot, ctr1, itA, 1), fr.key0, fr.key1);
+    const uint4 rB = philox(make_uint4(slot, ctr1, itB, 1), fr.key0, fr.key1);
+    auto mode_of = [&](const uint4 &w, const uint4 &r, const Draw &d) {
+        const uint32_t rj = d.j == 0 ? r.x : (d.j == 1 ? r.y : r.z);
+        uint32_t L;
+        int rank;
+        mode_at_rec(w, a.p.n_trees, a.mv.leaves_per_tree, (int)draw_below(rj, (uint32_t)rec_modes(w, a.p.n_trees)), &L,
+                    &rank);
+        return a.mv.mrgb[(size_t)L * a.mv.m_max + rank];  // (0, 0) for an empty M(u)
+    };
+    const uchar4 mA = mode_of(wA, rA, dA), mB = mode_of(wB, rB, dB);
+    auto passes = [&](const int3 &c, const uchar4 &m) {
+        return max(abs(c.x - (int)m.x), max(abs(c.y - (int)m.y), abs(c.z - (int)m.z))) <= a.p.colour_thresh;
+    };
+    sA = okA && passes(colA, mA);
+    sB = okB && passes(colB, mB);
+}
+
 // rec, dep: the three pixels' records and depths when already gathered
 // (else read here).
 __device__ __forceinline__ bool stage2(const HypArgs &a, const CheckThr &ct, const Frame &fr,
@@ -182,30 +229,51 @@ __device__ __forceinline__ bool stage2(const HypArgs &a, const CheckThr &ct, con
 // lanes converged on the rarely reached stage 2.
 constexpr int HG_RING = 128;  // < 32 pending after a drain + 64 appended
 
-// WARPS slots per block; registers stay capped at 64 (32 warps per SM).
-template <int WARPS, int REDRAW>
+// WARPS warps per block; registers stay capped at 64 (32 warps per SM).
+// A slot is served by a.team warps of a block, which take its groups of
+// iterations in turn: with few slots in a call (a frame that lost track) one
+// warp per slot leaves most of the GPU idle and walks 94 groups one after
+// the other.  A warp stops at its first success, or when its next group lies
+// behind another's; the lowest success of the team is the slot's.  The team
+// grows while the call's slots times the team fit the GPU's 32 warps per SM:
+// one 640x480 frame of 1024 slots 95 us with teams of four (189 alone), a
+// 160x120 frame of 64 slots 37 us with teams of 16 (383).  More warps than
+// fit would only repeat the work of slots that succeed early.
+//
+// PATH: how stage 1 learns whether a pixel is usable and its colour matches,
+// fixed at compile time so that no path pays for another's registers.
+enum HypPath {
+    HYP_GENERAL,    // pixel records or leaf maps
+    HYP_MASKS_ONLY, // colour-check masks (frames whose bitmap is too large)
+    HYP_MASKS,      // bitmap in shared memory, colour-check masks
+    HYP_RECORDS     // bitmap in shared memory, pixel records
+};
+
+template <int WARPS, int REDRAW, int PATH>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
     constexpr int HG_WARPS = WARPS;
     __shared__ int4 s_ring[HG_WARPS][HG_RING];   // it | j << 30, pixels of the triple
-    __shared__ uint2 s_mode[HG_WARPS][HG_RING];  // mode indices m0 | m1 << 16, m2 (without the bitmap)
-    extern __shared__ uint32_t s_bits[];         // the frame's non-empty-M(u) bitmap (with pbits)
+    __shared__ int s_best[HG_WARPS];             // lowest successful iteration of each slot so far
+    // with the bitmap: the frame's non-empty-M(u) bitmap; without: per ring
+    // entry its mode indices m0 | m1 << 16, m2
+    extern __shared__ __align__(8) uint32_t s_bits[];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int slot = blockIdx.x * HG_WARPS + w;
+    const int team = a.team, mate = w % team, sl = w / team;  // the slot's warps, this one, the block's slot
+    const int slot = blockIdx.x * (HG_WARPS / team) + sl;
     const int b = blockIdx.y;
     const Frame fr = a.frames[b];
-    const bool use_bits = a.pbits != nullptr && a.pcm != nullptr;
-    if (use_bits) {  // every thread of the block stages the bitmap, before any may leave
+    if (fr.W * fr.H == 0) {  // empty frame (e.g. accepted by an earlier cascade level)
+        if (mate == 0 && lane == 0 && slot < a.p.n_hyp) a.hyp_iter[(size_t)b * a.p.n_hyp + slot] = -1;
+        return;
+    }
+    constexpr bool use_bits = PATH == HYP_MASKS || PATH == HYP_RECORDS;
+    if (use_bits) {  // every thread of the block stages the bitmap
         const int nw = (fr.W * fr.H + 31) >> 5;
         const uint32_t *src = a.pbits + (size_t)b * (a.hw_max / 32 + 1);
         for (int k = threadIdx.x; k < nw; k += blockDim.x) s_bits[k] = src[k];
-        __syncthreads();
     }
-    if (slot >= a.p.n_hyp) return;
-    int32_t *iter_out = a.hyp_iter + (size_t)b * a.p.n_hyp + slot;
-    if (fr.W * fr.H == 0) {  // empty frame (e.g. accepted by an earlier cascade level)
-        if (lane == 0) *iter_out = -1;
-        return;
-    }
+    if (threadIdx.x < HG_WARPS) s_best[threadIdx.x] = INT_MAX;
+    __syncthreads();
     const uint16_t *lv = a.leaves + (size_t)b * a.p.n_trees * a.hw_max;
     const uint16_t *mc = a.mcount + (size_t)b * a.hw_max;
     const uint4 *pr = a.prec ? a.prec + (size_t)b * a.hw_max : nullptr;
@@ -215,7 +283,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
     ct.sq_hi = __double2float_ru(a.p.min_sq_dist * (1.0 + 2e-5));
     ct.tol = (float)a.p.max_trans_err;
     int4 *ring = s_ring[w];
-    uint2 *rmode = s_mode[w];
+    uint2 *rmode = (uint2 *)s_bits + w * HG_RING;
     unsigned head = 0, tail = 0;  // warp-uniform ring counters
     const unsigned lt = (1u << lane) - 1u;
     // Stage 2 on the pending entries head .. head + n - 1 (n <= 32); the
@@ -237,18 +305,20 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
             const int pix[3] = {r.y, r.z, r.w};
             it = r.x & 0x3fffffff;
             int m[3];
-            if (use_bits && pr) {
+            if (use_bits) {
                 // every gather that depends on the pixels alone, issued
-                // together: |M(u)|, the pixel records and the depths; then
-                // the mode draws of the attempt from its second Philox block
+                // together: |M(u)| (where there are masks), the pixel records
+                // and the depths; then the mode draws of the attempt from its
+                // second Philox block
                 uint32_t c3[3];
                 uint4 rec[3];
                 float dep[3];
 #pragma unroll
                 for (int i = 0; i < 3; ++i) {
-                    c3[i] = cm[pix[i]].y >> 24;
+                    if (PATH == HYP_MASKS) c3[i] = cm[pix[i]].y >> 24;
                     rec[i] = pr[pix[i]];
                     dep[i] = fr.depth[pix[i]];
+                    if (PATH != HYP_MASKS) c3[i] = (uint32_t)rec_modes(rec[i], a.p.n_trees);
                 }
                 const uint32_t ctr1 = (TAG_HYP << 16) | (uint32_t)a.p.level;
                 const uint4 r1 = philox(make_uint4(slot, ctr1, it, 1), fr.key0, fr.key1);
@@ -257,23 +327,15 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
                 m[2] = (int)draw_below(r1.z, c3[2]);
                 ok = stage2(a, ct, fr, lv, pr, pix, m, rec, dep);
             } else {
-                if (use_bits) {
-                    const uint32_t ctr1 = (TAG_HYP << 16) | (uint32_t)a.p.level;
-                    const uint4 r1 = philox(make_uint4(slot, ctr1, it, 1), fr.key0, fr.key1);
-                    m[0] = (int)draw_below(r1.x, cm[pix[0]].y >> 24);
-                    m[1] = (int)draw_below(r1.y, cm[pix[1]].y >> 24);
-                    m[2] = (int)draw_below(r1.z, cm[pix[2]].y >> 24);
-                } else {
-                    const uint2 mm = rmode[e];
-                    m[0] = (int)(mm.x & 0xffffu);
-                    m[1] = (int)(mm.x >> 16);
-                    m[2] = (int)mm.y;
-                }
+                const uint2 mm = rmode[e];
+                m[0] = (int)(mm.x & 0xffffu);
+                m[1] = (int)(mm.x >> 16);
+                m[2] = (int)mm.y;
                 ok = stage2(a, ct, fr, lv, pr, pix, m);
             }
         }
         const unsigned win = __ballot_sync(0xffffffffu, ok);
-        if (win && lane == __ffs(win) - 1) *iter_out = it;
+        if (win && lane == __ffs(win) - 1) atomicMin(&s_best[sl], it);
         head += n;
         return win != 0;
     };
@@ -286,16 +348,24 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
         }
         tail += __popc(mask);
     };
-    // iterations in groups of 64 (masks: two per lane) or 32; survivors are
-    // appended in iteration order
-    const int step = cm ? 64 : 32;
-    for (int base = 0; base < a.p.max_iter; base += step) {
-        if (cm) {
+    // iterations in groups of 64 (two per lane) or 32, every team-th group by
+    // this warp; survivors are appended in iteration order
+    constexpr bool pairs = PATH != HYP_GENERAL;
+    constexpr int step = pairs ? 64 : 32;
+    bool done = slot >= a.p.n_hyp;
+    for (int base = mate * step; base < a.p.max_iter && !done; base += team * step) {
+        if (*(volatile int *)&s_best[sl] < base) {  // a team mate's success comes first
+            head = tail;
+            break;
+        }
+        if (pairs) {
             Draw dA, dB;
             bool sA, sB;
             const int itA = base + lane, itB = base + 32 + lane;
-            if (use_bits)
+            if (PATH == HYP_MASKS)
                 stage1_bits2<REDRAW>(a, fr, cm, s_bits, slot, itA, itB, dA, dB, sA, sB);
+            else if (PATH == HYP_RECORDS)
+                stage1_rec2<REDRAW>(a, fr, pr, s_bits, slot, itA, itB, dA, dB, sA, sB);
             else
                 stage1_mask2<REDRAW>(a, fr, cm, slot, itA, itB, dA, dB, sA, sB);
             append(sA && itA < a.p.max_iter, itA, dA);
@@ -308,16 +378,18 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
         }
         n_att += (unsigned)min(step, a.p.max_iter - base);
         __syncwarp();
-        while (tail - head >= 32) {
-            if (drain(32)) {
-                count();
-                return;
-            }
+        while (tail - head >= 32 && !done) {
+            done = drain(32);
             __syncwarp();
         }
     }
-    if (!(tail - head > 0 && drain(tail - head)) && lane == 0) *iter_out = -1;
+    if (!done && tail - head > 0) drain(tail - head);
     count();
+    __syncthreads();
+    if (mate == 0 && lane == 0 && slot < a.p.n_hyp) {
+        const int it = s_best[sl];
+        a.hyp_iter[(size_t)b * a.p.n_hyp + slot] = it == INT_MAX ? -1 : it;
+    }
 }
 
 // Colour-check masks (Sec. 3.2.3, check 1 precomputed): bit m of pixel u is
@@ -360,6 +432,25 @@ __global__ void __launch_bounds__(256) k_colour_mask(const Frame *__restrict__ f
         }
     }
     pcm[o] = make_uint2(lo, hi | ((uint32_t)cnt << 24));
+}
+
+// The non-empty-M(u) bitmap alone, for more modes per pixel than the masks cover.
+__global__ void __launch_bounds__(256) k_mode_bits(const Frame *__restrict__ frames, const uint4 *__restrict__ prec,
+                                                   int hw_max, int n_trees, uint32_t *__restrict__ pbits) {
+    const int b = blockIdx.y;
+    const Frame fr = frames[b];
+    const int px = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = px < fr.W * fr.H;
+    const bool some = in && rec_modes(prec[(size_t)b * hw_max + px], n_trees) > 0;
+    const unsigned word = __ballot_sync(0xffffffffu, some);
+    if (in && (threadIdx.x & 31) == 0) pbits[(size_t)b * (hw_max / 32 + 1) + (px >> 5)] = word;
+}
+
+rl_status launch_mode_bits(const Frame *frames, const uint4 *prec, int hw_max, int n_trees, uint32_t *pbits, int n,
+                           cudaStream_t s) {
+    k_mode_bits<<<dim3((hw_max + 255) / 256, n), 256, 0, s>>>(frames, prec, hw_max, n_trees, pbits);
+    RL_LAUNCH_CK();
+    return RL_OK;
 }
 
 rl_status launch_colour_mask(const Frame *frames, const uint16_t *mcount, const uint4 *prec, int hw_max,
@@ -434,47 +525,67 @@ __global__ void k_sample_batch(const Frame *__restrict__ frames, const uint16_t 
     xc_out[o] = x;
 }
 
-template <int REDRAW>
+template <int REDRAW, int PATH>
 static void launch_hypgen_shape(const HypArgs &a, int warps, int n, size_t sm, cudaStream_t s) {
-    const int N = a.p.n_hyp;
+    const int N = a.p.n_hyp * a.team;  // warps wanted per frame
     switch (warps) {
-    case 2: k_hypgen<2, REDRAW><<<dim3((N + 1) / 2, n), 64, sm, s>>>(a); break;
-    case 8: k_hypgen<8, REDRAW><<<dim3((N + 7) / 8, n), 256, sm, s>>>(a); break;
-    case 16: k_hypgen<16, REDRAW><<<dim3((N + 15) / 16, n), 512, sm, s>>>(a); break;
-    default: k_hypgen<4, REDRAW><<<dim3((N + 3) / 4, n), 128, sm, s>>>(a); break;
+    case 2: k_hypgen<2, REDRAW, PATH><<<dim3((N + 1) / 2, n), 64, sm, s>>>(a); break;
+    case 8: k_hypgen<8, REDRAW, PATH><<<dim3((N + 7) / 8, n), 256, sm, s>>>(a); break;
+    case 16: k_hypgen<16, REDRAW, PATH><<<dim3((N + 15) / 16, n), 512, sm, s>>>(a); break;
+    default: k_hypgen<4, REDRAW, PATH><<<dim3((N + 3) / 4, n), 128, sm, s>>>(a); break;
     }
+}
+
+template <int REDRAW>
+static void launch_hypgen_path(const HypArgs &a, int warps, int n, size_t bits_smem, cudaStream_t s) {
+    const size_t mode_smem = (size_t)warps * HG_RING * sizeof(uint2);
+    if (!a.pbits && !a.pcm)
+        launch_hypgen_shape<REDRAW, HYP_GENERAL>(a, warps, n, mode_smem, s);
+    else if (!a.pbits)
+        launch_hypgen_shape<REDRAW, HYP_MASKS_ONLY>(a, warps, n, mode_smem, s);
+    else if (a.pcm)
+        launch_hypgen_shape<REDRAW, HYP_MASKS>(a, warps, n, bits_smem, s);
+    else
+        launch_hypgen_shape<REDRAW, HYP_RECORDS>(a, warps, n, bits_smem, s);
 }
 
 rl_status launch_hypgen(const Frame *frames, const uint16_t *leaves, const uint16_t *mcount,
                         const uint4 *prec, const uint2 *pcm, const uint32_t *pbits, int hw_max, ModeView mv,
                         const RParams &p, double *hyp_pose, int32_t *hyp_iter, unsigned long long *work, int n,
-                        cudaStream_t s, int warps) {
+                        cudaStream_t s, int warps, int n_active, int sm_count) {
     // the bitmap path needs the frame's bitmap in shared memory
     const size_t bits_smem = (size_t)(hw_max / 32 + 1) * 4;
-    const bool bits = pcm && pbits && bits_smem <= kHypBitsSmemMax;
-    HypArgs a{frames, leaves, mcount, prec, pcm, hw_max, mv, p, hyp_pose, hyp_iter, work, bits ? pbits : nullptr};
-    const size_t sm = bits ? bits_smem : 0;
+    const bool bits = prec && pbits && bits_smem <= kHypBitsSmemMax;
+    int team = 1;
+    while (2 * team <= warps && (int64_t)p.n_hyp * n_active * 2 * team <= (int64_t)sm_count * 32) team *= 2;
+    HypArgs a{frames, leaves, mcount, prec, pcm, hw_max, mv, p, hyp_pose, hyp_iter, work, bits ? pbits : nullptr, team};
     if (p.redraw)
-        launch_hypgen_shape<1>(a, warps, n, sm, s);
+        launch_hypgen_path<1>(a, warps, n, bits_smem, s);
     else
-        launch_hypgen_shape<0>(a, warps, n, sm, s);
+        launch_hypgen_path<0>(a, warps, n, bits_smem, s);
     RL_LAUNCH_CK();
     return RL_OK;
 }
 
-template <int REDRAW>
-static rl_status prepare_hypgen_reading() {
+template <int REDRAW, int PATH>
+static rl_status prepare_hypgen_path() {
     const int sm = (int)kHypBitsSmemMax;
-    RL_CK(cudaFuncSetAttribute(k_hypgen<2, REDRAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-    RL_CK(cudaFuncSetAttribute(k_hypgen<4, REDRAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-    RL_CK(cudaFuncSetAttribute(k_hypgen<8, REDRAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-    RL_CK(cudaFuncSetAttribute(k_hypgen<16, REDRAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    RL_CK(cudaFuncSetAttribute(k_hypgen<2, REDRAW, PATH>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    RL_CK(cudaFuncSetAttribute(k_hypgen<4, REDRAW, PATH>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    RL_CK(cudaFuncSetAttribute(k_hypgen<8, REDRAW, PATH>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    RL_CK(cudaFuncSetAttribute(k_hypgen<16, REDRAW, PATH>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
     return RL_OK;
 }
 
 rl_status prepare_hypgen() {
-    RL_TRY(prepare_hypgen_reading<0>());
-    return prepare_hypgen_reading<1>();
+    RL_TRY((prepare_hypgen_path<0, HYP_GENERAL>()));
+    RL_TRY((prepare_hypgen_path<0, HYP_MASKS_ONLY>()));
+    RL_TRY((prepare_hypgen_path<0, HYP_MASKS>()));
+    RL_TRY((prepare_hypgen_path<0, HYP_RECORDS>()));
+    RL_TRY((prepare_hypgen_path<1, HYP_GENERAL>()));
+    RL_TRY((prepare_hypgen_path<1, HYP_MASKS_ONLY>()));
+    RL_TRY((prepare_hypgen_path<1, HYP_MASKS>()));
+    return prepare_hypgen_path<1, HYP_RECORDS>();
 }
 
 rl_status launch_compact(const int32_t *hyp_iter, int N, int32_t *hyp_list, int32_t *n_hyp, int n,

@@ -185,7 +185,7 @@ struct QueryState {
     uint16_t *mcount;        // [B][HWmax] |M(u)| per pixel
     uint4 *prec;             // [B][HWmax] per-pixel leaves + counts (<= 5 trees), else null
     uint2 *pcm;              // [B][HWmax] colour-check bits of M(u) | |M(u)| << 56 (|M(u)| <= 56), else null
-    uint32_t *pbits;         // [B][HWmax / 32 + 1] bit p: M(u) of pixel p is non-empty (with pcm)
+    uint32_t *pbits;         // [B][HWmax / 32 + 1] bit p: M(u) of pixel p is non-empty (with prec)
     double *hyp_pose;        // [B][N][12]
     int32_t *hyp_iter;       // [B][N]
     int32_t *hyp_list;       // [B][N] slots of successful hypotheses
@@ -392,8 +392,10 @@ rl_status update_modes(rl_forest *f, int64_t begin, int64_t count, cudaStream_t 
 rl_status reset_leaves(rl_forest *f, cudaStream_t s);
 ModeView mode_view(const rl_forest *f);
 // The launch sequence of n frames whose query state is q (r->q, or a slice
-// of it for a sub-batch: query_slice).
-rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int level, cudaStream_t s);
+// of it for a sub-batch: query_slice); n_active: frames at work on the GPU
+// at once, the call's other sub-batches included (it shapes launches, never
+// results).
+rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, int level, cudaStream_t s);
 // q for the frames b0, b0 + 1, ... of r's batch.
 QueryState query_slice(const rl_reloc *r, int b0);
 // Batch of n frames whose descriptors (device pointers, per-frame sizes and

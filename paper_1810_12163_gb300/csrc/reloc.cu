@@ -163,7 +163,7 @@ static void prof_resolve(rl_reloc *r) {
 
 #define PROF(kid) ProfScope prof_scope_##kid##__LINE__(r, kid, s)
 
-rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int level, cudaStream_t s) {
+rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, int level, cudaStream_t s) {
     rl_forest *f = r->forest;
     RParams p = r->rp;
     p.level = level;
@@ -180,7 +180,8 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int level, cud
     // count map is written
     { PROF(K_LEAVES); RL_TRY(launch_leaves(f, q.frames, n, p.n_trees, hw_max, q.prec ? nullptr : q.leaves, r->max_w, r->max_h, s, p.k_top, q.prec ? nullptr : q.mcount, q.prec, r->tune.leaves_threads, r->nodes_s, r->host_frames[0].fx)); }
     if (q.pcm) { PROF(K_CMASK); RL_TRY(launch_colour_mask(q.frames, q.mcount, q.prec, hw_max, mv, p, q.pcm, q.pbits, n, hw_max, s, r->tune.mask_threads)); }
-    { PROF(K_HYPGEN); RL_TRY(launch_hypgen(q.frames, q.leaves, q.mcount, q.prec, q.pcm, q.pbits, hw_max, mv, p, q.hyp_pose, q.hyp_iter, work, n, s, r->tune.hypgen_warps)); }
+    else if (q.pbits) { PROF(K_CMASK); RL_TRY(launch_mode_bits(q.frames, q.prec, hw_max, p.n_trees, q.pbits, n, s)); }
+    { PROF(K_HYPGEN); RL_TRY(launch_hypgen(q.frames, q.leaves, q.mcount, q.prec, q.pcm, q.pbits, hw_max, mv, p, q.hyp_pose, q.hyp_iter, work, n, s, r->tune.hypgen_warps, n_active, r->forest->ctx->sm_count)); }
     { PROF(K_HYPPOSE); RL_TRY(launch_hyppose(q.frames, q.leaves, q.mcount, q.prec, hw_max, mv, p, q.hyp_pose, q.hyp_iter, n, s)); }
     { PROF(K_COMPACT); RL_TRY(launch_compact(q.hyp_iter, N, q.hyp_list, q.n_hyp, n, s)); }
     { PROF(K_SAMPLE); RL_TRY(launch_sample_batch(q.frames, q.mcount, q.prec, hw_max, p, 0, q.pix, q.xc, n, s));
@@ -370,7 +371,7 @@ static rl_status run_relocalise_parts(rl_reloc *r, int n, int level, cudaStream_
     // replayed graph, walk the unscaled nodes)
     RL_TRY(launch_scale_nodes(r->forest, r->rp.n_trees, r->nodes_s, r->host_frames[0].fx, s));
     const int parts = r->prof.on ? 1 : std::max(1, std::min(r->tune.streams, n / kMinPart));
-    if (parts <= 1) return run_relocalise(r, r->q, n, level, s);
+    if (parts <= 1) return run_relocalise(r, r->q, n, n, level, s);
     for (int i = 0; i < parts - 1; ++i) {
         if (!r->side[i]) RL_CK(cudaStreamCreateWithFlags(&r->side[i], cudaStreamNonBlocking));
         if (!r->join_ev[i]) RL_CK(cudaEventCreateWithFlags(&r->join_ev[i], cudaEventDisableTiming));
@@ -382,7 +383,7 @@ static rl_status run_relocalise_parts(rl_reloc *r, int n, int level, cudaStream_
         const int nb = n / parts + (i < n % parts ? 1 : 0);
         cudaStream_t si = i == 0 ? s : r->side[i - 1];
         if (i > 0) RL_CK(cudaStreamWaitEvent(si, r->fork_ev, 0));
-        RL_TRY(run_relocalise(r, query_slice(r, b0), nb, level, si));
+        RL_TRY(run_relocalise(r, query_slice(r, b0), nb, n, level, si));
         if (i > 0) RL_CK(cudaEventRecord(r->join_ev[i - 1], si));
         b0 += nb;
     }
@@ -604,7 +605,7 @@ extern "C" rl_status rl_reloc_create(rl_forest *f, rl_scene *scene, const rl_ran
     A(mcount, B * hw);
     if (p->n_trees_used <= kRecTrees) A(prec, B * hw);
     if (p->n_trees_used <= kRecTrees && maxm <= kMaskModes) A(pcm, B * hw);
-    if (q.pcm) A(pbits, B * (hw / 32 + 1));
+    if (q.prec) A(pbits, B * (hw / 32 + 1));
     A(hyp_pose, B * N * 12);
     A(hyp_iter, B * N);
     A(hyp_list, B * N);
@@ -832,8 +833,12 @@ static CascadeOut cascade_out_slice(const CascadeOut &o, int b0) {
     return s;
 }
 
-// All levels for the nb frames b0, b0 + 1, ... of the call.
-static rl_status cascade_enqueue_part(rl_cascade *c, int b0, int nb, cudaStream_t s) {
+// A later level shapes its launches for a quarter of the call's frames: most
+// were accepted before and are empty frames there.
+constexpr int kLaterLevelShare = 4;
+
+// All levels for the nb frames b0, b0 + 1, ... of the call of n frames.
+static rl_status cascade_enqueue_part(rl_cascade *c, int b0, int nb, int n, cudaStream_t s) {
     const int L = (int)c->levels.size();
     const CascadeOut out = cascade_out_slice(c->out, b0);
     RL_CK(cudaMemsetAsync(out.done, 0, sizeof(int32_t) * nb, s));
@@ -848,7 +853,7 @@ static rl_status cascade_enqueue_part(rl_cascade *c, int b0, int nb, cudaStream_
                                                  r->stage_rgb + (size_t)b0 * hw * 3, hw);
             RL_LAUNCH_CK();
         }
-        RL_TRY(run_relocalise(r, q, nb, l, s));
+        RL_TRY(run_relocalise(r, q, nb, l == 0 ? n : std::max(1, n / kLaterLevelShare), l, s));
         LaterFrames later{};
         for (int k = l + 1; k < L && later.n < 8; ++k) later.f[later.n++] = c->levels[k]->q.frames + b0;
         const float tau = l < L - 1 ? (float)c->thresholds[l] : INFINITY;
@@ -866,7 +871,7 @@ static rl_status cascade_enqueue(rl_cascade *c, int n, cudaStream_t s) {
     for (rl_reloc *r : c->levels)  // each level's nodes scaled for its focal length
         RL_TRY(launch_scale_nodes(r->forest, r->rp.n_trees, r->nodes_s, r->host_frames[0].fx, s));
     const int parts = prof ? 1 : std::max(1, std::min(c->levels[0]->tune.streams, n / kMinPart));
-    if (parts <= 1) return cascade_enqueue_part(c, 0, n, s);
+    if (parts <= 1) return cascade_enqueue_part(c, 0, n, n, s);
     for (int i = 0; i < parts - 1; ++i) {
         if (!c->side[i]) RL_CK(cudaStreamCreateWithFlags(&c->side[i], cudaStreamNonBlocking));
         if (!c->join_ev[i]) RL_CK(cudaEventCreateWithFlags(&c->join_ev[i], cudaEventDisableTiming));
@@ -878,7 +883,7 @@ static rl_status cascade_enqueue(rl_cascade *c, int n, cudaStream_t s) {
         const int nb = n / parts + (i < n % parts ? 1 : 0);
         cudaStream_t si = i == 0 ? s : c->side[i - 1];
         if (i > 0) RL_CK(cudaStreamWaitEvent(si, c->fork_ev, 0));
-        RL_TRY(cascade_enqueue_part(c, b0, nb, si));
+        RL_TRY(cascade_enqueue_part(c, b0, nb, n, si));
         if (i > 0) RL_CK(cudaEventRecord(c->join_ev[i - 1], si));
         b0 += nb;
     }
