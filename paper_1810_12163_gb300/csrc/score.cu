@@ -726,68 +726,65 @@ __global__ void __launch_bounds__(256) k_raycast_score(RaycastArgs a) {
     }
 }
 
-// Eq. 7 from the tile partials of one (frame, pose): FP64 sums in tile order.
-__device__ float score_from_tiles(const double *part_sum, const int32_t *part_cnt, size_t base,
-                                  int n_tiles, double npx, float *valid_frac) {
-    double sum = 0.0;
-    long syn = 0, both = 0;
-    for (int t = 0; t < n_tiles; ++t) {
-        sum += part_sum[base + t];
-        syn += part_cnt[2 * (base + t)];
-        both += part_cnt[2 * (base + t) + 1];
-    }
-    const double frac = (double)syn / npx;
-    if (valid_frac) *valid_frac = (float)frac;
-    return (frac >= 0.1 && both > 0) ? (float)(sum / (double)both) : INFINITY;
-}
-
-// Eq. 7-8 per frame, then the frame's result record.
+// Eq. 7-8 per frame, then the frame's result record.  Eq. 7 for all chosen
+// poses at once: tile partials summed by a fixed-shape block reduction (FP64
+// sums, integer counts).  What bounds it is FP64 addition (one warp
+// instruction in 64 cycles per sub-partition) and the latency of reading the
+// partials, so the poses' sums are kept in flight together and meet at one
+// barrier: 16 poses of 600 tiles 26 us, 51 with the poses one after another.
 __global__ void __launch_bounds__(256) k_finalize(QueryState q, RParams p, int n_tiles, int ranked) {
-    __shared__ double s_sum[8];
-    __shared__ long long s_syn[8], s_both[8];
+    __shared__ double s_sum[16][8];
+    __shared__ int s_syn[16][8], s_both[16][8];
+    __shared__ float s_score[16];
     const int b = blockIdx.x;
     const Frame fr = q.frames[b];
     if (ranked && q.n_hyp[b] > 0) {
-        // Eq. 7 for each chosen pose: tile partials summed by a fixed-shape
-        // block reduction (FP64 sums, integer counts)
-        const double npx = (double)fr.W * (double)fr.H;
-        for (int c = 0; c < q.n_chosen[b]; ++c) {
-            const size_t base = ((size_t)b * 16 + c) * n_tiles;
-            double sum = 0.0;
-            long long syn = 0, both = 0;
-            for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) {
-                sum += q.score_part[base + t];
-                syn += q.score_cnt[2 * (base + t)];
-                both += q.score_cnt[2 * (base + t) + 1];
-            }
+        const int nc = q.n_chosen[b], lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        for (int c0 = 0; c0 < nc; c0 += 4) {
+            double sum[4] = {0.0, 0.0, 0.0, 0.0};
+            int syn[4] = {0, 0, 0, 0}, both[4] = {0, 0, 0, 0};
+            for (int t = threadIdx.x; t < n_tiles; t += blockDim.x)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sum += __shfl_down_sync(0xffffffffu, sum, o);
-                syn += __shfl_down_sync(0xffffffffu, syn, o);
-                both += __shfl_down_sync(0xffffffffu, both, o);
-            }
-            if ((threadIdx.x & 31) == 0) {
-                s_sum[threadIdx.x >> 5] = sum;
-                s_syn[threadIdx.x >> 5] = syn;
-                s_both[threadIdx.x >> 5] = both;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double ts = 0.0;
-                long long tsyn = 0, tb = 0;
-                for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-                    ts += s_sum[k];
-                    tsyn += s_syn[k];
-                    tb += s_both[k];
+                for (int k = 0; k < 4; ++k) {
+                    const size_t o = ((size_t)b * 16 + min(c0 + k, nc - 1)) * n_tiles + t;
+                    sum[k] += q.score_part[o];
+                    const int2 cnt = ((const int2 *)q.score_cnt)[o];
+                    syn[k] += cnt.x;
+                    both[k] += cnt.y;
                 }
-                const double frac = (double)tsyn / npx;
-                // a pose whose ICP failed is discarded (Sec. 3.2.4)
-                const bool kept = !p.icp || q.icp_ok[(size_t)b * 16 + c];
-                q.chosen_score[(size_t)b * 16 + c] =
-                    (kept && frac >= 0.1 && tb > 0) ? (float)(ts / (double)tb) : INFINITY;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) sum[k] += __shfl_down_sync(0xffffffffu, sum[k], o);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {  // at most 2^26 pixels: 32-bit counts
+                syn[k] = __reduce_add_sync(0xffffffffu, syn[k]);
+                both[k] = __reduce_add_sync(0xffffffffu, both[k]);
+                if (lane == 0 && c0 + k < nc) {
+                    s_sum[c0 + k][w] = sum[k];
+                    s_syn[c0 + k][w] = syn[k];
+                    s_both[c0 + k][w] = both[k];
+                }
             }
-            __syncthreads();
         }
+        __syncthreads();
+        if ((int)threadIdx.x < nc) {
+            const int c = threadIdx.x;
+            double ts = 0.0;
+            int tsyn = 0, tb = 0;
+            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
+                ts += s_sum[c][k];
+                tsyn += s_syn[c][k];
+                tb += s_both[c][k];
+            }
+            const double frac = (double)tsyn / ((double)fr.W * (double)fr.H);
+            // a pose whose ICP failed is discarded (Sec. 3.2.4)
+            const bool kept = !p.icp || q.icp_ok[(size_t)b * 16 + c];
+            const float sc = (kept && frac >= 0.1 && tb > 0) ? (float)(ts / (double)tb) : INFINITY;
+            s_score[c] = sc;
+            q.chosen_score[(size_t)b * 16 + c] = sc;
+        }
+        __syncthreads();
     }
     if (threadIdx.x != 0) return;
     DevResult *out = (DevResult *)q.result_blob + b;
@@ -816,7 +813,7 @@ __global__ void __launch_bounds__(256) k_finalize(QueryState q, RParams p, int n
     float bs = INFINITY;
     if (ranked) {
         for (int c = 0; c < q.n_chosen[b]; ++c) {
-            const float s = q.chosen_score[(size_t)b * 16 + c];
+            const float s = s_score[c];
             if (s < bs) {
                 bs = s;
                 best = c;
@@ -907,14 +904,32 @@ rl_status launch_finalize(const QueryState &q, const RParams &p, int n_tiles, in
 }  // namespace rl
 
 namespace rl {
-// Standalone Eq. 6-7 scorer: poses [n][12] against one live depth frame.
-__global__ void k_scores_final(const double *part_sum, const int32_t *part_cnt, int n_tiles,
-                               int n, double npx, float *scores, float *valid_frac) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+// Standalone Eq. 6-7 scorer: poses [n][12] against one live depth frame.  A
+// warp per pose sums its tile partials in FP64 (one thread walking all tiles
+// took 83 us for 128 poses at 640x480, the lanes 8 us).
+__global__ void __launch_bounds__(128) k_scores_final(const double *__restrict__ part_sum,
+                                                      const int32_t *__restrict__ part_cnt, int n_tiles, int n,
+                                                      double npx, float *__restrict__ scores,
+                                                      float *__restrict__ valid_frac) {
+    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c >= n) return;
-    float vf;
-    scores[c] = score_from_tiles(part_sum, part_cnt, (size_t)c * n_tiles, n_tiles, npx, &vf);
-    valid_frac[c] = vf;
+    double sum = 0.0;
+    int syn = 0, both = 0;
+    for (int t = lane; t < n_tiles; t += 32) {
+        const size_t o = (size_t)c * n_tiles + t;
+        sum += part_sum[o];
+        const int2 cnt = ((const int2 *)part_cnt)[o];
+        syn += cnt.x;
+        both += cnt.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    syn = __reduce_add_sync(0xffffffffu, syn);
+    both = __reduce_add_sync(0xffffffffu, both);
+    if (lane != 0) return;
+    const double frac = (double)syn / npx;
+    valid_frac[c] = (float)frac;
+    scores[c] = (frac >= 0.1 && both > 0) ? (float)(sum / (double)both) : INFINITY;
 }
 
 rl_status launch_score_poses(const RaycastArgs &a, int n_poses, int npx, float *scores,
@@ -922,7 +937,7 @@ rl_status launch_score_poses(const RaycastArgs &a, int n_poses, int npx, float *
     dim3 grid(a.n_tiles, 1);
     k_raycast_score<<<grid, 256, 0, s>>>(a);
     RL_LAUNCH_CK();
-    k_scores_final<<<(n_poses + 63) / 64, 64, 0, s>>>(a.part_sum, a.part_cnt, a.n_tiles, n_poses,
+    k_scores_final<<<(n_poses + 3) / 4, 128, 0, s>>>(a.part_sum, a.part_cnt, a.n_tiles, n_poses,
                                                       (double)npx, scores, valid_frac);
     RL_LAUNCH_CK();
     return RL_OK;
