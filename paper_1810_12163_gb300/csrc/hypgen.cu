@@ -493,36 +493,64 @@ __global__ void __launch_bounds__(1024) k_compact(const int32_t *__restrict__ hy
     if (tid == 0) n_hyp[b] = running;
 }
 
-// Pixel batch `batch`: eta draws, each redrawn up to batch_attempts times
-// until its pixel has a non-empty M(u) (which implies depth); skipped (-1)
-// otherwise.
-__global__ void k_sample_batch(const Frame *__restrict__ frames, const uint16_t *__restrict__ mcount,
-                               const uint4 *__restrict__ prec, int hw_max, RParams p, int batch,
-                               int32_t *__restrict__ pix_out, float4 *__restrict__ xc_out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// Pixel batches of a call and their mode table, all rounds at once (neither
+// depends on the hypotheses).  A warp per draw: draw j of batch t is redrawn
+// up to batch_attempts times until its pixel has a non-empty M(u) (which
+// implies depth), skipped (-1) otherwise; then M(u) of the pixel, decoded to
+// FP32 (position, Cholesky factor), goes into one row of mpad records, a
+// lane per mode.  What bounds it is the two dependent gathers of a row; one
+// launch for the seven batches of the paper-sized relocaliser, 12 us for six
+// 333x250 frames, where sampling and decoding batch by batch took 14
+// launches and 80 us of the call.
+__global__ void __launch_bounds__(256) k_sample_table(QueryState q, int hw_max, ModeView mv, RParams p, int n_draws) {
+    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int b = blockIdx.y;
-    if (j >= p.eta) return;
-    const Frame fr = frames[b];
-    const uint16_t *mc = mcount + (size_t)b * hw_max;
-    const uint4 *pr = prec ? prec + (size_t)b * hw_max : nullptr;
+    if (i >= n_draws) return;
+    const int batch = i / p.eta, j = i % p.eta;
+    const Frame fr = q.frames[b];
+    const uint16_t *mc = q.mcount + (size_t)b * hw_max;
+    const uint4 *pr = q.prec ? q.prec + (size_t)b * hw_max : nullptr;
     const uint32_t WH = (uint32_t)(fr.W * fr.H);
-    int pix = -1;
+    int pix = -1, cnt = 0;
     for (int at = 0; at < p.batch_attempts && WH > 0; ++at) {
         const uint4 r = philox(make_uint4(batch, (TAG_BATCH << 16) | (uint32_t)p.level, j, at),
                                fr.key0, fr.key1);
-        const int q = (int)draw_below(r.x, WH);
-        if (pixel_modes(mc, pr, q, p.n_trees) == 0) continue;
-        pix = q;
+        const int u = (int)draw_below(r.x, WH);
+        cnt = pixel_modes(mc, pr, u, p.n_trees);
+        if (cnt == 0) continue;
+        pix = u;
         break;
     }
-    const size_t o = (size_t)b * p.max_pix + (size_t)batch * p.eta + j;
-    pix_out[o] = pix;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (pix >= 0) {
-        const float3 c = backproject(fr, pix);
-        x = make_float4(c.x, c.y, c.z, 0.f);
+    const size_t row = (size_t)b * p.max_pix + i;
+    if (lane == 0) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (pix >= 0) {
+            const float3 c = backproject(fr, pix);
+            x = make_float4(c.x, c.y, c.z, 0.f);
+        }
+        q.pix[row] = pix;
+        q.xc[row] = x;
+        q.tab_cnt[row] = (int16_t)cnt;
     }
-    xc_out[o] = x;
+    for (int m = lane; m < cnt; m += 32) {
+        uint32_t L;
+        int rank;
+        if (pr)
+            mode_at_rec(pr[pix], p.n_trees, mv.leaves_per_tree, m, &L, &rank);
+        else
+            mode_at(mv, q.leaves + (size_t)b * p.n_trees * hw_max, hw_max, pix, p.n_trees, p.k_top, m, &L, &rank);
+        const float3 mp = mode_pos(mv, L, rank);
+        const size_t me = (size_t)L * mv.m_max + rank;
+        const size_t o = row * p.mpad + m;
+        if (p.use_cov) {
+            const float4 u0 = mv.mU[2 * me], u1 = mv.mU[2 * me + 1];
+            q.tab0[o] = make_float4(mp.x, mp.y, mp.z, u0.x);
+            q.tab1[o] = make_float4(u0.y, u0.z, u0.w, u1.x);
+            q.tab2[o] = u1.y;
+        } else {
+            q.tab0[o] = make_float4(mp.x, mp.y, mp.z, 1.f);
+        }
+    }
 }
 
 template <int REDRAW, int PATH>
@@ -595,11 +623,9 @@ rl_status launch_compact(const int32_t *hyp_iter, int N, int32_t *hyp_list, int3
     return RL_OK;
 }
 
-rl_status launch_sample_batch(const Frame *frames, const uint16_t *mcount, const uint4 *prec, int hw_max,
-                              const RParams &p, int batch, int32_t *pix, float4 *xc, int n,
-                              cudaStream_t s) {
-    dim3 grid((p.eta + 127) / 128, n);
-    k_sample_batch<<<grid, 128, 0, s>>>(frames, mcount, prec, hw_max, p, batch, pix, xc);
+rl_status launch_sample_table(const QueryState &q, int hw_max, ModeView mv, const RParams &p, int n, cudaStream_t s) {
+    const int draws = p.eta * (p.max_rounds + 1);
+    k_sample_table<<<dim3((draws + 7) / 8, n), 256, 0, s>>>(q, hw_max, mv, p, draws);
     RL_LAUNCH_CK();
     return RL_OK;
 }

@@ -30,9 +30,8 @@ struct EnergyArgs {
     const int16_t *q_tab_cnt;
 };
 
-// Mode table of pixel batch `batch` (decoded M(u) of each drawn pixel).
-rl_status launch_build_table(const QueryState &q, int hw_max, ModeView mv, const RParams &p, int batch,
-                             int n, cudaStream_t s);
+// Pixel batches of all rounds and their mode table (decoded M(u) of each drawn pixel).
+rl_status launch_sample_table(const QueryState &q, int hw_max, ModeView mv, const RParams &p, int n, cudaStream_t s);
 
 struct SelectArgs {
     int phase, round;
@@ -142,9 +141,6 @@ rl_status launch_hyppose(const Frame *frames, const uint16_t *leaves, const uint
                          double *hyp_pose, int32_t *hyp_iter, int n, cudaStream_t s);
 rl_status launch_compact(const int32_t *hyp_iter, int N, int32_t *hyp_list, int32_t *n_hyp, int n,
                          cudaStream_t s);
-rl_status launch_sample_batch(const Frame *frames, const uint16_t *mcount, const uint4 *prec, int hw_max,
-                              const RParams &p, int batch, int32_t *pix, float4 *xc, int n,
-                              cudaStream_t s);
 rl_status launch_subsample(const Frame *src, Frame *dst_desc, float *dst_depth, uint8_t *dst_rgb,
                            int s_factor, int n, int max_w, int max_h, cudaStream_t s);
 

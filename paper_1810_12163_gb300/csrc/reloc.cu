@@ -184,8 +184,7 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
     { PROF(K_HYPGEN); RL_TRY(launch_hypgen(q.frames, q.leaves, q.mcount, q.prec, q.pcm, q.pbits, hw_max, mv, p, q.hyp_pose, q.hyp_iter, work, n, s, r->tune.hypgen_warps, n_active, r->forest->ctx->sm_count)); }
     { PROF(K_HYPPOSE); RL_TRY(launch_hyppose(q.frames, q.leaves, q.mcount, q.prec, hw_max, mv, p, q.hyp_pose, q.hyp_iter, n, s)); }
     { PROF(K_COMPACT); RL_TRY(launch_compact(q.hyp_iter, N, q.hyp_list, q.n_hyp, n, s)); }
-    { PROF(K_SAMPLE); RL_TRY(launch_sample_batch(q.frames, q.mcount, q.prec, hw_max, p, 0, q.pix, q.xc, n, s));
-      RL_TRY(launch_build_table(q, hw_max, mv, p, 0, n, s)); }
+    { PROF(K_SAMPLE); RL_TRY(launch_sample_table(q, hw_max, mv, p, n, s)); }
 
     const int maxm = p.maxm;
     int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(32, 40960 / (p.mpad * 36)));
@@ -235,8 +234,6 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
     // preemptive rounds
     for (int round = 0; round < p.max_rounds; ++round) {
         const int n_pix = p.eta * (round + 2);
-        { PROF(K_SAMPLE); RL_TRY(launch_sample_batch(q.frames, q.mcount, q.prec, hw_max, p, round + 1, q.pix, q.xc, n, s));
-          RL_TRY(launch_build_table(q, hw_max, mv, p, round + 1, n, s)); }
         const bool lm = p.pose_update && p.lm_max_iter > 0;
         if (lm) {
             LmArgs la{q, q.leaves, hw_max, mv, p, n_pix, work, maxm, maxm | 1, r->lm_wait_limit};

@@ -489,47 +489,6 @@ __global__ void __launch_bounds__(LM3_THREADS, 2) k_lm_spread(LmArgs a) {
     }
 }
 
-// Mode table of batch `batch`: for each drawn pixel, M(u) decoded to FP32
-// (position, Cholesky factor) into one row of mpad records.
-__global__ void k_build_table(QueryState q, int hw_max, ModeView mv, RParams p, int batch) {
-    const int b = blockIdx.y;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= p.eta * p.mpad) return;
-    const int i = batch * p.eta + e / p.mpad, m = e % p.mpad;
-    const size_t row = (size_t)b * p.max_pix + i;
-    const int pix = q.pix[row];
-    const int cnt = pix < 0 ? 0
-                            : pixel_modes(q.mcount + (size_t)b * hw_max,
-                                          q.prec ? q.prec + (size_t)b * hw_max : nullptr, pix, p.n_trees);
-    if (m == 0) q.tab_cnt[row] = (int16_t)cnt;
-    if (m >= cnt) return;
-    uint32_t L;
-    int rank;
-    if (q.prec)
-        mode_at_rec(q.prec[(size_t)b * hw_max + pix], p.n_trees, mv.leaves_per_tree, m, &L, &rank);
-    else
-        mode_at(mv, q.leaves + (size_t)b * p.n_trees * hw_max, hw_max, pix, p.n_trees, p.k_top, m, &L, &rank);
-    const float3 mp = mode_pos(mv, L, rank);
-    const size_t me = (size_t)L * mv.m_max + rank;
-    const size_t o = row * p.mpad + m;
-    if (p.use_cov) {
-        const float4 u0 = mv.mU[2 * me], u1 = mv.mU[2 * me + 1];
-        q.tab0[o] = make_float4(mp.x, mp.y, mp.z, u0.x);
-        q.tab1[o] = make_float4(u0.y, u0.z, u0.w, u1.x);
-        q.tab2[o] = u1.y;
-    } else {
-        q.tab0[o] = make_float4(mp.x, mp.y, mp.z, 1.f);
-    }
-}
-
-rl_status launch_build_table(const QueryState &q, int hw_max, ModeView mv, const RParams &p, int batch,
-                             int n, cudaStream_t s) {
-    dim3 grid((p.eta * p.mpad + 255) / 256, n);
-    k_build_table<<<grid, 256, 0, s>>>(q, hw_max, mv, p, batch);
-    RL_LAUNCH_CK();
-    return RL_OK;
-}
-
 // z-depth of the first box face hit by the ray of pixel (u, v) (exit point
 // from inside the box, entry point from outside), in FP64.
 __device__ bool ray_depth64(const double *P, int u, int v, float fx, float fy, float cx, float cy,
