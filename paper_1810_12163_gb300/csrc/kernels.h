@@ -57,6 +57,8 @@ struct LmArgs {
     int maxm;                  // |M(u)| bound: trees x min(k_top, m_max)
     int maxm_pad;              // maxm rounded up to an odd count (shared-memory rows)
     uint32_t wait_limit;       // probes of a wait for a staged tile before it gives up
+    int n_active;              // frames at work on the GPU at once (shapes the launch, never the result)
+    int sm_count;
 };
 
 rl_status prepare_kernels();

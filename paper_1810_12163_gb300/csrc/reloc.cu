@@ -236,7 +236,7 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
         const int n_pix = p.eta * (round + 2);
         const bool lm = p.pose_update && p.lm_max_iter > 0;
         if (lm) {
-            LmArgs la{q, q.leaves, hw_max, mv, p, n_pix, work, maxm, maxm | 1, r->lm_wait_limit};
+            LmArgs la{q, q.leaves, hw_max, mv, p, n_pix, work, maxm, maxm | 1, r->lm_wait_limit, n_active, f->ctx->sm_count};
             PROF(K_LM);
             RL_TRY(launch_lm(la, n, s));
         }

@@ -7,6 +7,8 @@
 // shape, so results do not depend on how many frames share a launch.
 #include <math.h>
 
+#include <cooperative_groups.h>
+
 #include "internal.h"
 #include "relocgb_dev.cuh"
 #include "kernels.h"
@@ -260,37 +262,57 @@ __global__ void __launch_bounds__(1024) k_select(SelectArgs a) {
 // ---------------------------------------------------------------------------
 
 // LM, hypotheses spread over threads.  A round's n hypotheses of a frame are
-// split over up to LM3_BPQ blocks; inside a block, thread t works for
-// hypothesis h = t % HB on the pixels g, g + G, ... (g = t / HB, G = 256/HB,
-// HB = the next power of two >= the block's hypothesis count).  As rounds
-// halve n, each hypothesis gets more threads.  Partial normal equations are
-// tree-reduced over the G groups in shared memory (fixed shape), the 6x6
-// system of each hypothesis is solved in FP64 by one thread, and the trial
-// cost with the same correspondences is reduced the same way.
+// split over up to LM3_BPQ parts; inside a part, hypothesis h has G = 256 / HB
+// pixel groups (HB = the next power of two >= the part's hypothesis count),
+// group g taking the pixels g, g + G, ...  As rounds halve n, each hypothesis
+// gets more groups.  Partial normal equations are tree-reduced over the
+// groups (fixed shape), the 6x6 system of each hypothesis is solved in FP64
+// by one thread, and the trial cost with the same correspondences is reduced
+// the same way.
+//
+// A part is one cluster of CT blocks: block c takes the groups c, c + CT, ...,
+// and CT adjacent lanes share a pair's mode scan (every CT-th mode; ties to
+// the lower index), so the sums and their order do not depend on CT.  The
+// tree's levels of at least CT groups apart lie within a block, the last ones
+// go through distributed shared memory, every block holding the same totals
+// and taking the same decisions.  With one block per part a call of few
+// frames leaves most of the GPU idle (four frames: 16 blocks) on scans of up
+// to 250 modes; CT grows to 8 while the call's blocks still fit two per SM.
+// A large batch keeps CT = 1: the lanes that share a scan idle through the
+// accumulation, about a quarter more instructions.  Measured on four 640x480
+// frames, 64 hypotheses, up to 250 modes per pixel, six rounds: 4.5 ms with
+// CT = 8, 17.9 with one block per part.
 constexpr int LM3_THREADS = 256;
 constexpr int LM3_BPQ = 4;
+constexpr int LM3_HMAX = 64 / LM3_BPQ;  // hypotheses of a part (n_cull <= 64)
+constexpr int LM3_NV = 29;              // 21 J^T J, 6 J^T r, cost, inliers
 
+template <int CT>
 __global__ void __launch_bounds__(LM3_THREADS, 2) k_lm_spread(LmArgs a) {
-    __shared__ float s_red[LM3_THREADS * 8];         // 8 partial values per thread per pass
-    __shared__ double s_H[64][12];                    // current pose per local hypothesis
-    __shared__ double s_Hn[64][12];                   // trial pose
-    __shared__ double s_lambda[64];
-    __shared__ float s_tot[64][28];
-    __shared__ int s_state[64];                       // 1 active, 0 stopped
-    __shared__ int s_nin[64];
+    constexpr int PAIRS = LM3_THREADS / CT;           // (hypothesis, group) pairs of a block
+    __shared__ float s_red[PAIRS * (LM3_NV + 4)];     // partial sums of each pair
+    __shared__ float s_trial[PAIRS];
+    __shared__ double s_H[LM3_HMAX][12];              // current pose per hypothesis of the part
+    __shared__ double s_Hn[LM3_HMAX][12];             // trial pose
+    __shared__ double s_lambda[LM3_HMAX];
+    __shared__ float s_tot[LM3_HMAX][LM3_NV];
+    __shared__ int s_state[LM3_HMAX];                 // 1 active, 0 stopped
+    constexpr int RS = LM3_NV + 4;                    // odd row stride
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int rank = CT > 1 ? (int)cluster.block_rank() : 0;
     const int b = blockIdx.y;
     const int n = a.q.n_cur[b];
     if (!round_active(n, a.p)) return;
-    // hypotheses of this block: [h0, h0 + nb)
+    // hypotheses of this part: [h0, h0 + nb)
     const int per = (n + LM3_BPQ - 1) / LM3_BPQ;
-    const int h0 = blockIdx.x * per;
+    const int h0 = (int)(blockIdx.x / CT) * per;
     const int nb = min(per, n - h0);
     if (nb <= 0) return;
     int HB = 1;
     while (HB < nb) HB <<= 1;
-    const int G = LM3_THREADS / HB;
-    const int t = threadIdx.x;
-    const int hl = t % HB, g = t / HB;
+    const int G = LM3_THREADS / HB, GL = G / CT;      // groups, and those of this block
+    const int t = threadIdx.x, sub = t % CT, pair = t / CT;
+    const int hl = pair % HB, g = pair / HB * CT + rank;
     const bool mine = hl < nb;
     const int NC = a.p.n_cull;
     const size_t row0 = (size_t)b * a.p.max_pix;
@@ -300,7 +322,7 @@ __global__ void __launch_bounds__(LM3_THREADS, 2) k_lm_spread(LmArgs a) {
     const float4 *t1 = a.q.tab1 + row0 * stride;
     const float *t2 = a.q.tab2 + row0 * stride;
     const int16_t *tcnt = a.q.tab_cnt + row0;
-    // correspondences [pixel][nb] of this block's hypotheses (local mode index, -1 none)
+    // correspondences [pixel][nb] of the part's hypotheses (local mode index, -1 none)
     int32_t *corr = a.q.corr + ((size_t)b * NC + h0) * a.p.max_pix;
     const float thr2 = (float)(a.p.lm_inlier_thresh * a.p.lm_inlier_thresh);
     const bool cov = a.p.use_cov;
@@ -310,111 +332,135 @@ __global__ void __launch_bounds__(LM3_THREADS, 2) k_lm_spread(LmArgs a) {
         s_state[i] = 1;
     }
     __syncthreads();
+    // Tree sum over the groups of value k of row `stride_` arrays in `part`
+    // (left in the rows of local group 0), then over the cluster; f(h, k, sum).
+    auto reduce = [&](float *part, int nv, int rs, auto f) {
+        __syncthreads();
+        for (int s = GL >> 1; s > 0; s >>= 1) {
+            for (int e = t; e < s * HB * nv; e += LM3_THREADS)
+                part[e / nv * rs + e % nv] += part[(e / nv + s * HB) * rs + e % nv];
+            __syncthreads();
+        }
+        if (CT > 1) cluster.sync();
+        for (int e = t; e < nb * nv; e += LM3_THREADS) {
+            const int h = e / nv, k = e % nv;
+            float v[CT];
+#pragma unroll
+            for (int r = 0; r < CT; ++r) v[r] = (CT > 1 ? cluster.map_shared_rank(part, r) : part)[h * rs + k];
+#pragma unroll
+            for (int s = CT / 2; s > 0; s >>= 1)
+#pragma unroll
+                for (int r = 0; r < s; ++r) v[r] += v[r + s];
+            f(h, k, v[0]);
+        }
+        __syncthreads();
+    };
+    const int steps = (a.n_pix + G - 1) / G;  // pixels of a group, the same for every lane
     unsigned w_pairs = 0, w_modes = 0, w_in = 0, w_trial = 0;
     for (int it = 0; it < a.p.lm_max_iter; ++it) {
         const bool act = mine && s_state[hl];
-        if (!__syncthreads_or(act)) break;
+        if (!__syncthreads_or(act)) break;  // the same in every block of the cluster
         float acc[28];
 #pragma unroll
         for (int k = 0; k < 28; ++k) acc[k] = 0.f;
         int nin = 0;
-        if (act) {
-            const float r00 = (float)s_H[hl][0], r01 = (float)s_H[hl][1], r02 = (float)s_H[hl][2], tx = (float)s_H[hl][3];
-            const float r10 = (float)s_H[hl][4], r11 = (float)s_H[hl][5], r12 = (float)s_H[hl][6], ty = (float)s_H[hl][7];
-            const float r20 = (float)s_H[hl][8], r21 = (float)s_H[hl][9], r22 = (float)s_H[hl][10], tz = (float)s_H[hl][11];
-            for (int i = g; i < a.n_pix; i += G) {
-                const int cnt = tcnt[i];
+        {
+            float P[12];
+#pragma unroll
+            for (int k = 0; k < 12; ++k) P[k] = act ? (float)s_H[hl][k] : 0.f;
+            for (int st = 0; st < steps; ++st) {
+                const int i = st * G + g;
+                const bool on = act && i < a.n_pix;
+                const int cnt = on ? (int)tcnt[i] : 0;
+                const size_t base = (size_t)i * stride;
+                float y0 = 0.f, y1 = 0.f, y2 = 0.f;
+                if (cnt > 0) {
+                    const float4 x = xcs[i];
+                    y0 = fmaf(P[0], x.x, fmaf(P[1], x.y, fmaf(P[2], x.z, P[3])));
+                    y1 = fmaf(P[4], x.x, fmaf(P[5], x.y, fmaf(P[6], x.z, P[7])));
+                    y2 = fmaf(P[8], x.x, fmaf(P[9], x.y, fmaf(P[10], x.z, P[11])));
+                }
+                float best = INFINITY;
                 int best_m = -1;
+                if (cov) {
+#pragma unroll 4
+                    for (int m = sub; m < cnt; m += CT) {
+                        const float4 m0 = __ldg(&t0[base + m]), m1 = __ldg(&t1[base + m]);
+                        const float u22 = __ldg(&t2[base + m]);
+                        const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
+                        const float w0 = fmaf(m0.w, v0, fmaf(m1.x, v1, m1.y * v2));
+                        const float w1 = fmaf(m1.z, v1, m1.w * v2);
+                        const float w2 = u22 * v2;
+                        const float d2 = fmaf(w0, w0, fmaf(w1, w1, w2 * w2));
+                        if (d2 < best) {
+                            best = d2;
+                            best_m = m;
+                        }
+                    }
+                } else {
+#pragma unroll 4
+                    for (int m = sub; m < cnt; m += CT) {
+                        const float4 m0 = __ldg(&t0[base + m]);
+                        const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
+                        const float d2 = fmaf(v0, v0, fmaf(v1, v1, v2 * v2));
+                        if (d2 < best) {
+                            best = d2;
+                            best_m = m;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int off = 1; off < CT; off <<= 1) {
+                    const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+                    const int om = __shfl_xor_sync(0xffffffffu, best_m, off);
+                    if (om >= 0 && (best_m < 0 || ob < best || (ob == best && om < best_m))) {
+                        best = ob;
+                        best_m = om;
+                    }
+                }
+                if (!on || sub != 0) continue;
                 if (cnt > 0) {
                     ++w_pairs;
                     w_modes += cnt;
-                    const float4 x = xcs[i];
-                    const float y0 = fmaf(r00, x.x, fmaf(r01, x.y, fmaf(r02, x.z, tx)));
-                    const float y1 = fmaf(r10, x.x, fmaf(r11, x.y, fmaf(r12, x.z, ty)));
-                    const float y2 = fmaf(r20, x.x, fmaf(r21, x.y, fmaf(r22, x.z, tz)));
-                    const size_t base = (size_t)i * stride;
-                    float best = INFINITY;
-                    if (cov) {
-                        for (int m = 0; m < cnt; ++m) {
-                            const float4 m0 = __ldg(&t0[base + m]), m1 = __ldg(&t1[base + m]);
-                            const float u22 = __ldg(&t2[base + m]);
-                            const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
-                            const float w0 = fmaf(m0.w, v0, fmaf(m1.x, v1, m1.y * v2));
-                            const float w1 = fmaf(m1.z, v1, m1.w * v2);
-                            const float w2 = u22 * v2;
-                            const float d2 = fmaf(w0, w0, fmaf(w1, w1, w2 * w2));
-                            if (d2 < best) {
-                                best = d2;
-                                best_m = m;
-                            }
+                }
+                if (best_m >= 0) {
+                    const float4 m0 = __ldg(&t0[base + best_m]);
+                    const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
+                    if (fmaf(v0, v0, fmaf(v1, v1, v2 * v2)) <= thr2) {
+                        ++nin;
+                        ++w_in;
+                        if (cov) {
+                            const float4 m1 = __ldg(&t1[base + best_m]);
+                            lm_accumulate(y0, y1, y2, v0, v1, v2, m0.w, m1.x, m1.y, m1.z, m1.w,
+                                           __ldg(&t2[base + best_m]), acc);
+                        } else {
+                            lm_accumulate(y0, y1, y2, v0, v1, v2, 1.f, 0.f, 0.f, 1.f, 0.f, 1.f, acc);
                         }
                     } else {
-                        for (int m = 0; m < cnt; ++m) {
-                            const float4 m0 = __ldg(&t0[base + m]);
-                            const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
-                            const float d2 = fmaf(v0, v0, fmaf(v1, v1, v2 * v2));
-                            if (d2 < best) {
-                                best = d2;
-                                best_m = m;
-                            }
-                        }
-                    }
-                    if (best_m >= 0) {
-                        const float4 m0 = __ldg(&t0[base + best_m]);
-                        const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
-                        if (fmaf(v0, v0, fmaf(v1, v1, v2 * v2)) <= thr2) {
-                            ++nin;
-                            ++w_in;
-                            if (cov) {
-                                const float4 m1 = __ldg(&t1[base + best_m]);
-                                lm_accumulate(y0, y1, y2, v0, v1, v2, m0.w, m1.x, m1.y, m1.z, m1.w,
-                                               __ldg(&t2[base + best_m]), acc);
-                            } else {
-                                lm_accumulate(y0, y1, y2, v0, v1, v2, 1.f, 0.f, 0.f, 1.f, 0.f, 1.f, acc);
-                            }
-                        } else {
-                            best_m = -1;
-                        }
+                        best_m = -1;
                     }
                 }
                 corr[(size_t)i * nb + hl] = best_m;
             }
         }
-        // tree reduction of the 28 sums and the inlier count over the groups
-        for (int part = 0; part < 4; ++part) {
-            for (int k = 0; k < 7; ++k) s_red[t * 8 + k] = acc[part * 7 + k];
-            if (part == 0) s_red[t * 8 + 7] = __int_as_float(nin);
-            __syncthreads();
-            for (int s = G >> 1; s > 0; s >>= 1) {
-                if (g < s)
-                    for (int k = 0; k < 8; ++k) {
-                        if (k == 7 && part != 0) continue;
-                        const int o1 = t * 8 + k, o2 = (t + s * HB) * 8 + k;
-                        if (k == 7)
-                            s_red[o1] = __int_as_float(__float_as_int(s_red[o1]) + __float_as_int(s_red[o2]));
-                        else
-                            s_red[o1] += s_red[o2];
-                    }
-                __syncthreads();
-            }
-            if (g == 0 && mine) {
-                for (int k = 0; k < 7; ++k) s_tot[hl][part * 7 + k] = s_red[t * 8 + k];
-                if (part == 0) s_nin[hl] = __float_as_int(s_red[t * 8 + 7]);
-            }
-            __syncthreads();
+        if (sub == 0) {
+#pragma unroll
+            for (int k = 0; k < 28; ++k) s_red[pair * RS + k] = acc[k];
+            s_red[pair * RS + 28] = (float)nin;
         }
+        reduce(s_red, LM3_NV, RS, [&](int h, int k, float v) { s_tot[h][k] = v; });
         // FP64 solve per active hypothesis
-        if (g == 0 && act) {
-            int status = s_nin[hl] < 3 ? 1 : 0;
+        if (t < nb && s_state[t]) {
+            int status = s_tot[t][28] < 3.f ? 1 : 0;
             double step[6];
             if (!status) {
                 double A[36], rhs[6];
                 int k = 0;
                 for (int r = 0; r < 6; ++r)
-                    for (int c = r; c < 6; ++c, ++k) A[6 * r + c] = A[6 * c + r] = (double)s_tot[hl][k];
+                    for (int c = r; c < 6; ++c, ++k) A[6 * r + c] = A[6 * c + r] = (double)s_tot[t][k];
                 for (int r = 0; r < 6; ++r) {
-                    A[6 * r + r] += s_lambda[hl] * (double)s_tot[hl][r * 6 - r * (r - 1) / 2];
-                    rhs[r] = -(double)s_tot[hl][21 + r];
+                    A[6 * r + r] += s_lambda[t] * (double)s_tot[t][r * 6 - r * (r - 1) / 2];
+                    rhs[r] = -(double)s_tot[t][21 + r];
                 }
                 if (!chol_solve6(A, rhs, step)) {
                     status = 1;
@@ -425,68 +471,93 @@ __global__ void __launch_bounds__(LM3_THREADS, 2) k_lm_spread(LmArgs a) {
                 }
             }
             if (status) {
-                s_state[hl] = 0;
+                s_state[t] = 0;
             } else {
                 double Hn[12];
-                for (int i = 0; i < 12; ++i) Hn[i] = s_H[hl][i];
+                for (int i = 0; i < 12; ++i) Hn[i] = s_H[t][i];
                 se3_left(step, Hn);
-                for (int i = 0; i < 12; ++i) s_Hn[hl][i] = Hn[i];
+                for (int i = 0; i < 12; ++i) s_Hn[t][i] = Hn[i];
             }
         }
         __syncthreads();
-        // trial cost with the same correspondences
+        // Trial cost with the same correspondences.  The CT lanes of a pair
+        // take a pixel each, their residuals are added in pixel order.
         const bool act2 = mine && s_state[hl];
         float trial = 0.f;
-        if (act2) {
-            const float s00 = (float)s_Hn[hl][0], s01 = (float)s_Hn[hl][1], s02 = (float)s_Hn[hl][2], u0t = (float)s_Hn[hl][3];
-            const float s10 = (float)s_Hn[hl][4], s11 = (float)s_Hn[hl][5], s12 = (float)s_Hn[hl][6], u1t = (float)s_Hn[hl][7];
-            const float s20 = (float)s_Hn[hl][8], s21 = (float)s_Hn[hl][9], s22 = (float)s_Hn[hl][10], u2t = (float)s_Hn[hl][11];
-            for (int i = g; i < a.n_pix; i += G) {
-                const int m = corr[(size_t)i * nb + hl];
-                if (m < 0) continue;
-                ++w_trial;
-                const float4 x = xcs[i];
-                const size_t e = (size_t)i * stride + m;
-                const float4 m0 = __ldg(&t0[e]);
-                const float y0 = fmaf(s00, x.x, fmaf(s01, x.y, fmaf(s02, x.z, u0t)));
-                const float y1 = fmaf(s10, x.x, fmaf(s11, x.y, fmaf(s12, x.z, u1t)));
-                const float y2 = fmaf(s20, x.x, fmaf(s21, x.y, fmaf(s22, x.z, u2t)));
-                const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
-                if (cov) {
-                    const float4 m1 = __ldg(&t1[e]);
-                    const float r0 = fmaf(m0.w, v0, fmaf(m1.x, v1, m1.y * v2));
-                    const float r1 = fmaf(m1.z, v1, m1.w * v2);
-                    const float r2 = __ldg(&t2[e]) * v2;
-                    trial = fmaf(r0, r0, fmaf(r1, r1, fmaf(r2, r2, trial)));
-                } else {
-                    trial = fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, trial)));
+        {
+            float P[12];
+#pragma unroll
+            for (int k = 0; k < 12; ++k) P[k] = act2 ? (float)s_Hn[hl][k] : 0.f;
+            for (int st = 0; st < steps; st += CT) {
+                const int i = (st + sub) * G + g;
+                const int m = act2 && i < a.n_pix ? corr[(size_t)i * nb + hl] : -1;
+                float r0 = 0.f, r1 = 0.f, r2 = 0.f;
+                if (m >= 0) {
+                    ++w_trial;
+                    const float4 x = xcs[i];
+                    const size_t e = (size_t)i * stride + m;
+                    const float4 m0 = __ldg(&t0[e]);
+                    const float y0 = fmaf(P[0], x.x, fmaf(P[1], x.y, fmaf(P[2], x.z, P[3])));
+                    const float y1 = fmaf(P[4], x.x, fmaf(P[5], x.y, fmaf(P[6], x.z, P[7])));
+                    const float y2 = fmaf(P[8], x.x, fmaf(P[9], x.y, fmaf(P[10], x.z, P[11])));
+                    const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
+                    if (cov) {
+                        const float4 m1 = __ldg(&t1[e]);
+                        r0 = fmaf(m0.w, v0, fmaf(m1.x, v1, m1.y * v2));
+                        r1 = fmaf(m1.z, v1, m1.w * v2);
+                        r2 = __ldg(&t2[e]) * v2;
+                    } else {
+                        r0 = v0;
+                        r1 = v1;
+                        r2 = v2;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < CT; ++k) {
+                    const float q0 = __shfl_sync(0xffffffffu, r0, k, CT), q1 = __shfl_sync(0xffffffffu, r1, k, CT),
+                                q2 = __shfl_sync(0xffffffffu, r2, k, CT);
+                    trial = fmaf(q0, q0, fmaf(q1, q1, fmaf(q2, q2, trial)));  // + 0 where there is none
                 }
             }
         }
-        s_red[t * 8] = trial;
-        __syncthreads();
-        for (int s = G >> 1; s > 0; s >>= 1) {
-            if (g < s) s_red[t * 8] += s_red[(t + s * HB) * 8];
-            __syncthreads();
-        }
-        if (g == 0 && act2) {
-            if (s_red[t * 8] < s_tot[hl][27]) {
-                for (int i = 0; i < 12; ++i) s_H[hl][i] = s_Hn[hl][i];
-                s_lambda[hl] /= 10.0;
+        if (sub == 0) s_trial[pair] = trial;
+        reduce(s_trial, 1, 1, [&](int h, int, float v) {
+            if (!s_state[h]) return;
+            if (v < s_tot[h][27]) {
+                for (int i = 0; i < 12; ++i) s_H[h][i] = s_Hn[h][i];
+                s_lambda[h] /= 10.0;
             } else {
-                s_lambda[hl] *= 10.0;
+                s_lambda[h] *= 10.0;
             }
-        }
-        __syncthreads();
+        });
     }
-    for (int i = t; i < nb * 12; i += LM3_THREADS)
-        a.q.cur_pose[((size_t)b * NC + h0 + i / 12) * 12 + i % 12] = s_H[i / 12][i % 12];
-    if (a.work && mine) {
+    if (rank == 0)
+        for (int i = t; i < nb * 12; i += LM3_THREADS)
+            a.q.cur_pose[((size_t)b * NC + h0 + i / 12) * 12 + i % 12] = s_H[i / 12][i % 12];
+    if (a.work && (w_pairs | w_trial)) {
         atomicAdd(&a.work[W_LM_PAIRS], (unsigned long long)w_pairs);
         atomicAdd(&a.work[W_LM_MODES], (unsigned long long)w_modes);
         atomicAdd(&a.work[W_LM_INLIERS], (unsigned long long)w_in);
         atomicAdd(&a.work[W_LM_TRIAL], (unsigned long long)w_trial);
     }
+    if (CT > 1) cluster.sync();  // no block leaves while another may still read its shared memory
+}
+
+template <int CT>
+static rl_status launch_lm_spread(const LmArgs &a, int n, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(LM3_BPQ * CT, n);
+    cfg.blockDim = dim3(LM3_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CT;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    RL_CK(cudaLaunchKernelEx(&cfg, k_lm_spread<CT>, a));
+    return RL_OK;
 }
 
 // z-depth of the first box face hit by the ray of pixel (u, v) (exit point
@@ -828,10 +899,11 @@ bool lm_uses_cluster(const RParams &p) {
 // kernel; n_cull <= 64 (checked when the relocaliser is created).
 rl_status launch_lm(const LmArgs &a, int n, cudaStream_t s) {
     if (lm_uses_cluster(a.p)) return launch_lm_cluster(a, n, s);
-    dim3 grid(LM3_BPQ, n);
-    k_lm_spread<<<grid, LM3_THREADS, 0, s>>>(a);
-    RL_LAUNCH_CK();
-    return RL_OK;
+    const int fit = 2 * a.sm_count / LM3_BPQ;  // parts of one block each that fit two blocks per SM
+    if (8 * a.n_active <= fit) return launch_lm_spread<8>(a, n, s);
+    if (4 * a.n_active <= fit) return launch_lm_spread<4>(a, n, s);
+    if (2 * a.n_active <= fit) return launch_lm_spread<2>(a, n, s);
+    return launch_lm_spread<1>(a, n, s);
 }
 
 // Kernel attributes set once, outside any stream capture.
