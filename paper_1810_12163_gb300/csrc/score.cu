@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(256) k_energy(EnergyArgs a) {
 
 __global__ void __launch_bounds__(1024) k_select(SelectArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ float s_tile[64][33];
     float *sE = (float *)smem;                       // [n]
     int *sS = (int *)(sE + a.p.n_hyp);               // [n]
     double *sP = (double *)(sS + a.p.n_hyp);         // [n_cull][12]
@@ -185,10 +186,45 @@ __global__ void __launch_bounds__(1024) k_select(SelectArgs a) {
     const int n = a.count[b];
     if (a.phase == 1 && !round_active(n, a.p)) return;
     const int N = a.p.n_hyp, NC = a.p.n_cull;
+    const bool from_parts = !(a.phase == 1 && a.energy_from_lm);
+    // Long rows of partial energies (modes too many for 32 pixels a chunk) are
+    // read by the whole block, 64 rows by 32 chunks at a time and the next
+    // tile's loads in flight, and summed in chunk order from shared memory: a
+    // thread walking its own row of 125 to 875 chunks took 30 to 75 us.
+    // Shorter rows are a line or two, read directly.
+    const bool tiled = from_parts && a.n_chunks_used > 64;
+    if (tiled) {
+        const int nct = (a.n_chunks_used + 31) / 32, nt = (n + 63) / 64 * nct;
+        const int r0 = tid >> 5, c0 = tid & 31;
+        auto part = [&](int tile, int r) {
+            const int h = tile / nct * 64 + r, c = tile % nct * 32 + c0;
+            return tile < nt && h < n && c < a.n_chunks_used ? a.part[((size_t)b * a.part_h + h) * a.n_chunks + c] : 0.f;
+        };
+        float e = 0.f, p0 = part(0, r0), p1 = part(0, r0 + 32);
+        for (int tile = 0; tile < nt; ++tile) {
+            s_tile[r0][c0] = p0;
+            s_tile[r0 + 32][c0] = p1;
+            p0 = part(tile + 1, r0);
+            p1 = part(tile + 1, r0 + 32);
+            __syncthreads();
+            const int h = tile / nct * 64 + tid, cb = tile % nct * 32;
+            if (tid < 64 && h < n) {
+                const int m = min(32, a.n_chunks_used - cb);
+                for (int c = 0; c < m; ++c) e += s_tile[tid][c];
+                if (tile % nct == nct - 1) {
+                    sE[h] = e;
+                    e = 0.f;
+                }
+            }
+            __syncthreads();
+        }
+    }
     for (int i = tid; i < n; i += blockDim.x) {
         float e = 0.f;
-        if (a.phase == 1 && a.energy_from_lm) {
+        if (!from_parts) {
             e = a.q.cur_energy[(size_t)b * NC + i];
+        } else if (tiled) {
+            e = sE[i];
         } else {
             const float *pp = a.part + ((size_t)b * a.part_h + i) * a.n_chunks;
             for (int c = 0; c < a.n_chunks_used; ++c) e += pp[c];
