@@ -354,10 +354,8 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
     constexpr int step = pairs ? 64 : 32;
     bool done = slot >= a.p.n_hyp;
     for (int base = mate * step; base < a.p.max_iter && !done; base += team * step) {
-        if (*(volatile int *)&s_best[sl] < base) {  // a team mate's success comes first
-            head = tail;
-            break;
-        }
+        // a team mate's success comes first (what is pending may come before it)
+        if (*(volatile int *)&s_best[sl] < base) break;
         if (pairs) {
             Draw dA, dB;
             bool sA, sB;
