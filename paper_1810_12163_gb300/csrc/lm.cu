@@ -1,14 +1,26 @@
 // Levenberg-Marquardt refinement of a preemptive round (Sec. 3.2.3) with one
 // thread-block cluster per frame.
 //
-// The CTAS CTAs of a cluster share the frame's surviving hypotheses
+// The RANKS CTAs of a cluster share the frame's surviving hypotheses
 // (n <= 64) and split its pixel set by tiles of LMC_P pixels: CTA c takes
-// tiles c, c + CTAS, ...  The first round (most hypotheses, fewest pixels)
+// tiles c, c + RANKS, ...  The first round (most hypotheses, fewest pixels)
 // uses clusters of 4.  Later rounds have few hypotheses and up to 3.5x the
 // pixels; a frame's LM there is a chain of passes whose length is set by its
 // slowest hypothesis, so they use clusters of 8 to shorten each pass.  The
 // cluster size is a function of the round alone, so a frame's results do not
 // depend on the batch it runs in.
+//
+// A cluster holds RANKS x SUBS CTAs: RANKS of them split the pixels, and SUBS
+// sets of these split the listed hypotheses.  What a thread sums, and in
+// which order, depends on RANKS and on the hypotheses listed alone; SUBS only
+// spreads the hypotheses over more CTAs, whose lanes then share the mode scan
+// of a pair (S lanes of it each).  A call of few frames leaves most SMs idle
+// with SUBS = 1 (one frame: 4 of 152), so SUBS grows while the call's CTAs
+// fit the GPU.  Measured on 640x480 frames of up to 50 modes per pixel: first
+// round of 8 frames 1391 us with SUBS = 1, 941 with 4; of one frame 572 and
+// 439; a later round (RANKS = 8) of 8 frames 445 and, with 2, 365.  What
+// bounds it then is the issue of two warps per sub-partition (36% of cycles)
+// on the scans and the normal equations' serial chains.
 //
 // A pass streams the CTA's tiles of the mode table (rows of decoded M(u))
 // into shared memory with bulk asynchronous copies on an mbarrier pipeline.
@@ -43,6 +55,8 @@
 // before it exits.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "internal.h"
 #include "kernels.h"
 #include "lm_dev.cuh"
@@ -51,11 +65,13 @@ namespace rl {
 
 namespace cg = cooperative_groups;
 
-constexpr int LMC_CTAS_FIRST = 4;  // cluster size of the first preemptive round
-constexpr int LMC_CTAS_LATER = 8;  // and of the later rounds
+constexpr int LMC_RANKS_FIRST = 4;  // CTAs that split the pixels in the first preemptive round
+constexpr int LMC_RANKS_LATER = 8;  // and in the later rounds
 constexpr int LMC_THREADS = 256;
 constexpr int LMC_P = 16;        // pixels per tile (max_pix is a multiple)
-constexpr int LMC_STAGES = 2;
+constexpr int LMC_STAGES = 2;      // tiles in flight with two CTAs per SM (SUBS = 1)
+constexpr int LMC_STAGES_SUB = 4;  // and with one (SUBS > 1)
+constexpr int LMC_SPLIT_MODES = 24;  // |M(u)| bound from which the CTAs of a set share scans
 constexpr int LMC_HMAX = 64;
 constexpr int LMC_NV = 31;       // 21 J^T J + 6 J^T r + cost, inlier count, trial cost, Eq. 5 energy
 constexpr int LMC_PS = 33;       // odd stride of the per-thread partials (no bank conflicts)
@@ -76,7 +92,7 @@ __host__ __device__ inline uint32_t lmc_a16(uint32_t x) { return (x + 15u) & ~15
 // Shared-memory layout for rows of `stride` modes.  Region 0 holds the
 // staged tiles during the pixel pass and the per-thread partial sums during
 // the reductions (never both at once).
-__host__ __device__ inline LmcLayout lmc_layout(int stride, bool cov) {
+__host__ __device__ inline LmcLayout lmc_layout(int stride, bool cov, int n_stages) {
     LmcLayout L;
     const uint32_t rows = (uint32_t)LMC_P * (uint32_t)stride;
     uint32_t o = 0;
@@ -87,7 +103,7 @@ __host__ __device__ inline LmcLayout lmc_layout(int stride, bool cov) {
     L.cnt = o; o += lmc_a16(LMC_P * 2);
     L.stage = o;
     L.tx = rows * 16 + (cov ? rows * 20 : 0) + LMC_P * 16 + LMC_P * 2;
-    const uint32_t stages = LMC_STAGES * L.stage;
+    const uint32_t stages = (uint32_t)n_stages * L.stage;
     const uint32_t partials = LMC_THREADS * LMC_PS * 4;
     o = lmc_a16(stages > partials ? stages : partials);
     L.H = o; o += LMC_HMAX * 12 * 8;
@@ -102,7 +118,7 @@ __host__ __device__ inline LmcLayout lmc_layout(int stride, bool cov) {
     L.act = o; o += LMC_HMAX * 4 + 16;  // list, then its length
     L.list = o; o += LMC_LIST * 4;      // pairs to search in full (int16) and their nearest modes (int16)
     L.flag = o; o += 16;
-    L.bar = o; o += LMC_STAGES * 8;
+    L.bar = o; o += 2 * (uint32_t)n_stages * 8;  // full and empty barrier of each stage
     L.total = lmc_a16(o);
     return L;
 }
@@ -127,8 +143,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, uint32_t limit = kWaitLimit) {
     for (uint32_t i = 0; i < limit; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
+    return false;
+}
+
+// The same, given up as soon as another thread of the CTA has given up.
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, uint32_t limit,
+                                                  const volatile int *abort) {
+    for (uint32_t i = 0; i < limit && !*abort; ++i)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
@@ -205,17 +233,19 @@ __device__ __noinline__ void lm_solve_half(const float *T, double lambda, const 
     }
 }
 
-template <int CTAS>
-__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k_lm_cluster(LmArgs a) {
+template <int RANKS, int SUBS>
+__global__ void __cluster_dims__(RANKS *SUBS, 1, 1) __launch_bounds__(LMC_THREADS, SUBS == 1 ? 2 : 1) k_lm_cluster(LmArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     cg::cluster_group cluster = cg::this_cluster();
-    const int crank = (int)cluster.block_rank();
+    // this CTA's share of the pixels (crank) and of the listed hypotheses (hset)
+    const int crank = (int)cluster.block_rank() % RANKS, hset = (int)cluster.block_rank() / RANKS;
     const int b = blockIdx.y;
     const int n = a.q.n_cur[b];
     if (!round_active(n, a.p)) return;  // same n in every CTA of the cluster
     const bool cov = a.p.use_cov;
     const int stride = a.p.mpad;
-    const LmcLayout L = lmc_layout(stride, cov);
+    constexpr int STAGES = SUBS == 1 ? LMC_STAGES : LMC_STAGES_SUB;
+    const LmcLayout L = lmc_layout(stride, cov, STAGES);
     const int t = threadIdx.x;
 
     float *s_acc = (float *)smem;
@@ -245,32 +275,36 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
     int16_t *corr0 = (int16_t *)(a.q.corr + (size_t)b * NC * a.p.max_pix);
     const size_t cstride = (size_t)NC * a.p.max_pix;
     const int n_tiles = (a.n_pix + LMC_P - 1) / LMC_P;
-    const int my_tiles = crank < n_tiles ? (n_tiles - crank + CTAS - 1) / CTAS : 0;
+    const int my_tiles = crank < n_tiles ? (n_tiles - crank + RANKS - 1) / RANKS : 0;
     const float thr2 = (float)(a.p.lm_inlier_thresh * a.p.lm_inlier_thresh);
     // direct passes after the first: at most LMC_DIRECT hypotheses, and the
     // CTA's local pixel indices fit the list entries' 10 bits (the same
     // decision in every CTA of the cluster)
-    const bool dir_ok = n <= LMC_DIRECT && (n_tiles + CTAS - 1) / CTAS * LMC_P <= 1024;
+    const bool dir_ok = n <= LMC_DIRECT && (n_tiles + RANKS - 1) / RANKS * LMC_P <= 1024;
 
-    // Lane roles of a pass over the k hypotheses listed in s_act: list entry
-    // hs = (t / S) % HB on pixel group g = (t / S) / HB.  With fewer than 16
-    // hypotheses a tile has fewer (hypothesis, pixel) pairs than threads: S
-    // adjacent lanes then share a pair and split its mode scan (every S-th
-    // mode), and the nearest mode is found by a shuffle reduction (ties: lower
-    // index, as a sequential scan finds it).  hl: the hypothesis served.
-    int HB = 1, S = 1, Gp = 1, sub = 0, hs = 0, g = 0, hl = 0, k_act = 0;
+    // Lane roles of a pass over the k hypotheses listed in s_act.  HB = the
+    // next power of two >= k; the pixels of a tile are dealt to Gp groups (as
+    // many as 256 threads hold pairs of HB entries, 16 at most, the tile's
+    // pixels, while tiles are staged).  This CTA has the HQ entries hset * HQ
+    // + 0, 1, ...; entry hs and group g are served by the S adjacent lanes
+    // left over per pair, which split its mode scan (every S-th mode), and
+    // the nearest mode is found by a shuffle reduction (ties: lower index, as
+    // a sequential scan finds it).  hl: the hypothesis served.
+    int HB = 1, HQ = 1, S = 1, Gp = 1, sub = 0, hs = 0, g = 0, hl = 0, k_act = 0;
     bool mine = false;
     auto roles = [&](int k, bool direct) {
         k_act = k;
         HB = 1;
         while (HB < k) HB <<= 1;
-        const int G = LMC_THREADS / HB;
-        S = !direct && G > LMC_P ? G / LMC_P : 1;
-        Gp = G / S;  // pixel groups
+        HQ = HB > SUBS ? HB / SUBS : 1;
+        Gp = LMC_THREADS / HB;
+        if (!direct && Gp > LMC_P) Gp = LMC_P;
+        S = direct ? 1 : LMC_THREADS / (HQ * Gp);
         sub = t % S;
-        hs = (t / S) % HB;
-        g = (t / S) / HB;
-        mine = hs < k;
+        const int pr = t / S;  // direct passes with SUBS > 1 leave threads without a pair
+        hs = hset * HQ + pr % HQ;
+        g = pr / HQ;
+        mine = g < Gp && hs < k;
         hl = mine ? s_act[hs] : 0;
     };
 
@@ -287,18 +321,37 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
     }
     if (t == 0) {
         *s_abort = 0;
-        for (int s = 0; s < LMC_STAGES; ++s) mbar_init(bar0 + 8 * s, 1);
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(bar0 + 8 * s, 1);
+            mbar_init(bar0 + 8 * (STAGES + s), LMC_THREADS / 32);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
 
-    // thread 0 is the producer: my j-th tile into stage s
-    // per stage: copies issued (thread 0), phases consumed, phases seen complete
-    uint32_t issued[LMC_STAGES] = {}, waited[LMC_STAGES] = {}, landed[LMC_STAGES] = {};
-    auto issue = [&](int j, int s) {
+    // Tiles are numbered through all passes: tile number q uses stage q %
+    // STAGES for the (q / STAGES)-th time.  Thread 0 is the producer.  With
+    // SUBS > 1 (one CTA per SM) a warp that is done with a tile arrives at its
+    // stage's empty barrier, so the warps need not keep step within a pass;
+    // with two CTAs per SM a block barrier per tile is as fast.
+    uint32_t q_pass = 0;                   // number of the pass's first tile
+    uint32_t q_issued = 0, q_landed = 0;   // thread 0: tiles issued, tiles seen to land
+    auto give_up = [&]() {
+        *s_abort = 1;
+        a.q.dev_err[b] = 1;
+    };
+    auto full_ok = [&](uint32_t q) {
+        return mbar_wait_bounded(bar0 + 8 * (q % STAGES), (q / STAGES) & 1u, a.wait_limit, s_abort);
+    };
+    auto issue = [&](int j) {  // the pass's j-th tile of this CTA
+        const uint32_t q = q_pass + (uint32_t)j, s = q % STAGES;
+        if (SUBS > 1 && q >= STAGES && !mbar_wait_bounded(bar0 + 8 * (STAGES + s), (q / STAGES - 1) & 1u, kWaitLimit, s_abort)) {
+            give_up();
+            return;
+        }
         const uint32_t bar = bar0 + 8 * s;
         const uint32_t st = sbase + s * L.stage;
-        const size_t r = (size_t)(crank + j * CTAS) * LMC_P;  // first row of the tile
+        const size_t r = (size_t)(crank + j * RANKS) * LMC_P;  // first row of the tile
         const uint32_t rows = (uint32_t)LMC_P * stride;
         mbar_expect_tx(bar, L.tx);
         bulk_g2s(st + L.t0, g_t0 + r * stride, rows * 16, bar);
@@ -308,7 +361,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
         }
         bulk_g2s(st + L.xc, g_xc + r, LMC_P * 16, bar);
         bulk_g2s(st + L.cnt, g_cnt + r, LMC_P * 2, bar);
-        ++issued[s];
+        ++q_issued;
     };
 
     unsigned w_pairs = 0, w_modes = 0, w_in = 0, w_trial = 0, w_evals = 0;
@@ -468,36 +521,50 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
         return true;
     };
 
-    // One tile of a pass with S > 1: pixel g of the tile for hypothesis hl,
-    // modes sub, sub + S, ... on this lane; every lane reaches the shuffles.
-    auto split_tile = [&](bool live, int s, int j, bool trial, bool rec, const int16_t *cr, int16_t *cw, LmcPass &o,
+    // One tile of a pass with S > 1: pixels g, g + Gp, ... of the tile for
+    // hypothesis hl, modes sub, sub + S, ... on this lane; every lane reaches
+    // the shuffles.  REC: anchors the pair (direct passes follow).
+    auto split_tile = [&](auto rec_t, bool live, int s, int j, bool trial, const int16_t *cr, int16_t *cw, LmcPass &o,
                           float r00, float r01, float r02, float tx, float r10, float r11, float r12, float ty,
                           float r20, float r21, float r22, float tz) {
+        constexpr bool REC = decltype(rec_t)::value;
         const uint8_t *st = smem + s * L.stage;
         const float4 *s_t0 = (const float4 *)(st + L.t0);
         const float4 *s_t1 = (const float4 *)(st + L.t1);
         const float *s_t2 = (const float *)(st + L.t2);
         const float4 *s_xc = (const float4 *)(st + L.xc);
         const int16_t *s_cnt = (const int16_t *)(st + L.cnt);
-        const int i0 = (crank + j * CTAS) * LMC_P;
-        const int il = g;
-        const bool on = live && il < min(LMC_P, a.n_pix - i0);
-        const int cnt = on ? (int)s_cnt[il] : 0;
-        const int base = il * stride;
-        float y0 = 0.f, y1 = 0.f, y2 = 0.f;
-        if (cnt > 0) {
-            const float4 x = s_xc[il];
-            y0 = fmaf(r00, x.x, fmaf(r01, x.y, fmaf(r02, x.z, tx)));
-            y1 = fmaf(r10, x.x, fmaf(r11, x.y, fmaf(r12, x.z, ty)));
-            y2 = fmaf(r20, x.x, fmaf(r21, x.y, fmaf(r22, x.z, tz)));
-        }
-        float best = INFINITY, second = INFINITY;  // second: for the anchor (direct passes follow)
-        float fro2 = 0.f, mu2 = 0.f;
-        int best_m = -1;
-        if (rec)
-            for (int m = sub; m < cnt; m += S) row_maxima(s_t0 + base, s_t1 + base, s_t2 + base, m, fro2, mu2);
-        if (cov) {
-            auto d2of = [&](int m) {
+        const int i0 = (crank + j * RANKS) * LMC_P;
+        const int np = min(LMC_P, a.n_pix - i0);
+        for (int il0 = 0; il0 < LMC_P; il0 += Gp) {
+            const int il = il0 + g;
+            const bool on = live && il < np;
+            const int cnt = on ? (int)s_cnt[il] : 0;
+            const int base = il * stride;
+            const size_t ci = (size_t)(i0 + il) * n + hl;
+            const int m_old = trial && on ? (int)cr[ci] : -1;  // read before the scan, used after it
+            float y0 = 0.f, y1 = 0.f, y2 = 0.f;
+            if (cnt > 0) {
+                const float4 x = s_xc[il];
+                y0 = fmaf(r00, x.x, fmaf(r01, x.y, fmaf(r02, x.z, tx)));
+                y1 = fmaf(r10, x.x, fmaf(r11, x.y, fmaf(r12, x.z, ty)));
+                y2 = fmaf(r20, x.x, fmaf(r21, x.y, fmaf(r22, x.z, tz)));
+            }
+            float best = INFINITY, second = INFINITY;  // second: for the anchor
+            float fro2 = 0.f, mu2 = 0.f;
+            int best_m = -1;
+            if (REC)
+                for (int m = sub; m < cnt; m += S) row_maxima(s_t0 + base, s_t1 + base, s_t2 + base, m, fro2, mu2);
+            auto take = [&](float d, int m) {
+                if (d < best) {
+                    if (REC) second = best;
+                    best = d;
+                    best_m = m;
+                } else if (REC) {
+                    second = fminf(second, d);
+                }
+            };
+            auto d2cov = [&](int m) {
                 const float4 m0 = s_t0[base + m], m1 = s_t1[base + m];
                 const float u22 = s_t2[base + m];
                 const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
@@ -506,91 +573,91 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
                 const float w2 = u22 * v2;
                 return fmaf(w0, w0, fmaf(w1, w1, w2 * w2));
             };
-            int m = sub;
-            for (; m + S < cnt; m += 2 * S) {
-                const float da = d2of(m), db = d2of(m + S);
-                if (da < best) { second = best; best = da; best_m = m; } else { second = fminf(second, da); }
-                if (db < best) { second = best; best = db; best_m = m + S; } else { second = fminf(second, db); }
-            }
-            if (m < cnt) {
-                const float da = d2of(m);
-                if (da < best) { second = best; best = da; best_m = m; } else { second = fminf(second, da); }
-            }
-        } else {
-            auto d2of = [&](int m) {
+            auto d2euc = [&](int m) {
                 const float4 m0 = s_t0[base + m];
                 const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
                 return fmaf(v0, v0, fmaf(v1, v1, v2 * v2));
             };
-            int m = sub;
-            for (; m + S < cnt; m += 2 * S) {
-                const float da = d2of(m), db = d2of(m + S);
-                if (da < best) { second = best; best = da; best_m = m; } else { second = fminf(second, da); }
-                if (db < best) { second = best; best = db; best_m = m + S; } else { second = fminf(second, db); }
-            }
-            if (m < cnt) {
-                const float da = d2of(m);
-                if (da < best) { second = best; best = da; best_m = m; } else { second = fminf(second, da); }
-            }
-        }
-        for (int off = 1; off < S; off <<= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, best, off);
-            const float os = __shfl_xor_sync(0xffffffffu, second, off);
-            const int om = __shfl_xor_sync(0xffffffffu, best_m, off);
-            if (om >= 0 && (best_m < 0 || ob < best || (ob == best && om < best_m))) {
-                second = fminf(best, fminf(second, os));
-                best = ob;
-                best_m = om;
-            } else {
-                second = fminf(second, fminf(ob, os));
-            }
-            fro2 = fmaxf(fro2, __shfl_xor_sync(0xffffffffu, fro2, off));
-            mu2 = fmaxf(mu2, __shfl_xor_sync(0xffffffffu, mu2, off));
-        }
-        if (sub != 0 || !on) return;
-        const size_t ci = (size_t)(i0 + il) * n + hl;
-        if (rec && cnt > 0) anchor(ci, y0, y1, y2, best, second, best_m, fro2, mu2);
-        const int m_old = trial ? (int)cr[ci] : -1;
-        if (cnt > 0) {
-            ++w_pairs;
-            w_modes += cnt;
-            w_evals += cnt;
-            o.energy += sqrtf(best);
-            if (best_m >= 0) {
-                const float4 m0 = s_t0[base + best_m];
-                const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
-                if (fmaf(v0, v0, fmaf(v1, v1, v2 * v2)) <= thr2) {
-                    ++o.nin;
-                    ++w_in;
-                    if (cov) {
-                        const float4 m1 = s_t1[base + best_m];
-                        lm_accumulate(y0, y1, y2, v0, v1, v2, m0.w, m1.x, m1.y, m1.z, m1.w, s_t2[base + best_m],
-                                      o.acc);
-                    } else {
-                        lm_accumulate(y0, y1, y2, v0, v1, v2, 1.f, 0.f, 0.f, 1.f, 0.f, 1.f, o.acc);
+            // independent chains per step, compared in mode order
+            auto scan = [&](auto d2of) {
+                int m = sub;
+                if (SUBS > 1) {
+                    for (; m + 3 * S < cnt; m += 4 * S) {
+                        const float da = d2of(m), db = d2of(m + S), dc = d2of(m + 2 * S), dd = d2of(m + 3 * S);
+                        take(da, m);
+                        take(db, m + S);
+                        take(dc, m + 2 * S);
+                        take(dd, m + 3 * S);
                     }
-                } else {
-                    best_m = -1;
+                }
+                for (; m + S < cnt; m += 2 * S) {
+                    const float da = d2of(m), db = d2of(m + S);
+                    take(da, m);
+                    take(db, m + S);
+                }
+                if (m < cnt) take(d2of(m), m);
+            };
+            if (cov) scan(d2cov);
+            else scan(d2euc);
+            for (int off = 1; off < S; off <<= 1) {
+                const float ob = __shfl_xor_sync(0xffffffffu, best, off);
+                const float os = REC ? __shfl_xor_sync(0xffffffffu, second, off) : 0.f;
+                const int om = __shfl_xor_sync(0xffffffffu, best_m, off);
+                if (om >= 0 && (best_m < 0 || ob < best || (ob == best && om < best_m))) {
+                    if (REC) second = fminf(best, fminf(second, os));
+                    best = ob;
+                    best_m = om;
+                } else if (REC) {
+                    second = fminf(second, fminf(ob, os));
+                }
+                if (REC) {
+                    fro2 = fmaxf(fro2, __shfl_xor_sync(0xffffffffu, fro2, off));
+                    mu2 = fmaxf(mu2, __shfl_xor_sync(0xffffffffu, mu2, off));
                 }
             }
-            if (m_old >= 0) {  // the previous correspondence at the trial pose
-                ++w_trial;
-                const float4 m0 = s_t0[base + m_old];
-                const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
-                if (cov) {
-                    const float4 m1 = s_t1[base + m_old];
-                    const float q0 = fmaf(m0.w, v0, fmaf(m1.x, v1, m1.y * v2));
-                    const float q1 = fmaf(m1.z, v1, m1.w * v2);
-                    const float q2 = s_t2[base + m_old] * v2;
-                    o.trial = fmaf(q0, q0, fmaf(q1, q1, fmaf(q2, q2, o.trial)));
-                } else {
-                    o.trial = fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, o.trial)));
+            if (sub != 0 || !on) continue;
+            if (REC && cnt > 0) anchor(ci, y0, y1, y2, best, second, best_m, fro2, mu2);
+            if (cnt > 0) {
+                ++w_pairs;
+                w_modes += cnt;
+                w_evals += cnt;
+                o.energy += sqrtf(best);
+                if (best_m >= 0) {
+                    const float4 m0 = s_t0[base + best_m];
+                    const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
+                    if (fmaf(v0, v0, fmaf(v1, v1, v2 * v2)) <= thr2) {
+                        ++o.nin;
+                        ++w_in;
+                        if (cov) {
+                            const float4 m1 = s_t1[base + best_m];
+                            lm_accumulate(y0, y1, y2, v0, v1, v2, m0.w, m1.x, m1.y, m1.z, m1.w, s_t2[base + best_m],
+                                          o.acc);
+                        } else {
+                            lm_accumulate(y0, y1, y2, v0, v1, v2, 1.f, 0.f, 0.f, 1.f, 0.f, 1.f, o.acc);
+                        }
+                    } else {
+                        best_m = -1;
+                    }
                 }
+                if (m_old >= 0) {  // the previous correspondence at the trial pose
+                    ++w_trial;
+                    const float4 m0 = s_t0[base + m_old];
+                    const float v0 = y0 - m0.x, v1 = y1 - m0.y, v2 = y2 - m0.z;
+                    if (cov) {
+                        const float4 m1 = s_t1[base + m_old];
+                        const float q0 = fmaf(m0.w, v0, fmaf(m1.x, v1, m1.y * v2));
+                        const float q1 = fmaf(m1.z, v1, m1.w * v2);
+                        const float q2 = s_t2[base + m_old] * v2;
+                        o.trial = fmaf(q0, q0, fmaf(q1, q1, fmaf(q2, q2, o.trial)));
+                    } else {
+                        o.trial = fmaf(v0, v0, fmaf(v1, v1, fmaf(v2, v2, o.trial)));
+                    }
+                }
+            } else {
+                best_m = -1;
             }
-        } else {
-            best_m = -1;
+            cw[ci] = (int16_t)best_m;  // local mode index in the row, -1: none
         }
-        cw[ci] = (int16_t)best_m;  // local mode index in the row, -1: none
     };
     // The pass; act: this thread's hypothesis takes part, P: its pose;
     // first: the round's first pass.  Frames with at most LMC_DIRECT
@@ -619,10 +686,10 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
         __syncthreads();
         if (dir_ok && !first) {
             // rows from global memory; chunks of Gp * LMC_KP of the CTA's
-            // pixels (local pixel j is pixel j % 16 of tile crank + (j / 16) * CTAS)
+            // pixels (local pixel j is pixel j % 16 of tile crank + (j / 16) * RANKS)
             const int n_local = my_tiles * LMC_P;
             const int lane = t & 31;
-            auto pixel_of = [&](int j) { return (crank + (j / LMC_P) * CTAS) * LMC_P + j % LMC_P; };
+            auto pixel_of = [&](int j) { return (crank + (j / LMC_P) * RANKS) * LMC_P + j % LMC_P; };
             int c = 0;
             for (int c0 = 0; c0 < n_local; c0 += Gp * LMC_KP, c ^= 1) {
                 int pend[LMC_KP];
@@ -699,23 +766,28 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
             return o;
         }
         const bool rec = dir_ok && first;  // anchor every pair for the direct passes that follow
-        if (t == 0 && !*s_abort)
-            for (int j = 0; j < LMC_STAGES && j < my_tiles; ++j) issue(j, j);
+        if (t == 0)
+            for (int j = 0; j < STAGES && j < my_tiles && !*s_abort; ++j) issue(j);
         for (int j = 0; j < my_tiles; ++j) {
-            const int s = j % LMC_STAGES;
-            const uint32_t parity = waited[s] & 1u;
-            ++waited[s];
+            if (SUBS > 1) {  // the stage of the tile before, once every warp is done with it
+                if (t == 0 && j > 0 && j - 1 + STAGES < my_tiles && !*s_abort) issue(j - 1 + STAGES);
+                __syncwarp();
+            }
+            const uint32_t q = q_pass + (uint32_t)j;
+            const int s = (int)(q % STAGES);
             if (!*s_abort) {
-                if (mbar_wait_bounded(bar0 + 8 * s, parity, a.wait_limit)) {
-                    ++landed[s];
+                if (full_ok(q)) {
+                    q_landed = q + 1;
                 } else {
-                    *s_abort = 1;
-                    a.q.dev_err[b] = 1;
+                    give_up();
                 }
             }
-            if (S > 1) {
-                split_tile(act && !*s_abort, s, j, trial, rec, cr, cw, o, r00, r01, r02, tx, r10, r11, r12, ty, r20,
-                           r21, r22, tz);
+            if (rec) {
+                split_tile(std::true_type(), act && !*s_abort, s, j, trial, cr, cw, o, r00, r01, r02, tx, r10, r11,
+                           r12, ty, r20, r21, r22, tz);
+            } else if (SUBS > 1 || S > 1) {
+                split_tile(std::false_type(), act && !*s_abort, s, j, trial, cr, cw, o, r00, r01, r02, tx, r10, r11,
+                           r12, ty, r20, r21, r22, tz);
             } else if (act && !*s_abort) {
                 // one lane per pair: at least 16 hypotheses, so never a frame
                 // whose pairs need anchors (rec implies S > 1)
@@ -725,7 +797,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
                 const float *s_t2 = (const float *)(st + L.t2);
                 const float4 *s_xc = (const float4 *)(st + L.xc);
                 const int16_t *s_cnt = (const int16_t *)(st + L.cnt);
-                const int i0 = (crank + j * CTAS) * LMC_P;
+                const int i0 = (crank + j * RANKS) * LMC_P;
                 const int np = min(LMC_P, a.n_pix - i0);
                 for (int il = g; il < np; il += Gp) {
                     const size_t ci = (size_t)(i0 + il) * n + hl;
@@ -816,9 +888,16 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
                     cw[ci] = (int16_t)best_m;  // local mode index in the row, -1: none
                 }
             }
-            __syncthreads();  // stage s consumed by every thread
-            if (t == 0 && !*s_abort && j + LMC_STAGES < my_tiles) issue(j + LMC_STAGES, s);
+            if (SUBS > 1) {
+                __syncwarp();
+                if ((t & 31) == 0) mbar_arrive(bar0 + 8 * (STAGES + s));  // this warp is done with the stage
+            } else {
+                __syncthreads();  // stage s consumed by every thread
+                if (t == 0 && j + STAGES < my_tiles && !*s_abort) issue(j + STAGES);
+            }
         }
+        q_pass += (uint32_t)my_tiles;
+        if (SUBS > 1) __syncthreads();  // every tile consumed: the partial sums may overwrite them
         return o;
     };
     // Sums of this CTA's pass over groups (fixed order) into loc buffer lb,
@@ -832,21 +911,24 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
         mypart[30] = o.energy;
         __syncthreads();
         float *loc = s_loc + lb * (LMC_HMAX * LMC_NV);
-        for (int e = t; e < k_act * LMC_NV; e += LMC_THREADS) {
+        const int own = min(HQ, k_act - hset * HQ);  // this CTA's entries (none: <= 0)
+        for (int e = t; e < own * LMC_NV; e += LMC_THREADS) {
             const int j = e / LMC_NV, k = e % LMC_NV;
             float v = 0.f;
-            // the lanes holding list entry j's partials, in group order
-            for (int gg = 0; gg < Gp; ++gg) v += s_acc[(S * (gg * HB + j)) * LMC_PS + k];
-            loc[s_act[j] * LMC_NV + k] = v;
+            // the lanes holding entry j's partials, in group order
+#pragma unroll 4
+            for (int gg = 0; gg < Gp; ++gg) v += s_acc[(S * (gg * HQ + j)) * LMC_PS + k];
+            loc[s_act[hset * HQ + j] * LMC_NV + k] = v;
         }
         // Double-buffered loc: a CTA rewrites buffer lb two reductions later,
         // after the next barrier, which every CTA reaches only after reading
         // buffer lb here; one barrier per reduction suffices.
         cluster.sync();
         for (int e = t; e < k_act * LMC_NV; e += LMC_THREADS) {
-            const int h = s_act[e / LMC_NV], k = e % LMC_NV;
+            const int j = e / LMC_NV, h = s_act[j], k = e % LMC_NV, r0 = j / HQ * RANKS;
             float v = 0.f;
-            for (int r = 0; r < CTAS; ++r) v += cluster.map_shared_rank(loc, r)[h * LMC_NV + k];
+#pragma unroll
+            for (int r = 0; r < RANKS; ++r) v += cluster.map_shared_rank(loc, r0 + r)[h * LMC_NV + k];
             dst[h][k] = v;
         }
         __syncthreads();
@@ -913,7 +995,7 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
         __syncthreads();
     }
     __syncthreads();  // the last accept/reject updates of s_H before other threads write them out
-    if (crank == 0) {
+    if (cluster.block_rank() == 0) {
         for (int i = t; i < n * 12; i += LMC_THREADS)
             a.q.cur_pose[((size_t)b * NC + i / 12) * 12 + i % 12] = s_H[i / 12][i % 12];
         // Eq. 5 over the round's pixel set at each refined pose, from the pass
@@ -928,33 +1010,59 @@ __global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(LMC_THREADS, 2) k
         atomicAdd(&a.work[W_LM_EVALS], (unsigned long long)w_evals);
     }
     if (t == 0 && *s_abort)  // copies still in flight must land before the CTA exits
-        for (int s = 0; s < LMC_STAGES; ++s)
-            while (landed[s] < issued[s] && mbar_wait_bounded(bar0 + 8 * s, landed[s] & 1u)) ++landed[s];
+        while (q_landed < q_issued &&
+               mbar_wait_bounded(bar0 + 8 * (q_landed % STAGES), (q_landed / STAGES) & 1u))
+            ++q_landed;
     cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
-size_t lm_cluster_smem(int mpad, bool cov) { return lmc_layout(mpad, cov).total; }
+size_t lm_cluster_smem(int mpad, bool cov) { return lmc_layout(mpad, cov, LMC_STAGES).total; }
 
-rl_status launch_lm_cluster(const LmArgs &a, int n, cudaStream_t s) {
-    const size_t sm = lm_cluster_smem(a.p.mpad, a.p.use_cov);
-    const bool first = a.n_pix <= 2 * a.p.eta;  // round r refines on eta * (r + 2) pixels
-    if (first) {
-        k_lm_cluster<LMC_CTAS_FIRST><<<dim3(LMC_CTAS_FIRST, n), LMC_THREADS, sm, s>>>(a);
-    } else {
-        k_lm_cluster<LMC_CTAS_LATER><<<dim3(LMC_CTAS_LATER, n), LMC_THREADS, sm, s>>>(a);
-    }
+template <int RANKS, int SUBS>
+static rl_status launch_lm_shape(const LmArgs &a, int n, cudaStream_t s) {
+    const size_t sm = lmc_layout(a.p.mpad, a.p.use_cov, SUBS == 1 ? LMC_STAGES : LMC_STAGES_SUB).total;
+    k_lm_cluster<RANKS, SUBS><<<dim3(RANKS * SUBS, n), LMC_THREADS, sm, s>>>(a);
     RL_LAUNCH_CK();
     return RL_OK;
 }
 
-rl_status prepare_lm_cluster() {
-    RL_CK(cudaFuncSetAttribute(k_lm_cluster<LMC_CTAS_FIRST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+// The cluster of a round with RANKS CTAs on the pixels.  SUBS > 1 while the
+// call's CTAs fit the SMs that whole clusters of 8 or 16 can fill (16 of the
+// 19 of a GPC), one per SM, and rows are long enough: the lanes that share a
+// scan idle through the normal equations, so with up to 9 modes per pixel
+// SUBS = 4 was slower (8 frames 3.43 ms a call against 2.99).  Rows too long
+// for the deeper pipeline's shared memory keep SUBS = 1.
+template <int RANKS, int MOST>
+static rl_status launch_lm_ranks(const LmArgs &a, int n, cudaStream_t s) {
+    const int ctas = a.n_active * RANKS, room = a.sm_count / 19 * 16;
+    if (a.p.maxm >= LMC_SPLIT_MODES && lmc_layout(a.p.mpad, a.p.use_cov, LMC_STAGES_SUB).total <= kLmClusterSmemMax) {
+        if (ctas * MOST <= room) return launch_lm_shape<RANKS, MOST>(a, n, s);
+        if (ctas * 2 <= room) return launch_lm_shape<RANKS, 2>(a, n, s);
+    }
+    return launch_lm_shape<RANKS, 1>(a, n, s);
+}
+
+rl_status launch_lm_cluster(const LmArgs &a, int n, cudaStream_t s) {
+    // round r refines on eta * (r + 2) pixels
+    return a.n_pix <= 2 * a.p.eta ? launch_lm_ranks<LMC_RANKS_FIRST, 4>(a, n, s)
+                                  : launch_lm_ranks<LMC_RANKS_LATER, 2>(a, n, s);
+}
+
+template <int RANKS, int SUBS>
+static rl_status prepare_lm_shape() {
+    RL_CK(cudaFuncSetAttribute(k_lm_cluster<RANKS, SUBS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kLmClusterSmemMax));
-    RL_CK(cudaFuncSetAttribute(k_lm_cluster<LMC_CTAS_LATER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kLmClusterSmemMax));
-    if (LMC_CTAS_LATER > 8)  // clusters above 8 CTAs are not portable and must be allowed explicitly
-        RL_CK(cudaFuncSetAttribute(k_lm_cluster<LMC_CTAS_LATER>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (RANKS * SUBS > 8)  // clusters above 8 CTAs are not portable and must be allowed explicitly
+        RL_CK(cudaFuncSetAttribute(k_lm_cluster<RANKS, SUBS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return RL_OK;
+}
+
+rl_status prepare_lm_cluster() {
+    RL_TRY((prepare_lm_shape<LMC_RANKS_FIRST, 1>()));
+    RL_TRY((prepare_lm_shape<LMC_RANKS_FIRST, 2>()));
+    RL_TRY((prepare_lm_shape<LMC_RANKS_FIRST, 4>()));
+    RL_TRY((prepare_lm_shape<LMC_RANKS_LATER, 1>()));
+    return prepare_lm_shape<LMC_RANKS_LATER, 2>();
 }
 
 }  // namespace rl
