@@ -248,17 +248,38 @@ class Scene:
             self.h = ctypes.c_void_p()
 
 
+_RESULT = np.dtype(Result)  # rl_result as a NumPy record
+_SCALARS = ("energy", "energy_per_pixel", "score", "level", "n_hypotheses", "n_chosen", "n_pixels", "status", "best",
+            "icp_mask")
+
+
+def result_dicts(out, n: int) -> list:
+    """The first n records of `out` (rl_result array) as dictionaries.
+
+    Fields are converted for all frames at once; converting each record by
+    itself through ctypes took 16 us a frame (64 frames of 16 chosen poses:
+    1.0 ms, now 0.17)."""
+    a = np.frombuffer(out, _RESULT, count=n)
+    pose = a["pose"].reshape(n, 4, 4).copy()
+    scalars = [a[k].tolist() for k in _SCALARS]
+    chosen = {"chosen_pose": a["chosen_pose"].reshape(n, -1, 4, 4).copy(),
+              "chosen_energy": a["chosen_energy"].astype(np.float64),
+              "chosen_score": a["chosen_score"].astype(np.float64),
+              "chosen_slot": a["chosen_slot"].astype(np.int64)}
+    frac = a["chosen_icp_frac"].astype(np.float64)
+    results = []
+    for i in range(n):
+        d = dict(zip(_SCALARS, (v[i] for v in scalars)), pose=pose[i])
+        nc = max(0, d["n_chosen"])
+        for k, v in chosen.items():
+            d[k] = v[i, :nc] if nc else np.array([])
+        d["chosen_icp_frac"] = frac[i, :max(nc, 1)]
+        results.append(d)
+    return results
+
+
 def result_dict(r: Result) -> dict:
-    nc = max(0, r.n_chosen)
-    return dict(
-        pose=np.array(r.pose).reshape(4, 4), energy=r.energy, energy_per_pixel=r.energy_per_pixel,
-        score=r.score, level=r.level, n_hypotheses=r.n_hypotheses, n_chosen=r.n_chosen,
-        n_pixels=r.n_pixels, status=r.status, best=r.best,
-        chosen_pose=np.array([np.array(r.chosen_pose[i]).reshape(4, 4) for i in range(nc)]),
-        chosen_energy=np.array(r.chosen_energy[:nc]), chosen_score=np.array(r.chosen_score[:nc]),
-        chosen_slot=np.array(r.chosen_slot[:nc]), icp_mask=r.icp_mask,
-        chosen_icp_frac=np.array(r.chosen_icp_frac[:max(nc, 1)]),
-    )
+    return result_dicts(r, 1)[0]
 
 
 class Relocaliser:
@@ -280,7 +301,7 @@ class Relocaliser:
         out = (Result * n)()
         call("rl_relocalise_batch", self.h, n, d.ptr, c.ptr, ctypes.byref(intrinsics(K)),
              seeds.ctypes.data_as(ctypes.c_void_p), d.mem, _stream_ptr(stream), out)
-        return out if raw else [result_dict(out[i]) for i in range(n)]
+        return out if raw else result_dicts(out, n)
 
     def relocalise(self, depth, rgb, K, seed, stream=None):
         return self.relocalise_batch(depth, rgb, K, [seed], stream)[0]
@@ -301,7 +322,7 @@ class Relocaliser:
         n = self._pending
         out = (Result * n)()
         call("rl_reloc_fetch", self.h, n, _stream_ptr(stream), out)
-        return out if raw else [result_dict(out[i]) for i in range(n)]
+        return out if raw else result_dicts(out, n)
 
     @property
     def tuning(self) -> dict:
@@ -404,7 +425,7 @@ class Cascade:
         out = (Result * n)()
         call("rl_cascade_relocalise_batch", self.h, n, d.ptr, c.ptr, ctypes.byref(intrinsics(K)),
              seeds.ctypes.data_as(ctypes.c_void_p), d.mem, _stream_ptr(stream), out)
-        return [result_dict(out[i]) for i in range(n)]
+        return result_dicts(out, n)
 
     def close(self):
         if self.h:
