@@ -90,8 +90,7 @@ __device__ __forceinline__ int walk_tree(const float4 *__restrict__ nodes, int d
 
 // All T trees of one pixel walked level by level, interleaved: T
 // independent chains of dependent node and probe loads in flight at once.
-// PRE: the nodes' offsets are already multiplied by s (k_scale_nodes).
-template <int T, bool PRE>
+template <int T>
 __device__ __forceinline__ void walk_trees(const float4 *__restrict__ nodes, int n_branch, int depth,
                                            const float *__restrict__ D, const uint8_t *__restrict__ C,
                                            int W, int H, float s, int x, int y, float d, float inv,
@@ -107,8 +106,8 @@ __device__ __forceinline__ void walk_trees(const float4 *__restrict__ nodes, int
 #pragma unroll
         for (int t = 0; t < T; ++t) {
             const uint32_t meta = __float_as_uint(nd[t].w);
-            const float ox = __fmul_rn(PRE ? nd[t].x : __fmul_rn(nd[t].x, s), inv);
-            const float oy = __fmul_rn(PRE ? nd[t].y : __fmul_rn(nd[t].y, s), inv);
+            const float ox = __fmul_rn(__fmul_rn(nd[t].x, s), inv);
+            const float oy = __fmul_rn(__fmul_rn(nd[t].y, s), inv);
             const int q = probe_coord(y, oy, H) * W + probe_coord(x, ox, W);
             float f;
             if ((meta & 255u) == 0u) {
@@ -125,13 +124,13 @@ __device__ __forceinline__ void walk_trees(const float4 *__restrict__ nodes, int
     for (int t = 0; t < T; ++t) leaf[t] = n[t] - ((1 << depth) - 1);
 }
 
-template <int T, bool PRE>
+template <int T>
 __device__ __forceinline__ int walk_and_store(const float4 *nodes, int n_branch, int depth, const Frame &fr,
                                               float s, int x, int y, float d, float inv, uint16_t *o,
                                               int hw_max, const uint8_t *nmodes, int lpt, int k_top,
                                               bool count, uint4 *rec) {
     int leaf[kRecTrees], cnt[kRecTrees];
-    walk_trees<T, PRE>(nodes, n_branch, depth, fr.depth, fr.rgb, fr.W, fr.H, s, x, y, d, inv, leaf);
+    walk_trees<T>(nodes, n_branch, depth, fr.depth, fr.rgb, fr.W, fr.H, s, x, y, d, inv, leaf);
     int total = 0;
 #pragma unroll
     for (int t = 0; t < T; ++t) {
@@ -148,13 +147,10 @@ __device__ __forceinline__ int walk_and_store(const float4 *nodes, int n_branch,
 // When `mcount` is given it also receives |M(u)| = sum over the trees of
 // min(modes of the reached leaf, k_top) per pixel (0 without depth); the
 // pixel records `prec` (at most kRecTrees trees) hold the per-tree counts.
-// nodes_s: the nodes scaled for focal length fx_s (k_scale_nodes), used for
-// the frames of that focal length, or null.
 __global__ void k_leaves(const float4 *__restrict__ nodes, int n_branch, int depth, int n_trees,
                          const Frame *__restrict__ frames, int hw_max, uint16_t *__restrict__ out,
                          const uint8_t *__restrict__ nmodes, int leaves_per_tree, int k_top,
-                         uint16_t *__restrict__ mcount, uint4 *__restrict__ prec,
-                         const float4 *__restrict__ nodes_s, float fx_s) {
+                         uint16_t *__restrict__ mcount, uint4 *__restrict__ prec) {
     const Frame fr = frames[blockIdx.y];
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= fr.W * fr.H) return;
@@ -173,12 +169,9 @@ __global__ void k_leaves(const float4 *__restrict__ nodes, int n_branch, int dep
     const float inv = __frcp_rn(d);
     int total = 0;
     const bool cnt = mcount != nullptr || prec != nullptr;  // per-tree counts wanted
-    const bool pre = nodes_s != nullptr && fr.fx == fx_s;  // the same for the whole block (one frame)
-#define RL_WALK(T)                                                                                          \
-    total = pre ? walk_and_store<T, true>(nodes_s, n_branch, depth, fr, s, x, y, d, inv, o, hw_max, nmodes, \
-                                          leaves_per_tree, k_top, cnt, rec)                                  \
-                : walk_and_store<T, false>(nodes, n_branch, depth, fr, s, x, y, d, inv, o, hw_max, nmodes,  \
-                                           leaves_per_tree, k_top, cnt, rec)
+#define RL_WALK(T)                                                                                            \
+    total = walk_and_store<T>(nodes, n_branch, depth, fr, s, x, y, d, inv, o, hw_max, nmodes, leaves_per_tree, \
+                              k_top, cnt, rec)
     switch (n_trees) {
     case 1: RL_WALK(1); break;
     case 2: RL_WALK(2); break;
@@ -199,26 +192,143 @@ __global__ void k_leaves(const float4 *__restrict__ nodes, int n_branch, int dep
 
 rl_status launch_leaves(const rl_forest *f, const Frame *frames_dev, int n_frames, int n_trees,
                         int hw_max, uint16_t *out, int max_w, int max_h, cudaStream_t s,
-                        int k_top, uint16_t *mcount, uint4 *prec, int threads, const float4 *nodes_s,
-                        float fx_s) {
+                        int k_top, uint16_t *mcount, uint4 *prec, int threads) {
     const int npx = max_w * max_h;
     dim3 grid((npx + threads - 1) / threads, n_frames);
     k_leaves<<<grid, threads, 0, s>>>(f->nodes, f->n_branch, f->p.depth, n_trees, frames_dev, hw_max, out,
                                   f->nmodes, f->leaves_per_tree, k_top, mcount,
-                                  n_trees <= kRecTrees ? prec : nullptr, nodes_s, fx_s);
+                                  n_trees <= kRecTrees ? prec : nullptr);
     RL_LAUNCH_CK();
     return RL_OK;
 }
 
-// The split nodes with their offsets multiplied by s = fx / 585 (Eq. 1-3's
+// ---------------------------------------------------------------------------
+// The walk of a relocalisation call (at most kRecTrees trees, pixel records
+// out).  It is bound by issue: 75 node tests per pixel of exact FP32 feature
+// arithmetic whose gathers mostly hit L1.  Three things keep a test short:
+//  - frames are packed first, 8 bytes per pixel (depth, 0 where invalid; the
+//    three colours), so a probe is one gather whatever the split tests;
+//  - both kinds of split are evaluated without a branch (below the first
+//    levels a warp's lanes differ): a colour byte c becomes the float 2^23 +
+//    c by one byte permute, and the difference of two such floats is exactly
+//    the difference of the colours;
+//  - the call's nodes carry the offsets times fx / 585 and the permute's
+//    selector, and a coordinate is clamped by one min-with-relu.
+// That is 33 instructions a test instead of 44.  Measured on 8 frames of
+// 640x480, 5 trees of depth 15: 208 us + 11 us of packing (was 267; 75% issue,
+// the gathers' latency next), one frame 38 + 4 us (51).
+// ---------------------------------------------------------------------------
+constexpr uint32_t kSplitDepth = 0x80000000u;  // packed node: Depth split; else the permute selector
+constexpr uint32_t kSplitByte = 0x7540u;       // bytes c, 0x00, 0x00, 0x4B of (colours, 0x4B000000)
+
+__device__ __forceinline__ float4 pack_node(float4 v, float s) {
+    const uint32_t meta = __float_as_uint(v.w);
+    const uint32_t sel = (meta & 255u) == 0u ? kSplitDepth : kSplitByte | (meta >> 8);
+    return make_float4(__fmul_rn(v.x, s), __fmul_rn(v.y, s), v.z, __uint_as_float(sel));
+}
+
+// frame b's pixels at out + b * stride
+__global__ void __launch_bounds__(256) k_pack_frames(const Frame *__restrict__ frames, uint2 *__restrict__ out,
+                                                     size_t stride) {
+    const Frame fr = frames[blockIdx.y];
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= fr.W * fr.H) return;
+    const float d = fr.depth[p];
+    const uint8_t *c = fr.rgb + (size_t)p * 3;
+    out[blockIdx.y * stride + p] = make_uint2(__float_as_uint(d > 0.0f ? d : 0.0f),
+                                              (uint32_t)c[0] | ((uint32_t)c[1] << 8) | ((uint32_t)c[2] << 16));
+}
+
+// nodes: packed for focal length fx_s when PRE, else the forest's
+template <int T, bool PRE>
+__device__ __forceinline__ uint4 walk_packed(const float4 *__restrict__ nodes, int n_branch, int depth,
+                                             const uint2 *__restrict__ px, int W, int H, float s, int x, int y,
+                                             uint2 own, float inv, const uint8_t *__restrict__ nmodes, int lpt,
+                                             int k_top) {
+    int n[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) n[t] = 0;
+    const float d = __uint_as_float(own.x);
+    const float fx = (float)x, fy = (float)y;
+    for (int level = 0; level < depth; ++level) {
+        float4 nd[T];
+#pragma unroll
+        for (int t = 0; t < T; ++t) nd[t] = __ldg(&nodes[(size_t)t * n_branch + n[t]]);
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            if (!PRE) nd[t] = pack_node(nd[t], s);
+            const float vx = __fadd_rn(__fadd_rn(fx, __fmul_rn(nd[t].x, inv)), 0.5f);
+            const float vy = __fadd_rn(__fadd_rn(fy, __fmul_rn(nd[t].y, inv)), 0.5f);
+            const int qx = __vimin_s32_relu(__float2int_rd(vx), W - 1), qy = __vimin_s32_relu(__float2int_rd(vy), H - 1);
+            const uint2 w = __ldg(&px[qy * W + qx]);
+            const uint32_t sel = __float_as_uint(nd[t].w);
+            const float fd = __fsub_rn(d, __uint_as_float(w.x));
+            const float fc = __fsub_rn(__uint_as_float(__byte_perm(own.y, 0x4B000000u, sel)),
+                                       __uint_as_float(__byte_perm(w.y, 0x4B000000u, sel)));
+            n[t] = 2 * n[t] + (((int)sel < 0 ? fd : fc) >= nd[t].z ? 2 : 1);
+        }
+    }
+    int leaf[kRecTrees], cnt[kRecTrees];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        leaf[t] = n[t] - ((1 << depth) - 1);
+        cnt[t] = min((int)__ldg(&nmodes[t * lpt + leaf[t]]), k_top);
+    }
+    return make_rec(leaf, cnt, T);
+}
+
+template <int T>
+__global__ void k_leaves_packed(const float4 *__restrict__ nodes, const float4 *__restrict__ nodes_s, float fx_s,
+                                int n_branch, int depth, const Frame *__restrict__ frames, int hw_max,
+                                const uint2 *__restrict__ packed, size_t stride, const uint8_t *__restrict__ nmodes,
+                                int leaves_per_tree, int k_top, uint4 *__restrict__ prec) {
+    const Frame fr = frames[blockIdx.y];
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= fr.W * fr.H) return;
+    const uint2 *px = packed + blockIdx.y * stride;
+    const uint2 own = px[p];
+    const float d = __uint_as_float(own.x);
+    uint4 rec = make_uint4(0, 0, 0, 0);
+    if (d > 0.0f) {
+        const int x = p % fr.W, y = p / fr.W;
+        const float s = __fdiv_rn(fr.fx, 585.0f);
+        const float inv = __frcp_rn(d);
+        // the same for the whole block (one frame)
+        rec = fr.fx == fx_s ? walk_packed<T, true>(nodes_s, n_branch, depth, px, fr.W, fr.H, s, x, y, own, inv, nmodes,
+                                                   leaves_per_tree, k_top)
+                            : walk_packed<T, false>(nodes, n_branch, depth, px, fr.W, fr.H, s, x, y, own, inv, nmodes,
+                                                    leaves_per_tree, k_top);
+    }
+    prec[(size_t)blockIdx.y * hw_max + p] = rec;
+}
+
+rl_status launch_leaves_packed(const rl_forest *f, const Frame *frames_dev, int n_frames, int n_trees, int hw_max,
+                               cudaStream_t s, int k_top, uint4 *prec, int threads, const float4 *nodes_s, float fx_s,
+                               uint2 *packed, size_t stride) {
+    k_pack_frames<<<dim3((hw_max + 255) / 256, n_frames), 256, 0, s>>>(frames_dev, packed, stride);
+    RL_LAUNCH_CK();
+    const dim3 grid((hw_max + threads - 1) / threads, n_frames);
+#define RL_WALK(T)                                                                                                 \
+    k_leaves_packed<T><<<grid, threads, 0, s>>>(f->nodes, nodes_s, fx_s, f->n_branch, f->p.depth, frames_dev, hw_max, \
+                                                packed, stride, f->nmodes, f->leaves_per_tree, k_top, prec)
+    switch (n_trees) {
+    case 1: RL_WALK(1); break;
+    case 2: RL_WALK(2); break;
+    case 3: RL_WALK(3); break;
+    case 4: RL_WALK(4); break;
+    default: RL_WALK(5); break;
+    }
+#undef RL_WALK
+    RL_LAUNCH_CK();
+    return RL_OK;
+}
+
+// A call's split nodes: offsets multiplied by s = fx / 585 (Eq. 1-3's
 // depth-normalised probe offset), rounded as the walk rounds its own first
-// product: the walk then needs one product per coordinate.
+// product, and the split in the walk's form.
 __global__ void k_scale_nodes(const float4 *__restrict__ nodes, float4 *__restrict__ out, int count, float fx) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    const float s = __fdiv_rn(fx, 585.0f);
-    const float4 v = nodes[i];
-    out[i] = make_float4(__fmul_rn(v.x, s), __fmul_rn(v.y, s), v.z, v.w);
+    if (i < count) out[i] = pack_node(nodes[i], __fdiv_rn(fx, 585.0f));
 }
 
 rl_status launch_scale_nodes(const rl_forest *f, int n_trees, float4 *out, float fx, cudaStream_t s) {

@@ -178,7 +178,24 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
     // with pixel records (at most kRecTrees trees) every consumer reads the
     // leaves and |M(u)| from them, so neither the per-tree leaf map nor the
     // count map is written
-    { PROF(K_LEAVES); RL_TRY(launch_leaves(f, q.frames, n, p.n_trees, hw_max, q.prec ? nullptr : q.leaves, r->max_w, r->max_h, s, p.k_top, q.prec ? nullptr : q.mcount, q.prec, r->tune.leaves_threads, r->nodes_s, r->host_frames[0].fx)); }
+    {
+        PROF(K_LEAVES);
+        // packed frames go where nothing is live yet: the colour masks' array
+        // (written after the walk) or the leaf maps' (not written with records)
+        uint2 *packed = q.pcm;
+        size_t stride = hw_max;
+        if (!packed && (size_t)p.n_trees * hw_max * sizeof(uint16_t) % sizeof(uint2) == 0 &&
+            p.n_trees * sizeof(uint16_t) >= sizeof(uint2)) {
+            packed = (uint2 *)q.leaves;
+            stride = (size_t)p.n_trees * hw_max * sizeof(uint16_t) / sizeof(uint2);
+        }
+        if (q.prec && packed)
+            RL_TRY(launch_leaves_packed(f, q.frames, n, p.n_trees, hw_max, s, p.k_top, q.prec, r->tune.leaves_threads,
+                                        r->nodes_s, r->host_frames[0].fx, packed, stride));
+        else
+            RL_TRY(launch_leaves(f, q.frames, n, p.n_trees, hw_max, q.prec ? nullptr : q.leaves, r->max_w, r->max_h, s,
+                                 p.k_top, q.prec ? nullptr : q.mcount, q.prec, r->tune.leaves_threads));
+    }
     if (q.pcm) { PROF(K_CMASK); RL_TRY(launch_colour_mask(q.frames, q.mcount, q.prec, hw_max, mv, p, q.pcm, q.pbits, n, hw_max, s, r->tune.mask_threads)); }
     else if (q.pbits) { PROF(K_CMASK); RL_TRY(launch_mode_bits(q.frames, q.prec, hw_max, p.n_trees, q.pbits, n, s)); }
     { PROF(K_HYPGEN); RL_TRY(launch_hypgen(q.frames, q.leaves, q.mcount, q.prec, q.pcm, q.pbits, hw_max, mv, p, q.hyp_pose, q.hyp_iter, work, n, s, r->tune.hypgen_warps, n_active, r->forest->ctx->sm_count)); }
