@@ -630,19 +630,78 @@ __device__ __noinline__ bool ray_depth_fp64(const double *P, int u, int v, float
     return ok;
 }
 
+// One ray of a camera inside or outside the box against the general slab
+// test: *depth of the first face hit, false when there is none.  A decision
+// within a relative margin of 1e-4 of changing is taken in FP64 (n64 counts
+// them).
+__device__ __noinline__ bool ray_depth_slab(const RaycastArgs &a, const Frame &fr, const float *P, const double *P64,
+                                            float dc0, float dc1, int u, int v, float *depth, unsigned &n64) {
+    float d[3], o[3];
+    for (int r = 0; r < 3; ++r) {
+        d[r] = fmaf(P[4 * r], dc0, fmaf(P[4 * r + 1], dc1, P[4 * r + 2]));
+        o[r] = P[4 * r + 3];
+    }
+    const float dn = fabsf(d[0]) + fabsf(d[1]) + fabsf(d[2]);
+    float tn = -INFINITY, tf = INFINITY;
+    bool unsure = false;
+    for (int ax = 0; ax < 3; ++ax) {
+        if (fabsf(d[ax]) <= 1e-5f * dn) {
+            unsure = true;
+            continue;
+        }
+        const float inv = __fdividef(1.0f, d[ax]);
+        const float ta = (a.lo[ax] - o[ax]) * inv, tb = (a.hi[ax] - o[ax]) * inv;
+        tn = fmaxf(tn, fminf(ta, tb));
+        tf = fminf(tf, fmaxf(ta, tb));
+    }
+    if (!unsure) {
+        const float scale = fmaxf(fabsf(tn), fabsf(tf));
+        if (fabsf(tf - tn) <= 1e-4f * scale || fabsf(tn) <= 1e-4f * scale || fabsf(tf) <= 1e-4f * scale) unsure = true;
+    }
+    if (unsure) {
+        ++n64;
+        return ray_depth_fp64(P64, u, v, fr.fx, fr.fy, fr.cx, fr.cy, a.lo64, a.hi64, depth);
+    }
+    if (tn <= tf && tn > 0.f) {
+        *depth = tn;
+        return true;
+    }
+    if (tn <= tf && tf > 0.f) {
+        *depth = tf;
+        return true;
+    }
+    return false;
+}
+
 // Each thread owns RC_PIX pixels of an RC_TILE-pixel tile and runs all poses
 // of the frame over them in turn (poses staged in shared memory, RC_CHUNK at a
-// time), so each pixel's live depth and viewing direction are read once.  The
-// hit test runs in FP32; a ray whose decision lies within a relative margin
-// of 1e-4 of changing (near-parallel faces, grazing edges, a face through the
-// camera) is re-evaluated in FP64, so the valid mask of Eq. 7 is the FP64
-// one.  Per pose the tile's sums are reduced over the thread's pixels in
-// order, then over lanes, then over warps in order, one partial per (pose,
-// tile).
-constexpr int RC_CHUNK = 16;
+// time), so each pixel's live depth and viewing direction are read once.
+//
+// A camera more than 1 mm inside the box: every ray leaves the box exactly
+// once, at the nearest exit plane; with t_ax = (bound - o) / d, bound = hi
+// for d >= +0 and lo for d <= -0 (a zero component then gives +inf), the
+// depth is min_ax t_ax, a continuous function of the ray with no hit/miss
+// decision to certify.  The approximate reciprocal maps +-0 to +-inf.  Other
+// cameras take the slab test.
+//
+// Per pose the tile's sums are reduced over the thread's pixels in order,
+// then over lanes (l + l' at distance 16, 8, 4, 2, 1), then over warps in
+// order, one partial per (pose, tile).  While every pose of a chunk is inside
+// the box, four poses' sums are reduced over the lanes together, the first
+// two steps halving the poses a lane carries: 6 shuffles for 4 poses instead
+// of 20; the counts of rays and of live pixels are then the same for every
+// pose.  (All 16 poses of a chunk at once take fewer shuffles still, but
+// their straight-line code is fetched cold by every block of a call of few
+// frames: one frame's ranking 31 us instead of 27.)  What bounds it is issue
+// (78% of cycles) and the ALU.  Measured at 640x480: 128 poses of a frame 49
+// us (109 with the sums of one pose reduced at a time and rescaling
+// divisions), 16 poses of 8 frames 78 us (90 to 101), of one frame 27 (25).
+constexpr int RC_CHUNK = 16, RC_GROUP = 4;
+static_assert(RC_GROUP == 4 && RC_CHUNK % RC_GROUP == 0, "the lanes' pose index takes bits 4 and 3");
 
-__global__ void __launch_bounds__(256) k_raycast_score(RaycastArgs a) {
-    __shared__ float sPf[RC_CHUNK][12];
+__global__ void __launch_bounds__(256, 4) k_raycast_score(RaycastArgs a) {
+    __shared__ __align__(16) float sPf[RC_CHUNK][12];
+    __shared__ __align__(16) float s_exit[RC_CHUNK][8];  // lo - o, hi - o per axis (x, y, z, -)
     __shared__ float s_sum[RC_CHUNK][8];
     __shared__ int s_syn[RC_CHUNK][8], s_both[RC_CHUNK][8];
     const int b = blockIdx.y;
@@ -670,102 +729,110 @@ __global__ void __launch_bounds__(256) k_raycast_score(RaycastArgs a) {
         }
     }
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int n_in = 0, n_live = 0;  // this thread's pixels, and those with depth
+#pragma unroll
+    for (int q = 0; q < RC_PIX; ++q) {
+        n_in += in[q];
+        n_live += in[q] && dl[q] > 0.f;
+    }
+    const int w_in = __reduce_add_sync(0xffffffffu, n_in), w_live = __reduce_add_sync(0xffffffffu, n_live);
     unsigned n64 = 0;  // rays re-evaluated in FP64 (profiling counter)
     for (int c0 = 0; c0 < n_poses; c0 += RC_CHUNK) {
         const int cnt = min(RC_CHUNK, n_poses - c0);
         __syncthreads();  // the previous chunk's poses and partials are consumed
-        for (int e = threadIdx.x; e < cnt * 12; e += blockDim.x) sPf[e / 12][e % 12] = (float)a.pose_of(b, c0 + e / 12)[e % 12];
+        // poses past the last repeat it; their sums are dropped
+        for (int e = threadIdx.x; e < RC_CHUNK * 12; e += blockDim.x)
+            sPf[e / 12][e % 12] = (float)a.pose_of(b, c0 + min(e / 12, cnt - 1))[e % 12];
         __syncthreads();
-        for (int k = 0; k < cnt; ++k) {
-            const float *P = sPf[k];
-            float sum = 0.f;
-            int syn = 0, both = 0;
-            // A camera more than 1 mm inside the box: every ray leaves the
-            // box exactly once, at the nearest exit plane; with t_ax = (bound
-            // - o) / d, bound = hi for d >= +0 and lo for d <= -0 (a zero
-            // component then gives +inf), the depth is min_ax t_ax, a
-            // continuous function of the ray with no hit/miss decision to
-            // certify.  Same value as the slab test below up to FP32 rounding.
-            // The approximate reciprocal (within 2 ulp) maps +-0 to +-inf.
-            const float ox = P[3], oy = P[7], oz = P[11];
-            const bool inside = ox - a.lo[0] > 1e-3f && a.hi[0] - ox > 1e-3f && oy - a.lo[1] > 1e-3f &&
-                                a.hi[1] - oy > 1e-3f && oz - a.lo[2] > 1e-3f && a.hi[2] - oz > 1e-3f;
-            if (inside) {
-                const float lx = a.lo[0] - ox, hx = a.hi[0] - ox, ly = a.lo[1] - oy, hy = a.hi[1] - oy;
-                const float lz = a.lo[2] - oz, hz = a.hi[2] - oz;
+        bool inside = true;
+        if (threadIdx.x < RC_CHUNK) {
+            const float *P = sPf[threadIdx.x];
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) {
+                const float o = P[4 * ax + 3];
+                inside = inside && o - a.lo[ax] > 1e-3f && a.hi[ax] - o > 1e-3f;
+                s_exit[threadIdx.x][ax] = a.lo[ax] - o;
+                s_exit[threadIdx.x][4 + ax] = a.hi[ax] - o;
+            }
+        }
+        if (__syncthreads_and(inside)) {
+#pragma unroll 1
+            for (int g = 0; g < cnt; g += RC_GROUP) {
+                float sum[RC_GROUP];
+#pragma unroll
+                for (int k = 0; k < RC_GROUP; ++k) {
+                    const float4 P0 = *(const float4 *)&sPf[g + k][0], P1 = *(const float4 *)&sPf[g + k][4],
+                                 P2 = *(const float4 *)&sPf[g + k][8];
+                    const float4 lo = *(const float4 *)&s_exit[g + k][0], hi = *(const float4 *)&s_exit[g + k][4];
+                    sum[k] = 0.f;
+#pragma unroll
+                    for (int q = 0; q < RC_PIX; ++q) {
+                        const float d0 = fmaf(P0.x, dc0[q], fmaf(P0.y, dc1[q], P0.z));
+                        const float d1 = fmaf(P1.x, dc0[q], fmaf(P1.y, dc1[q], P1.z));
+                        const float d2 = fmaf(P2.x, dc0[q], fmaf(P2.y, dc1[q], P2.z));
+                        const float t0 = (signbit(d0) ? lo.x : hi.x) * rcp_approx(d0);
+                        const float t1 = (signbit(d1) ? lo.y : hi.y) * rcp_approx(d1);
+                        const float t2 = (signbit(d2) ? lo.z : hi.z) * rcp_approx(d2);
+                        const float depth = fminf(t0, fminf(t1, t2));
+                        if (dl[q] > 0.f) sum[k] += fabsf(dl[q] - depth);  // no pixel: dl = 0
+                    }
+                }
+                // lanes with bit 16 (then 8) set carry the upper half of the poses on
+#pragma unroll
+                for (int o = 16, h = RC_GROUP / 2; h > 0; o >>= 1, h >>= 1)
+#pragma unroll
+                    for (int k = 0; k < h; ++k) {
+                        const bool up = lane & o;
+                        const float x = __shfl_xor_sync(0xffffffffu, up ? sum[k] : sum[k + h], o);
+                        sum[k] = (up ? sum[k + h] : sum[k]) + x;
+                    }
+#pragma unroll
+                for (int o = 16 / RC_GROUP; o > 0; o >>= 1) sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], o);
+                if ((lane & (32 / RC_GROUP - 1)) == 0) {
+                    const int k = g + (lane >> 4 & 1) * 2 + (lane >> 3 & 1);
+                    s_sum[k][w] = sum[0];
+                    s_syn[k][w] = w_in;
+                    s_both[k][w] = w_live;
+                }
+            }
+        } else {
+            for (int k = 0; k < cnt; ++k) {
+                const float *P = sPf[k];
+                float sum = 0.f;
+                int syn = 0, both = 0;
+                const float *E = s_exit[k];
+                const bool in_box = E[0] < -1e-3f && E[4] > 1e-3f && E[1] < -1e-3f && E[5] > 1e-3f && E[2] < -1e-3f &&
+                                    E[6] > 1e-3f;
 #pragma unroll
                 for (int q = 0; q < RC_PIX; ++q) {
                     if (!in[q]) continue;
-                    const float d0 = fmaf(P[0], dc0[q], fmaf(P[1], dc1[q], P[2]));
-                    const float d1 = fmaf(P[4], dc0[q], fmaf(P[5], dc1[q], P[6]));
-                    const float d2 = fmaf(P[8], dc0[q], fmaf(P[9], dc1[q], P[10]));
-                    const float t0 = (signbit(d0) ? lx : hx) * __fdividef(1.0f, d0);
-                    const float t1 = (signbit(d1) ? ly : hy) * __fdividef(1.0f, d1);
-                    const float t2 = (signbit(d2) ? lz : hz) * __fdividef(1.0f, d2);
-                    const float depth = fminf(t0, fminf(t1, t2));
-                    ++syn;
-                    if (dl[q] > 0.f) {
-                        ++both;
-                        sum += fabsf(dl[q] - depth);
-                    }
-                }
-            } else {
-#pragma unroll
-            for (int q = 0; q < RC_PIX; ++q) {
-                if (!in[q]) continue;
-                float d[3], o[3];
-                for (int r = 0; r < 3; ++r) {
-                    d[r] = fmaf(P[4 * r], dc0[q], fmaf(P[4 * r + 1], dc1[q], P[4 * r + 2]));
-                    o[r] = P[4 * r + 3];
-                }
-                const float dn = fabsf(d[0]) + fabsf(d[1]) + fabsf(d[2]);
-                float tn = -INFINITY, tf = INFINITY;
-                bool ok = true, unsure = false;
-                for (int ax = 0; ax < 3; ++ax) {
-                    if (fabsf(d[ax]) <= 1e-5f * dn) {
-                        unsure = true;
+                    float depth = 0.f;
+                    if (in_box) {
+                        const float d0 = fmaf(P[0], dc0[q], fmaf(P[1], dc1[q], P[2]));
+                        const float d1 = fmaf(P[4], dc0[q], fmaf(P[5], dc1[q], P[6]));
+                        const float d2 = fmaf(P[8], dc0[q], fmaf(P[9], dc1[q], P[10]));
+                        const float t0 = (signbit(d0) ? E[0] : E[4]) * rcp_approx(d0);
+                        const float t1 = (signbit(d1) ? E[1] : E[5]) * rcp_approx(d1);
+                        const float t2 = (signbit(d2) ? E[2] : E[6]) * rcp_approx(d2);
+                        depth = fminf(t0, fminf(t1, t2));
+                    } else if (!ray_depth_slab(a, fr, P, a.pose_of(b, c0 + k), dc0[q], dc1[q], u[q], v[q], &depth, n64)) {
                         continue;
                     }
-                    const float inv = __fdividef(1.0f, d[ax]);
-                    const float ta = (a.lo[ax] - o[ax]) * inv, tb = (a.hi[ax] - o[ax]) * inv;
-                    tn = fmaxf(tn, fminf(ta, tb));
-                    tf = fminf(tf, fmaxf(ta, tb));
-                }
-                float depth = 0.f;
-                if (!unsure) {
-                    const float scale = fmaxf(fabsf(tn), fabsf(tf));
-                    if (fabsf(tf - tn) <= 1e-4f * scale || fabsf(tn) <= 1e-4f * scale ||
-                        fabsf(tf) <= 1e-4f * scale)
-                        unsure = true;
-                }
-                if (unsure) {
-                    ++n64;
-                    ok = ray_depth_fp64(a.pose_of(b, c0 + k), u[q], v[q], fr.fx, fr.fy, fr.cx, fr.cy, a.lo64,
-                                        a.hi64, &depth);
-                } else if (tn <= tf && tn > 0.f) {
-                    depth = tn;
-                } else if (tn <= tf && tf > 0.f) {
-                    depth = tf;
-                } else {
-                    ok = false;
-                }
-                if (ok) {
                     ++syn;
                     if (dl[q] > 0.f) {
                         ++both;
                         sum += fabsf(dl[q] - depth);
                     }
                 }
-            }
-            }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-            syn = __reduce_add_sync(0xffffffffu, syn);
-            both = __reduce_add_sync(0xffffffffu, both);
-            if (lane == 0) {
-                s_sum[k][w] = sum;
-                s_syn[k][w] = syn;
-                s_both[k][w] = both;
+                for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+                syn = __reduce_add_sync(0xffffffffu, syn);
+                both = __reduce_add_sync(0xffffffffu, both);
+                if (lane == 0) {
+                    s_sum[k][w] = sum;
+                    s_syn[k][w] = syn;
+                    s_both[k][w] = both;
+                }
             }
         }
         __syncthreads();
