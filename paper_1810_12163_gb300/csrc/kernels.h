@@ -28,6 +28,8 @@ struct EnergyArgs {
     const float4 *q_tab1;
     const float *q_tab2;
     const int16_t *q_tab_cnt;
+    int n_active;              // frames at work on the GPU at once (shapes the launch, never the result)
+    int sm_count;
 };
 
 // Pixel batches of all rounds and their mode table (decoded M(u) of each drawn pixel).

@@ -224,6 +224,8 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
     ea.part = q.energy_part;
     ea.part_h = std::max(N, NC);
     ea.n_chunks = r->n_chunks;
+    ea.n_active = n_active;
+    ea.sm_count = f->ctx->sm_count;
     // initial cull on I_0
     ea.pose = q.hyp_pose;
     ea.pose_stride = N;
