@@ -113,6 +113,8 @@ struct IcpArgs {
     float lo[3], hi[3];
     IcpParams ip;
     unsigned long long *work;  // profiling counters or null
+    int n_active;              // frames at work on the GPU at once (shapes the launch, never the result)
+    int sm_count;
 };
 rl_status launch_icp(const IcpArgs &a, int n, cudaStream_t s);
 

@@ -299,6 +299,8 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
         }
         ia.ip = p.icp_p;
         ia.work = work;
+        ia.n_active = n_active;
+        ia.sm_count = f->ctx->sm_count;
         PROF(K_ICP);
         RL_TRY(launch_icp(ia, n, s));
     }
@@ -1382,6 +1384,8 @@ extern "C" rl_status rl_icp_poses(rl_scene *sc, const float *depth, const rl_int
             ia.hi[a] = (float)sc->hi[a];
         }
         ia.ip = icp_device_params(*ip);
+        ia.n_active = 1;
+        ia.sm_count = ctx->sm_count;
         st = launch_icp(ia, 1, s);
     }
     if (st == RL_OK && (cudaMemcpyAsync(p12.data(), pd, p12.size() * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
