@@ -17,7 +17,9 @@
 //    summed in groups of 8 whose sums are Kahan-added, then over at most 32
 //    lanes: within 14 u.  With x = -ln t the exact exponents,
 //    |rho32 - rho64| <= 8 u sum(t x) + (14 u + 2^-22) rho, and sum(t x) <=
-//    rho ln(n / rho) (the entropy bound, equality when all terms are equal);
+//    rho ln(n / rho) (the entropy bound, equality when all terms are equal).
+//    Terms below 2^-40 are left out where whole tiles of points are that far
+//    apart; they add at most n 2^-40;
 //  - a comparison matters only between points within tau_c, and for point i
 //    only if no point known to be denser is nearer; points at the same place
 //    have the same density by definition.  The few points left get an FP64
@@ -26,25 +28,34 @@
 // Cluster statistics and the covariance factor are FP64, members in index
 // order, so the modes are identical to the FP64 definition's.
 //
-// Work split: one block per leaf.  S adjacent lanes share a point's row (S a
-// power of two, as many as fit); with more rows than threads a thread takes
-// two at a time, so that one shared-memory read serves two pairs.  The pairs
-// within tau_c are collected as bit masks of 32 columns per lane first and
-// compared afterwards: with a tenth of the columns near, nearly every warp
-// would otherwise take the comparison branch on every column.  What bounds a
-// full leaf (1024 points, about 0.2 ms on its SM): FP32 issue of the two pair
-// loops (12 and 14 instructions a pair) and the FP64 sums of its clusters,
-// which are serial by definition; those run one warp per cluster, 32 members'
-// products computed by the lanes at once and the running sums on a lane each,
-// so that a member costs two dependent FP64 additions instead of 27 FP64
-// instructions of a warp.  A cluster of four blocks on each full leaf was
-// slower (2.2 against 1.5 ms at that stage): the full leaves fill the GPU.
+// Work split: one block per leaf.  The points are sorted along a Morton curve;
+// a warp takes 32 of them as rows, a lane each, and the groups of 8 columns
+// whose boxes are near enough to matter (0.74 m at sigma = 0.1 m for the
+// densities, tau_c for the parents): in a full leaf most are not.  A row's
+// own groups come first, so that its parent is soon found and columns farther
+// off or surely less dense are passed over by two comparisons; the others are
+// noted as a bit mask first and compared afterwards, since with one column in
+// ten near nearly every warp would otherwise take the comparison branch on
+// every column.  The clusters' FP64 sums run eight lanes a cluster, the four
+// clusters of a warp sharing its FP64 instructions.  The means are exact sums
+// wherever the values' bits span at most 53, and then any order will do;
+// otherwise, and for the covariances, the sums are serial by definition: the
+// lanes compute eight members' products at once, then carry a running sum
+// each (a warp per cluster took three FP64 instructions a member, a thread
+// per cluster 27).
+// Of 297 thousand cycles of a full leaf of 1024 points with the columns in
+// tiles of 32, the sort took 24, densities 44, parents 77, FP64 densities 54,
+// comparisons in FP64 29 and the sums 43 (training; 21, 52, 134, 20, 10 and
+// 93 online, where clusters are larger).  A cluster of four blocks on each
+// full leaf was slower: the full leaves fill the GPU.
 //
-// Measured on GB300: 10,240 leaves of 107 points on average, about 1,200 of
-// them full (24 frames of 640x480, 5 trees of depth 11, capacity 1024): 1.17
-// ms, 13.7 ms with FP64 densities on single lanes and one thread per
-// cluster's sums.  2,048 leaves of an online update, some 60 full: 0.29 ms,
-// 5.4 ms before.
+// Measured on GB300: 10,240 leaves of 107 points on average, about 800 of
+// more than 600 (24 frames of 640x480, 5 trees of depth 11, capacity 1024):
+// 0.67 ms; 1.17 ms with every pair of points looked at, 13.7 ms with FP64
+// densities on single lanes and one thread per cluster's sums.  2,048 leaves
+// of an online update, some 35 of more than 600 points: 0.20 ms, 0.29 ms and
+// 5.4 ms before; the largest leaf's serial parts bound that.  1,024 threads a
+// block: 1.05 and 0.20 ms.
 #include <type_traits>
 
 #include "internal.h"
@@ -104,49 +115,81 @@ __device__ __forceinline__ float ex2_approx(float x) {
 constexpr int RQS_THREADS = 512;
 constexpr int RQS_STAT_WARPS = 8;       // warps of the FP64 sums (four sub-partitions, two each)
 constexpr int RQS_BUF = 6 * 33;         // FP64 values per such warp: six rows of 32, odd stride
+constexpr int RQS_GROUP = 8;            // columns with a box of their own
 
-// Parzen rows of PP points p over the columns sub, sub + S, ...
-template <int PP>
-__device__ __forceinline__ void rqs_density(const float4 *pts, int n, float c2, const float4 (&p)[PP], int sub, int S,
-                                            float (&rho)[PP]) {
-    float comp[PP];
+// Squared distance between two boxes (0 if they meet), a little
+// below the exact value.
+__device__ __forceinline__ float box_gap2(const float4 alo, const float4 ahi, const float4 blo, const float4 bhi) {
+    const float x = fmaxf(0.f, fmaxf(blo.x - ahi.x, alo.x - bhi.x));
+    const float y = fmaxf(0.f, fmaxf(blo.y - ahi.y, alo.y - bhi.y));
+    const float z = fmaxf(0.f, fmaxf(blo.z - ahi.z, alo.z - bhi.z));
+    return fmaf(z, z, fmaf(y, y, x * x)) * 0.9999f;
+}
+
+// Morton code of 7 + 7 + 6 bits.
+__device__ __forceinline__ uint32_t morton20(uint32_t x, uint32_t y, uint32_t z) {
+    uint32_t m = 0;
 #pragma unroll
-    for (int k = 0; k < PP; ++k) rho[k] = comp[k] = 0.f;
-    auto add = [&](const float (&part)[PP]) {  // Kahan sum of the groups
-#pragma unroll
-        for (int k = 0; k < PP; ++k) {
-            const float y = part[k] - comp[k];
-            const float t = rho[k] + y;
-            comp[k] = (t - rho[k]) - y;
-            rho[k] = t;
-        }
-    };
-    int j = sub;
-    for (; j + 7 * S < n; j += 8 * S) {
-        float part[PP];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const float4 q = pts[j + u * S];
-#pragma unroll
-            for (int k = 0; k < PP; ++k) {
-                const float t = ex2_approx(dist2f(p[k], q) * c2);
-                part[k] = u == 0 ? t : part[k] + t;
-            }
-        }
-        add(part);
+    for (int b = 0; b < 7; ++b) {
+        m |= (x >> b & 1u) << (3 * b + 1);
+        m |= (y >> b & 1u) << (3 * b);
+        if (b < 6) m |= (z >> b & 1u) << (3 * b + 2);
     }
-    if (j < n) {
-        float part[PP];
-#pragma unroll
-        for (int k = 0; k < PP; ++k) part[k] = 0.f;
-        for (; j < n; j += S) {
-            const float4 q = pts[j];
-#pragma unroll
-            for (int k = 0; k < PP; ++k) part[k] += ex2_approx(dist2f(p[k], q) * c2);
+    return m;
+}
+
+// Calls f(g) for the column groups of row tile `mine`, then for every other
+// group whose box is within `cut` (squared) of the tile's; every lane of the
+// warp together.
+template <class F>
+__device__ __forceinline__ void near_groups(const float4 *box, int groups, int mine, float cut, F f) {
+    constexpr int PER = 32 / RQS_GROUP;
+    const int lane = threadIdx.x & 31, g0 = PER * mine, g1 = min(g0 + PER, groups);
+    float4 lo = box[2 * g0], hi = box[2 * g0 + 1];
+    for (int g = g0 + 1; g < g1; ++g) {
+        const float4 l = box[2 * g], h = box[2 * g + 1];
+        lo = make_float4(fminf(lo.x, l.x), fminf(lo.y, l.y), fminf(lo.z, l.z), 0.f);
+        hi = make_float4(fmaxf(hi.x, h.x), fmaxf(hi.y, h.y), fmaxf(hi.z, h.z), 0.f);
+    }
+    for (int t0 = -32; t0 < groups; t0 += 32) {
+        unsigned m;
+        if (t0 < 0) {
+            m = (1u << (g1 - g0)) - 1u;
+        } else {
+            const int g = t0 + lane, gc = min(g, groups - 1);
+            m = __ballot_sync(0xffffffffu, g < groups && (g < g0 || g >= g1) &&
+                                               !(box_gap2(lo, hi, box[2 * gc], box[2 * gc + 1]) > cut));
         }
-        add(part);
+        for (const int base = t0 < 0 ? g0 : t0; m; m &= m - 1) f(base + __ffs(m) - 1);
     }
 }
+
+// (double)x by its bits: conversions take the FP64 pipe.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x);
+    if ((b >> 23 & 255u) - 1u < 254u)
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+    return (double)x;  // zero, subnormal, not finite
+}
+
+// Exponents of the values other than zero of a sum.
+struct Span {
+    int lo = 255, hi = 0;
+    __device__ void add(float x) {
+        const uint32_t b = __float_as_uint(x) & 0x7fffffffu;
+        const int e = max((int)(b >> 23), 1);
+        if (b) {
+            lo = min(lo, e);
+            hi = max(hi, e);
+        }
+    }
+    __device__ void join(int o) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    // all partial sums of n of them are multiples of 2^(lo - 150) below n 2^(hi - 126)
+    __device__ bool exact(int n) const { return hi - lo + (32 - __clz(n)) <= 29; }
+};
 
 // Shared state of the parent search.
 struct RqsPar {
@@ -217,81 +260,54 @@ __device__ __forceinline__ void rqs_candidate(const RqsPar &r, const float4 p, i
     }
 }
 
-// Parents of PP points (i[k] < 0: none) over the columns sub, sub + S, ...
-template <int PP, int LEVEL>
-__device__ __forceinline__ void rqs_parents(const RqsPar &r, const float4 (&p)[PP], const int (&i)[PP], int sub, int S,
-                                            RqsBest (&o)[PP]) {
-    float ri[PP], ei[PP];
+// A point's search by a warp, lane by lane of the columns in index order.
+template <int LEVEL>
+__device__ __forceinline__ void rqs_row(const RqsPar &r, int i, RqsBest &o) {
+    const int lane = threadIdx.x & 31;
+    const float4 p = r.pts[i];
+    const float ri = r.rho[i], ei = r.err[i];
+    if (LEVEL != RQS_MARK) o = {-1, 0.f, INFINITY};
+    for (int j = lane; j < r.n; j += 32)
+        if (j != i && !(dist2f(p, r.pts[j]) > r.tau_hi)) rqs_candidate<LEVEL>(r, p, i, ri, ei, j, o);
+    if (LEVEL == RQS_MARK) return;
 #pragma unroll
-    for (int k = 0; k < PP; ++k) {
-        if (LEVEL != RQS_MARK) o[k] = {-1, 0.f, INFINITY};
-        ri[k] = i[k] >= 0 ? r.rho[i[k]] : 0.f;
-        ei[k] = i[k] >= 0 ? r.err[i[k]] : 0.f;
-    }
-    for (int j0 = sub; j0 < r.n; j0 += 32 * S) {
-        uint32_t near[PP];
-#pragma unroll
-        for (int k = 0; k < PP; ++k) near[k] = 0;
-        if (j0 + 31 * S < r.n) {
-#pragma unroll
-            for (int u = 0; u < 32; ++u) {
-                const float4 q = r.pts[j0 + u * S];
-#pragma unroll
-                for (int k = 0; k < PP; ++k)
-                    if (!(dist2f(p[k], q) > r.tau_hi)) near[k] |= 1u << u;
-            }
-        } else {
-            for (int u = 0; j0 + u * S < r.n; ++u) {
-                const float4 q = r.pts[j0 + u * S];
-#pragma unroll
-                for (int k = 0; k < PP; ++k)
-                    if (!(dist2f(p[k], q) > r.tau_hi)) near[k] |= 1u << u;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < PP; ++k) {
-            uint32_t m = i[k] >= 0 ? near[k] : 0u;
-            while (m) {
-                const int j = j0 + (__ffs(m) - 1) * S;
-                m &= m - 1;
-                if (j != i[k]) rqs_candidate<LEVEL>(r, p[k], i[k], ri[k], ei[k], j, o[k]);
-            }
-        }
-    }
-}
-
-// Merges the candidates of the S lanes of a point.
-__device__ __forceinline__ void rqs_merge(const float4 *pts, const float4 p, int S, RqsBest &o) {
-    for (int off = 1; off < S; off <<= 1) {
+    for (int off = 1; off < 32; off <<= 1) {
         const int oj = __shfl_xor_sync(0xffffffffu, o.j, off);
         const float od = __shfl_xor_sync(0xffffffffu, o.d2, off);
-        o.und = fminf(o.und, __shfl_xor_sync(0xffffffffu, o.und, off));
-        if (oj >= 0 && rqs_nearer(pts, p, oj, od, o.j, o.d2)) {
+        if (oj >= 0 && rqs_nearer(r.pts, p, oj, od, o.j, o.d2)) {
             o.j = oj;
             o.d2 = od;
         }
     }
 }
 
-// Dynamic shared memory, per point: float4 pts, double rho64 (later the two
-// int lists of the clusters), float rho and err, int parent, root, csize,
-// need; then the FP64 buffers.
+// Dynamic shared memory, per point: float4 pts, 16 bytes that hold the sorted
+// copy spts (x, y, z, an upper bound of the density) and later double rho64
+// (then the two int lists of the clusters), int root and csize; float rho and
+// err (first the sort keys), int parent and need; two float4 box per group of
+// columns; then the FP64 buffers.
 __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
-    const int K = a.kappa + (a.kappa & 1);
+    const int K = (a.kappa + 31) & ~31;
     float4 *pts = (float4 *)smem;
-    double *rho64 = (double *)(pts + K);
-    float *rho = (float *)(rho64 + K);
-    float *err = rho + K;
-    int *parent = (int *)(err + K);
-    int *root = parent + K;
+    float4 *spts = pts + K;
+    double *rho64 = (double *)spts;
+    int *root = (int *)(rho64 + K);
     int *csize = root + K;
-    int *need = csize + K;
-    double *bufs = (double *)(need + K);  // [RQS_STAT_WARPS][RQS_BUF]
+    float *rho = (float *)(spts + K);
+    float *err = rho + K;
+    uint32_t *keys = (uint32_t *)rho;     // [2 K]
+    int *parent = (int *)(err + K);
+    int *need = parent + K;
+    float4 *box = (float4 *)(need + K);   // [K / RQS_GROUP][2]
+    double *bufs = (double *)(box + K / RQS_GROUP * 2);  // [RQS_STAT_WARPS][RQS_BUF]
+    // until the parents are known: index of the sorted point k in the low half of need[k]
+    uint16_t *sorted = (uint16_t *)need;
+    uint8_t *open = (uint8_t *)need;      // [4 i + 3]: point i's parent is not decided
     // after the parents are known
     int *qual = (int *)rho64;             // [K] roots of the clusters large enough
     int *order = qual + K;                // [K] members of the kept clusters, by cluster
-    __shared__ int n_qual, n_list, any;
+    __shared__ int n_qual, n_list, n_near, any;
     __shared__ int cl_root[64], cl_start[65];
     __shared__ double mu[64][3], cov[64][6];
     __shared__ float cen[3];
@@ -303,120 +319,225 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
     // fewer points than the smallest cluster: no modes
     const int n = cnt < (uint32_t)a.min_cluster_size ? 0 : (cnt < (uint32_t)a.kappa ? (int)cnt : a.kappa);
 
+    float3 mn = make_float3(INFINITY, INFINITY, INFINITY), mx = make_float3(-INFINITY, -INFINITY, -INFINITY);
+    bool finite = true;
     for (int i = tid; i < n; i += NT) {
-        pts[i] = a.res[(size_t)L * a.kappa + i];
-        csize[i] = 0;
-        need[i] = 0;
-        rho64[i] = 0.0;
+        const float4 p = a.res[(size_t)L * a.kappa + i];
+        pts[i] = p;
+        mn = make_float3(fminf(mn.x, p.x), fminf(mn.y, p.y), fminf(mn.z, p.z));
+        mx = make_float3(fmaxf(mx.x, p.x), fmaxf(mx.y, p.y), fmaxf(mx.z, p.z));
+        finite = finite && isfinite(p.x) && isfinite(p.y) && isfinite(p.z);
     }
-    if (tid == 0) n_qual = n_list = any = 0;
-    __syncthreads();
+    if (tid == 0) n_qual = n_list = n_near = any = 0;
     int kept = 0;
     if (n > 0) {
-        int S = 1;  // lanes per row
-        while (S < 32 && 2 * S * n <= NT) S *= 2;
-        const int slots = NT / S, sub = tid % S, slot = tid / S;
-        const float c2 = (float)(-1.4426950408889634 * a.inv2s2);
-        // rows i and i + slots: two at a time where the warp has both
-        for (int i0 = slot; i0 - slot < n; i0 += 2 * slots) {
-            const int wbase = i0 - (lane / S);  // the warp's first row
-            if (wbase >= n) break;
-            const int i1 = i0 + slots;
-            float r[2];
-            if (wbase + slots < n) {
-                const float4 p[2] = {pts[min(i0, n - 1)], pts[min(i1, n - 1)]};
-                rqs_density<2>(pts, n, c2, p, sub, S, r);
-            } else {
-                const float4 p[1] = {pts[min(i0, n - 1)]};
-                float one[1];
-                rqs_density<1>(pts, n, c2, p, sub, S, one);
-                r[0] = one[0];
-                r[1] = 0.f;
-            }
-            for (int off = 1; off < S; off <<= 1) {
-                r[0] += __shfl_xor_sync(0xffffffffu, r[0], off);
-                r[1] += __shfl_xor_sync(0xffffffffu, r[1], off);
-            }
-            if (sub == 0) {
+        // ---- tiles of 32 points along a Morton curve (few points: as they are)
+        const int n_tiles = (n + 31) / 32, n32 = n_tiles * 32;
+        int P2 = 64;
+        while (P2 < n) P2 *= 2;
+        if (n > 64) {
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const int i = k ? i1 : i0;
-                    if (i >= n) continue;
-                    // the bound of the file comment (4.8e-7 and 1.08e-6)
-                    // with 2% for its own rounding and second-order terms
-                    const float ln = fmaxf(logf((float)n / r[k]), 0.f) + 0.01f;
-                    const float e = r[k] * (4.9e-7f * ln + 1.1e-6f) + 1e-30f * (float)n;
-                    rho[i] = r[k];
-                    err[i] = e;
+            for (int o = 16; o > 0; o >>= 1) {
+                mn = make_float3(fminf(mn.x, __shfl_xor_sync(0xffffffffu, mn.x, o)),
+                                 fminf(mn.y, __shfl_xor_sync(0xffffffffu, mn.y, o)),
+                                 fminf(mn.z, __shfl_xor_sync(0xffffffffu, mn.z, o)));
+                mx = make_float3(fmaxf(mx.x, __shfl_xor_sync(0xffffffffu, mx.x, o)),
+                                 fmaxf(mx.y, __shfl_xor_sync(0xffffffffu, mx.y, o)),
+                                 fmaxf(mx.z, __shfl_xor_sync(0xffffffffu, mx.z, o)));
+            }
+            float4 *ext = (float4 *)bufs;  // of the warps
+            if (lane == 0) {
+                ext[2 * w] = make_float4(mn.x, mn.y, mn.z, 0.f);
+                ext[2 * w + 1] = make_float4(mx.x, mx.y, mx.z, 0.f);
+            }
+            __syncthreads();
+            for (int k = 0; k < NT / 32; ++k) {
+                const float4 l = ext[2 * k], h = ext[2 * k + 1];
+                mn = make_float3(fminf(mn.x, l.x), fminf(mn.y, l.y), fminf(mn.z, l.z));
+                mx = make_float3(fmaxf(mx.x, h.x), fmaxf(mx.y, h.y), fmaxf(mx.z, h.z));
+            }
+            const float sx = 127.99f / fmaxf(mx.x - mn.x, 1e-6f), sy = 127.99f / fmaxf(mx.y - mn.y, 1e-6f),
+                        sz = 63.99f / fmaxf(mx.z - mn.z, 1e-6f);
+            for (int i = tid; i < P2; i += NT) {
+                uint32_t key = 0xFFFFFFFFu;
+                if (i < n) {
+                    const float4 p = pts[i];
+                    const uint32_t x = (uint32_t)min(max((int)((p.x - mn.x) * sx), 0), 127),
+                                   y = (uint32_t)min(max((int)((p.y - mn.y) * sy), 0), 127),
+                                   z = (uint32_t)min(max((int)((p.z - mn.z) * sz), 0), 63);
+                    key = morton20(x, y, z) << 12 | (uint32_t)i;
                 }
+                keys[i] = key;
+            }
+            __syncthreads();
+            // bitonic sort, strides below 32 within a warp
+            auto in_warp = [&](int k0, int k1) {
+                for (int i = tid; i < P2; i += NT) {
+                    uint32_t x = keys[i];
+                    for (int k = k0; k <= k1; k <<= 1)
+                        for (int j = min(k >> 1, 16); j > 0; j >>= 1) {
+                            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+                            x = ((i & k) == 0) == ((i & j) == 0) ? min(x, y) : max(x, y);
+                        }
+                    keys[i] = x;
+                }
+                __syncthreads();
+            };
+            in_warp(2, 32);
+            for (int k = 64; k <= P2; k <<= 1) {
+                for (int j = k >> 1; j >= 32; j >>= 1) {
+                    for (int e = tid; e < P2 / 2; e += NT) {
+                        const int i = 2 * e - (e & (j - 1));
+                        const uint32_t x = keys[i], y = keys[i + j];
+                        if ((x > y) == ((i & k) == 0)) {
+                            keys[i] = y;
+                            keys[i + j] = x;
+                        }
+                    }
+                    __syncthreads();
+                }
+                in_warp(k, k);
+            }
+        } else {
+            __syncthreads();
+        }
+        for (int k = tid; k < n32; k += NT) {
+            const int i = k < n ? (n > 64 ? (int)(keys[k] & 4095u) : k) : -1;
+            // padding: so far off that its terms are 0
+            const float4 p = i >= 0 ? pts[i] : make_float4(3e38f, 3e38f, 3e38f, 0.f);
+            spts[k] = make_float4(p.x, p.y, p.z, 0.f);
+            need[k] = i & 0xFFFF;
+        }
+        // every group counts where a point is not finite (its distances have no order)
+        const bool all = !__syncthreads_and(finite);
+        const int groups = (n + RQS_GROUP - 1) / RQS_GROUP;
+        for (int t = w; t < n_tiles; t += NT / 32) {
+            const float4 p = spts[min(t * 32 + lane, n - 1)];
+            float4 lo = p, hi = p;
+#pragma unroll
+            for (int o = 1; o < RQS_GROUP; o <<= 1) {
+                lo = make_float4(fminf(lo.x, __shfl_xor_sync(0xffffffffu, lo.x, o)),
+                                 fminf(lo.y, __shfl_xor_sync(0xffffffffu, lo.y, o)),
+                                 fminf(lo.z, __shfl_xor_sync(0xffffffffu, lo.z, o)), 0.f);
+                hi = make_float4(fmaxf(hi.x, __shfl_xor_sync(0xffffffffu, hi.x, o)),
+                                 fmaxf(hi.y, __shfl_xor_sync(0xffffffffu, hi.y, o)),
+                                 fmaxf(hi.z, __shfl_xor_sync(0xffffffffu, hi.z, o)), 0.f);
+            }
+            const int g = (t * 32 + lane) / RQS_GROUP;
+            if (lane % RQS_GROUP == 0 && g < groups) {
+                box[2 * g] = lo;
+                box[2 * g + 1] = hi;
             }
         }
         __syncthreads();
-        // Parent: nearest point of higher density within tau_c (ties:
-        // lower index).  Rows whose nearest undecided pair is not farther
-        // than the parent found in FP32 are listed in `root`.
+        // ---- densities (the sort keys are no longer needed)
+        const float c2 = fminf((float)(-1.4426950408889634 * a.inv2s2), -1.2e-38f);
+        const float cut = all ? INFINITY : -40.f / c2 * 1.0001f;  // terms beyond are below 2^-40
+        for (int t = w; t < n_tiles; t += NT / 32) {
+            const int k = t * 32 + lane;
+            const float4 p = spts[k];
+            float sum = 0.f, comp = 0.f;
+            near_groups(box, groups, t, cut, [&](int g) {
+                float part = 0.f;
+#pragma unroll
+                for (int u = 0; u < RQS_GROUP; ++u) {
+                    const float e = ex2_approx(dist2f(p, spts[g * RQS_GROUP + u]) * c2);
+                    part = u == 0 ? e : part + e;
+                }
+                const float yk = part - comp;  // Kahan sum of the groups
+                const float tk = sum + yk;
+                comp = (tk - sum) - yk;
+                sum = tk;
+            });
+            if (k < n) {
+                const int i = sorted[2 * k];
+                // the bound of the file comment (4.8e-7, 0.8e-6) with 2% for
+                // its own rounding and second-order terms
+                const float ln = fmaxf(logf((float)n / sum), 0.f) + 0.01f;
+                const float e = sum * (4.9e-7f * ln + 1.1e-6f) + 1e-12f * (float)n;
+                rho[i] = sum;
+                err[i] = e;
+                spts[k].w = sum + 1.2f * e;  // exceeds rho + err by more than its rounding
+            }
+        }
+        __syncthreads();
+        // ---- parent: nearest point of higher density within tau_c (ties:
+        // lower index).  A row whose nearest undecided pair is not farther
+        // than the parent found in FP32 is noted in `need`.
         const float tau2f = (float)a.tau2;
         const RqsPar rp{pts, rho, err, rho64, need, &any, a.tau2, tau2f * (1.f - 1.2e-6f), tau2f * (1.f + 1.2e-6f),
                         n};
-        auto found = [&](int i, const RqsBest &o) {
-            parent[i] = o.j;
-            if (o.und < INFINITY && (o.j < 0 || !(o.und > o.d2 * (1.f + 1e-6f)))) root[atomicAdd(&n_list, 1)] = i;
-        };
-        for (int i0 = slot; i0 - slot < n; i0 += 2 * slots) {
-            const int wbase = i0 - (lane / S);
-            if (wbase >= n) break;
-            const int i1 = i0 + slots;
-            if (wbase + slots < n) {
-                const float4 p[2] = {pts[min(i0, n - 1)], pts[min(i1, n - 1)]};
-                const int id[2] = {i0 < n ? i0 : -1, i1 < n ? i1 : -1};
-                RqsBest o[2];
-                rqs_parents<2, RQS_FP32>(rp, p, id, sub, S, o);
+        const float tcut = all ? INFINITY : rp.tau_hi;
+        for (int t = w; t < n_tiles; t += NT / 32) {
+            const int k = t * 32 + lane, i = k < n ? sorted[2 * k] : 0;
+            const float4 p = spts[k];
+            const float ri = rho[i], ei = err[i], least = ri - 1.2f * ei;
+            RqsBest o = {-1, 0.f, INFINITY};
+            float most = k < n ? rp.tau_hi : -1.f;  // candidates beyond are not nearer than the best so far
+            near_groups(box, groups, t, tcut, [&](int g) {
+                uint32_t near = 0;
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    rqs_merge(pts, p[k], S, o[k]);
-                    if (sub == 0 && id[k] >= 0) found(id[k], o[k]);
+                for (int u = 0; u < RQS_GROUP; ++u) {
+                    const float4 q = spts[g * RQS_GROUP + u];
+                    if (!(dist2f(p, q) > most) && !(q.w < least)) near |= 1u << u;  // a NaN goes on
                 }
-            } else {
-                const float4 p[1] = {pts[min(i0, n - 1)]};
-                const int id[1] = {i0 < n ? i0 : -1};
-                RqsBest o[1];
-                rqs_parents<1, RQS_FP32>(rp, p, id, sub, S, o);
-                rqs_merge(pts, p[0], S, o[0]);
-                if (sub == 0 && id[0] >= 0) found(id[0], o[0]);
+                if (k >= n) near = 0;
+                for (; near; near &= near - 1) {
+                    const int c = g * RQS_GROUP + __ffs(near) - 1;
+                    if (c == k || c >= n) continue;
+                    rqs_candidate<RQS_FP32>(rp, p, i, ri, ei, sorted[2 * c], o);
+                    if (o.j >= 0) most = o.d2 * (1.f + 1e-6f);
+                }
+            });
+            if (k < n) {
+                parent[i] = o.j;
+                open[4 * i + 3] = o.und < INFINITY && (o.j < 0 || !(o.und > o.d2 * (1.f + 1e-6f)));
             }
+        }
+        __syncthreads();
+        for (int i = tid; i < n; i += NT) {  // the sorted copy is no longer needed
+            rho64[i] = 0.0;
+            if (need[i] >> 24) root[atomicAdd(&n_list, 1)] = i;
+            need[i] = 0;
         }
         __syncthreads();
         const int listed = n_list;
         if (listed > 0) {
             // a warp per listed row: marks the points to be known in FP64
             for (int e = w; e < listed; e += NT / 32) {
-                const int id[1] = {root[e]};
-                const float4 p[1] = {pts[id[0]]};
-                RqsBest o[1] = {{parent[id[0]], 0.f, 0.f}};
-                if (o[0].j >= 0) o[0].d2 = dist2f(p[0], pts[o[0].j]);
-                rqs_parents<1, RQS_MARK>(rp, p, id, lane, 32, o);
+                const int i = root[e];
+                RqsBest o = {parent[i], 0.f, 0.f};
+                if (o.j >= 0) o.d2 = dist2f(pts[i], pts[o.j]);
+                rqs_row<RQS_MARK>(rp, i, o);
             }
             __syncthreads();
-            // their FP64 densities, by all threads, summed in any order
+            // their FP64 densities, by all threads, summed in any order; terms
+            // below e^-41 (at most 4096 of them, of a sum of 1 or more) left out
+            const float inv2s2 = (float)a.inv2s2;
+            int before = 0, *list = csize;
             for (int b0 = 0; b0 < n; b0 += 32)
                 for (unsigned m = __ballot_sync(0xffffffffu, b0 + lane < n && need[b0 + lane]); m; m &= m - 1) {
                     const int i = b0 + __ffs(m) - 1;
                     const float4 p = pts[i];
-                    double r = 0.0;
-                    for (int j = tid; j < n; j += NT) r += exp(-(dist2(p, pts[j]) * a.inv2s2));
+                    for (int j = tid; j < n; j += NT)
+                        if (!(dist2f(p, pts[j]) * inv2s2 > 41.f)) list[atomicAdd(&n_near, 1) - before] = j;
+                    __syncthreads();
+                    const int end = n_near, c = end - before;
+                    before = end;
+                    if (w * 32 < c) {
+                        double r = 0.0;
+                        for (int e = tid; e < c; e += NT) r += exp(-(dist2(p, pts[list[e]]) * a.inv2s2));
 #pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
-                    if (lane == 0) atomicAdd(&rho64[i], r);
+                        for (int off = 16; off > 0; off >>= 1) r += __shfl_xor_sync(0xffffffffu, r, off);
+                        if (lane == 0) atomicAdd(&rho64[i], r);
+                    }
+                    __syncthreads();
                 }
-            __syncthreads();
             auto again = [&](auto level) {
                 for (int e = w; e < listed; e += NT / 32) {
-                    const int id[1] = {root[e]};
-                    const float4 p[1] = {pts[id[0]]};
-                    RqsBest o[1];
-                    rqs_parents<1, decltype(level)::value>(rp, p, id, lane, 32, o);
-                    rqs_merge(pts, p[0], 32, o[0]);
-                    if (lane == 0) parent[id[0]] = o[0].j;
+                    RqsBest o;
+                    rqs_row<decltype(level)::value>(rp, root[e], o);
+                    if (lane == 0) parent[root[e]] = o.j;
                 }
             };
             again(std::integral_constant<int, RQS_FP64>());
@@ -429,10 +550,12 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
                         const float4 p = pts[i0];
                         double r = 0.0;
                         for (int j0 = 0; j0 < n; j0 += 32) {
-                            if (j0 + lane < n) buf[lane] = exp(-(dist2(p, pts[j0 + lane]) * a.inv2s2));
-                            __syncwarp();
-                            const int m = min(32, n - j0);
-                            for (int k = 0; k < m; ++k) r += buf[k];
+                            // a term below r 2^-55 leaves r as it is
+                            const int j = j0 + lane;
+                            const bool adds = j < n && !(dist2f(p, pts[min(j, n - 1)]) * inv2s2 > 38.7f - logf((float)r));
+                            if (adds) buf[lane] = exp(-(dist2(p, pts[j]) * a.inv2s2));
+                            unsigned m = __ballot_sync(0xffffffffu, adds);
+                            for (; m; m &= m - 1) r += buf[__ffs(m) - 1];
                             __syncwarp();
                         }
                         if (lane == 0) rho64[i0] = r;
@@ -441,6 +564,7 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
                 again(std::integral_constant<int, RQS_ORDER>());
             }
         }
+        for (int i = tid; i < n; i += NT) csize[i] = 0;
         __syncthreads();
         for (int i = tid; i < n; i += NT) {
             int r = i;
@@ -481,46 +605,88 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
             if (lane == 0) cl_start[0] = 0;
         }
         __syncthreads();
-        // Per-cluster statistics, members summed in index order, a warp each.
+        for (int k = w; k < kept; k += NT / 32) {  // the members of each in index order
+            const int r = cl_root[k], c = cl_start[k + 1] - cl_start[k];
+            int *mem = order + cl_start[k];
+            for (int i0 = 0, f = 0; f < c; i0 += 32) {
+                const unsigned in = __ballot_sync(0xffffffffu, i0 + lane < n && root[i0 + lane] == r);
+                if (in >> lane & 1u) mem[f + __popc(in & ((1u << lane) - 1u))] = i0 + lane;
+                f += __popc(in);
+            }
+        }
+        __syncthreads();
+        // Per-cluster statistics, members summed in index order: eight lanes a
+        // cluster, which widen and multiply eight members at once; lane o of
+        // the eight then carries the o-th running sum.  Four clusters of like
+        // size share a warp's FP64 instructions.
         if (w < RQS_STAT_WARPS)
-            for (int k = w; k < kept; k += RQS_STAT_WARPS) {
+            for (int k0 = 4 * w; k0 < kept; k0 += 4 * RQS_STAT_WARPS) {
+                const int o = lane & 7, k = k0 + (lane >> 3);
+                const int s0 = k < kept ? cl_start[k] : 0, c = k < kept ? cl_start[k + 1] - s0 : 0;
+                const int *mem = order + s0;
+                const int most = __shfl_sync(0xffffffffu, c, 0);  // clusters come by descending size
                 double *buf = bufs + w * RQS_BUF;
-                const int r = cl_root[k], c = cl_start[k + 1] - cl_start[k];
-                int *mem = order + cl_start[k];
-                for (int i0 = 0, f = 0; f < c; i0 += 32) {
-                    const unsigned in = __ballot_sync(0xffffffffu, i0 + lane < n && root[i0 + lane] == r);
-                    if (in >> lane & 1u) mem[f + __popc(in & ((1u << lane) - 1u))] = i0 + lane;
-                    f += __popc(in);
-                }
-                __syncwarp();
-                double s = 0.0;  // lane q: the q-th running sum
+                const double *row = buf + 33 * min(o, 5) + (lane & 24);
+                // Sums of FP32 values are exact, so the same in any order, while
+                // their bits span at most 53: a lane then adds every eighth.
+                double s0x = 0.0, s0y = 0.0, s0z = 0.0;
+                Span ex, ey, ez;
                 unsigned sr = 0, sg = 0, sb = 0;
-                for (int f = 0; f < c; f += 32) {
-                    const int m = min(32, c - f);
-                    if (lane < m) {
-                        const float4 p = pts[mem[f + lane]];
-                        buf[lane] = (double)p.x;
-                        buf[33 + lane] = (double)p.y;
-                        buf[66 + lane] = (double)p.z;
-                        const uint32_t rgb = __float_as_uint(p.w);
-                        sr += rgb & 255;
-                        sg += (rgb >> 8) & 255;
-                        sb += (rgb >> 16) & 255;
+                for (int f = o; f < c; f += 8) {
+                    const float4 p = pts[mem[f]];
+                    s0x += widen(p.x);
+                    s0y += widen(p.y);
+                    s0z += widen(p.z);
+                    ex.add(p.x);
+                    ey.add(p.y);
+                    ez.add(p.z);
+                    const uint32_t rgb = __float_as_uint(p.w);
+                    sr += rgb & 255;
+                    sg += (rgb >> 8) & 255;
+                    sb += (rgb >> 16) & 255;
+                }
+#pragma unroll
+                for (int e = 1; e < 8; e <<= 1) {
+                    s0x += __shfl_xor_sync(0xffffffffu, s0x, e);
+                    s0y += __shfl_xor_sync(0xffffffffu, s0y, e);
+                    s0z += __shfl_xor_sync(0xffffffffu, s0z, e);
+                    ex.join(e);
+                    ey.join(e);
+                    ez.join(e);
+                    sr += __shfl_xor_sync(0xffffffffu, sr, e);
+                    sg += __shfl_xor_sync(0xffffffffu, sg, e);
+                    sb += __shfl_xor_sync(0xffffffffu, sb, e);
+                }
+                double s = o == 0 ? s0x : o == 1 ? s0y : s0z;
+                const bool exact = ex.exact(c) && ey.exact(c) && ez.exact(c);
+                if (!__all_sync(0xffffffffu, exact)) {  // one by one
+                    double r = 0.0;
+                    for (int f = 0; f < most; f += 8) {
+                        const int m = c - f;
+                        if (o < m) {
+                            const float4 p = pts[mem[f + o]];
+                            buf[lane] = widen(p.x);
+                            buf[33 + lane] = widen(p.y);
+                            buf[66 + lane] = widen(p.z);
+                        }
+                        __syncwarp();
+                        if (o < 3)
+                            for (int e = 0; e < min(m, 8); ++e) r += row[e];
+                        __syncwarp();
                     }
-                    __syncwarp();
-                    if (lane < 3)
-                        for (int e = 0; e < m; ++e) s += buf[33 * lane + e];
-                    __syncwarp();
+                    if (!exact) s = r;
                 }
                 const double mean = s / c;
-                const double m0 = __shfl_sync(0xffffffffu, mean, 0), m1 = __shfl_sync(0xffffffffu, mean, 1),
-                             m2 = __shfl_sync(0xffffffffu, mean, 2);
+                const double m0 = __shfl_sync(0xffffffffu, mean, lane & 24),
+                             m1 = __shfl_sync(0xffffffffu, mean, (lane & 24) + 1),
+                             m2 = __shfl_sync(0xffffffffu, mean, (lane & 24) + 2);
                 s = 0.0;
-                for (int f = 0; f < c; f += 32) {
-                    const int m = min(32, c - f);
-                    if (lane < m) {
-                        const float4 p = pts[mem[f + lane]];
-                        const double e0 = (double)p.x - m0, e1 = (double)p.y - m1, e2 = (double)p.z - m2;
+                float4 next = o < c ? pts[mem[o]] : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int f = 0; f < most; f += 8) {
+                    const int m = c - f;
+                    const float4 p = next;
+                    if (o < m) {
+                        const double e0 = widen(p.x) - m0, e1 = widen(p.y) - m1, e2 = widen(p.z) - m2;
                         buf[lane] = e0 * e0;
                         buf[33 + lane] = e0 * e1;
                         buf[66 + lane] = e0 * e2;
@@ -529,21 +695,27 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
                         buf[165 + lane] = e2 * e2;
                     }
                     __syncwarp();
-                    if (lane < 6)
-                        for (int e = 0; e < m; ++e) s += buf[33 * lane + e];
+                    if (o + 8 < m) next = pts[mem[f + 8 + o]];
+                    if (o < 6) {
+                        double v[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) v[e] = row[e];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (e < m) s += v[e];
+                    }
                     __syncwarp();
                 }
-                if (lane < 6) cov[k][lane] = c > 1 ? s / (double)(c - 1) : 0.0;
-                if (lane < 3) mu[k][lane] = mean;
-                sr = __reduce_add_sync(0xffffffffu, sr);
-                sg = __reduce_add_sync(0xffffffffu, sg);
-                sb = __reduce_add_sync(0xffffffffu, sb);
-                if (lane == 0) {
-                    const size_t e = (size_t)L * a.m_max + k;
-                    const unsigned h = (unsigned)c / 2, d = (unsigned)c;
-                    a.mrgb[e] = make_uchar4((uint8_t)((sr + h) / d), (uint8_t)((sg + h) / d),
-                                            (uint8_t)((sb + h) / d), 0);
-                    a.msize[e] = c;
+                if (k < kept) {
+                    if (o < 6) cov[k][o] = c > 1 ? s / (double)(c - 1) : 0.0;
+                    if (o < 3) mu[k][o] = mean;
+                    if (o == 0) {
+                        const size_t e = (size_t)L * a.m_max + k;
+                        const unsigned h = (unsigned)c / 2, d = (unsigned)c;
+                        a.mrgb[e] = make_uchar4((uint8_t)((sr + h) / d), (uint8_t)((sg + h) / d),
+                                                (uint8_t)((sb + h) / d), 0);
+                        a.msize[e] = c;
+                    }
                 }
             }
         __syncthreads();
@@ -590,9 +762,9 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
 }
 
 static size_t rqs_smem(int kappa) {
-    const size_t K = (size_t)kappa + (kappa & 1);
-    return K * (sizeof(float4) + sizeof(double) + 2 * sizeof(float) + 4 * sizeof(int)) +
-           RQS_STAT_WARPS * RQS_BUF * sizeof(double);
+    const size_t K = ((size_t)kappa + 31) / 32 * 32;
+    return K * (2 * sizeof(float4) + 2 * sizeof(float) + 2 * sizeof(int)) +
+           K / RQS_GROUP * 2 * sizeof(float4) + RQS_STAT_WARPS * RQS_BUF * sizeof(double);
 }
 
 rl_status update_modes(rl_forest *f, int64_t begin, int64_t count, cudaStream_t s) {

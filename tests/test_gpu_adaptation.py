@@ -77,3 +77,39 @@ def test_reservoirs_and_modes_match_the_oracle(rg, name):
     assert modes.nmodes.max() > 0
     g.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("offset", [0.0, 1e-7, -3e-6, 1e-38])
+def test_means_of_values_of_any_range(rg, offset):
+    """A plane seen head-on: one column of points lies at x = offset, so the
+    sums of a cluster's x are exact or, where their bits span more than 53,
+    rounded in index order."""
+    fp = dict(workloads.FOREST_DEFAULT, n_trees=1, depth=1, kappa=700, m_max=8, min_cluster_size=3, tau_c=0.15,
+              grid_step=2)
+    ctx = rg.Context(0, arena_bytes=1 << 28)
+    g = rg.Forest.random(ctx, fp, 3)
+    o = oracle.forest_random(1, 1, fp["p_depth"], (fp["delta_lo"], fp["delta_hi"]),
+                             (fp["tau_depth_lo"], fp["tau_depth_hi"]), (fp["tau_rgb_lo"], fp["tau_rgb_hi"]),
+                             bool(fp["tau_zero"]), 3)
+    res = oracle.Reservoirs(o, fp["kappa"], 3)
+    K = dataclasses.replace(rooms.intrinsics_for(640, 480), width=96, height=72, fx=120.0, fy=120.0, cx=48.0, cy=36.0)
+    rng = np.random.default_rng(4)
+    d = (2.0 + 0.05 * rng.random((72, 96))).astype(np.float32)
+    rgb = rng.integers(0, 256, (72, 96, 3), dtype=np.uint8)
+    T = np.eye(4)
+    T[0, 3] = offset
+    g.adapt(d, rgb, K, T)
+    res.add_frame(d, rgb, K, T, fp["grid_step"], 0)
+    g.update_modes(-1)
+    modes = oracle.Modes(res.n_leaves, fp["m_max"])
+    oracle.update_modes(res, modes, fp["sigma"], fp["tau_c"], fp["min_cluster_size"], cov_eps=fp["cov_eps"],
+                        fp16_offsets=True)
+    e = g.export(reservoirs=True)
+    np.testing.assert_array_equal(e["res_count"], res.count)
+    np.testing.assert_array_equal(e["nmodes"], modes.nmodes)
+    np.testing.assert_array_equal(e["mode_size"], modes.size.reshape(e["mode_size"].shape))
+    np.testing.assert_allclose(e["mode_pos"], modes.pos.reshape(e["mode_pos"].shape), rtol=2e-7, atol=1e-9)
+    np.testing.assert_allclose(e["mode_U"], modes.U.reshape(e["mode_U"].shape), rtol=2e-7, atol=1e-9)
+    assert modes.size.max() > 50
+    g.close()
+    ctx.close()
