@@ -354,15 +354,22 @@ rl_status launch_scale_nodes(const rl_forest *f, int n_trees, float4 *out, float
 // counts are committed.
 //
 // Threads of steps 4 and 5 follow the list, so that the lanes of a warp
-// mostly loop over one segment; a block stages its segments in shared memory
-// and reads them by broadcast.  A leaf's cost is the square of its arrivals
-// in this frame (a thousand or two in the fullest leaf of a room), spread
-// over as many threads.
-// Measured on GB300 (640x480, 19,200 grid pixels, 5 trees of depth 11): 72 us
-// a frame (13 walk, 4 segments, 4 scatter, 20 slots, 28 insert, 3 commit);
-// 620 us with a thread per pixel walking all trees, ranks from all pairs of
-// pixels and the slot of every later example drawn again by each example.
+// mostly look at one segment.  Segments shorter than EX_WIDE are staged in
+// shared memory and read by broadcast, each example against all the others.
+// A longer one (a thousand or two in the fullest leaf of a room) gets a table
+// in every block that holds a part of it: a bitmap of its pixels, whose
+// running count is the rank, and the last pixel of each slot.
+// Measured on GB300 (640x480, 19,200 grid pixels, 5 trees of depth 11): 33 us
+// a frame (11 walk, 3 segments, 2 scatter, 8 slots, 8 insert, 2 commit).
+// Every entry against every other in long segments too: 18 us slots, 27 us
+// insert.  A thread per pixel walking all trees, ranks from all pairs of
+// pixels and the slot of every later example drawn again: 620 us.
 // ---------------------------------------------------------------------------
+constexpr int EX_THREADS = 128, EX_TILE = 1024;
+constexpr int EX_WIDE = 256;      // entries from which a segment gets a table
+constexpr int EX_TABLE = 4096;    // its words: 131,072 pixels at a time, or the largest capacity
+constexpr int EX_MAX_TREES = 16;
+
 struct Pose12 {
     double m[12];
 };
@@ -372,8 +379,10 @@ __global__ void k_adapt_examples(const float4 *__restrict__ nodes, int n_branch,
                                  const uint8_t *__restrict__ C, int W, int H, float fx, float fy,
                                  float cx, float cy, Pose12 T, int gw, int gh, int step, int origin,
                                  uint32_t *__restrict__ ex_leaf, uint32_t *__restrict__ ex_rank,
-                                 float4 *__restrict__ ex_pt, uint32_t *__restrict__ frame_cnt) {
+                                 float4 *__restrict__ ex_pt, uint32_t *__restrict__ frame_cnt,
+                                 uint32_t *__restrict__ used) {
     const int P = gw * gh;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < EX_MAX_TREES) used[threadIdx.x] = 0;
     const int g = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;  // a thread per (grid pixel, tree)
     if (g >= P) return;
     const int x = origin + (g % gw) * step, y = origin + (g / gw) * step;
@@ -437,8 +446,6 @@ __device__ __forceinline__ int64_t reservoir_slot(uint32_t L, uint32_t c, int ka
 }
 
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
-constexpr int EX_THREADS = 128, EX_TILE = 1024;
-
 // Runs f(first, last) on every thread of a block for the part of its segment
 // [sg.x, sg.x + sg.y) in each tile of the block's segments (load(q0, n) stages
 // entries q0 .. q0 + n in shared memory); threads without a segment have
@@ -468,21 +475,79 @@ __device__ __forceinline__ void segment_tiles(uint2 sg, Load load, F f) {
     }
 }
 
+// Runs f(segment) for the segments of EX_WIDE entries or more that the block
+// holds a part of: sg is the segment of the thread's entry, live >= 1 the
+// block's entries.  Being longer than a block, such a segment holds the
+// block's first entry or its last.
+template <class F>
+__device__ __forceinline__ void wide_segments(uint2 sg, uint32_t live, F f) {
+    static_assert(EX_WIDE >= EX_THREADS, "at most two wide segments in a block");
+    __shared__ uint2 ends[2];
+    if (threadIdx.x == 0) ends[0] = sg;
+    if (threadIdx.x == live - 1) ends[1] = sg;
+    __syncthreads();
+    const uint2 a = ends[0], b = ends[1];
+    if (a.y >= EX_WIDE) f(a);
+    if (b.y >= EX_WIDE && b.x != a.x) f(b);
+}
+
 // slot[k]: the slot of entry k of the list, or kNoSlot.
 __global__ void __launch_bounds__(EX_THREADS) k_adapt_slots(
     const uint32_t *__restrict__ ex_leaf, const uint32_t *__restrict__ list, int P, const uint2 *__restrict__ seg,
     const uint32_t *__restrict__ used, const uint32_t *__restrict__ res_count, int kappa, uint32_t k0, uint32_t k1,
     uint32_t *__restrict__ slot) {
-    __shared__ uint32_t s_g[EX_TILE];
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
-    const bool on = r < used[t];
+    __shared__ uint32_t s_g[EX_TILE], table[EX_TABLE], chunk[EX_THREADS], sum[EX_THREADS / 32];
+    const uint32_t r0 = blockIdx.x * EX_THREADS, r = r0 + threadIdx.x, t = blockIdx.y, end = used[t];
+    if (r0 >= end) return;
+    const bool on = r < end;
     const size_t k = (size_t)t * P + r;
     const uint32_t g = on ? list[k] : 0;
     const uint32_t L = on ? ex_leaf[(size_t)t * P + g] : 0;
     const uint2 sg = on ? seg[L] : make_uint2(0, 0);
     uint32_t rank = 0;
+    wide_segments(sg, min(end - r0, (uint32_t)EX_THREADS), [&](uint2 e) {
+        for (uint32_t w0 = 0; w0 < (uint32_t)P; w0 += EX_TABLE * 32) {  // the set bits below g
+            const uint32_t words = min((uint32_t)EX_TABLE, ((uint32_t)P - w0 + 31) / 32);
+            for (uint32_t i = threadIdx.x; i < words; i += EX_THREADS) table[i] = 0;
+            __syncthreads();
+            for (uint32_t q = threadIdx.x; q < e.y; q += EX_THREADS) {
+                const uint32_t d = list[e.x + q] - w0;
+                if (d < words * 32) atomicOr(&table[d >> 5], 1u << (d & 31));
+            }
+            __syncthreads();
+            // a thread's words, then the sums of the threads before it
+            const uint32_t per = (words + EX_THREADS - 1) / EX_THREADS, i0 = threadIdx.x * per;
+            uint32_t n = 0;
+            for (uint32_t i = i0; i < min(i0 + per, words); ++i) n += __popc(table[i]);
+            uint32_t upto = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+                if ((threadIdx.x & 31) >= o) upto += v;
+            }
+            if ((threadIdx.x & 31) == 31) sum[threadIdx.x >> 5] = upto;
+            __syncthreads();
+            uint32_t before = upto - n, total = 0;
+            for (uint32_t i = 0; i < EX_THREADS / 32; ++i) {
+                if (i < threadIdx.x >> 5) before += sum[i];
+                total += sum[i];
+            }
+            chunk[threadIdx.x] = before;
+            __syncthreads();
+            if (on && sg.x == e.x && sg.y && g >= w0) {
+                const uint32_t d = g - w0, word = d >> 5;
+                if (word >= words) {
+                    rank += total;
+                } else {
+                    rank += chunk[word / per] + __popc(table[word] & ((1u << (d & 31)) - 1u));
+                    for (uint32_t i = word / per * per; i < word; ++i) rank += __popc(table[i]);
+                }
+            }
+            __syncthreads();
+        }
+    });
     segment_tiles(
-        sg, [&](uint32_t q0, uint32_t n) {
+        sg.y < EX_WIDE ? sg : make_uint2(0, 0), [&](uint32_t q0, uint32_t n) {
             for (uint32_t q = threadIdx.x; q < n; q += EX_THREADS) s_g[q] = list[q0 + q];
         },
         [&](uint32_t first, uint32_t last) {
@@ -499,17 +564,30 @@ __global__ void __launch_bounds__(EX_THREADS) k_adapt_insert(
     const float4 *__restrict__ ex_pt, int P, const uint2 *__restrict__ seg, const uint32_t *__restrict__ used,
     const uint32_t *__restrict__ res_count, int kappa, float4 *__restrict__ res) {
     __shared__ uint2 s_gs[EX_TILE];
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
+    __shared__ uint32_t table[EX_TABLE];
+    const uint32_t r0 = blockIdx.x * EX_THREADS, r = r0 + threadIdx.x, t = blockIdx.y, end = used[t];
+    if (r0 >= end) return;
     const size_t k = (size_t)t * P + r;
-    const uint32_t mine = r < used[t] ? slot[k] : kNoSlot;
+    const uint32_t mine = r < end ? slot[k] : kNoSlot;
     const bool on = mine != kNoSlot;
-    const uint32_t g = on ? list[k] : 0;
-    const uint32_t L = on ? ex_leaf[(size_t)t * P + g] : 0;
-    uint2 sg = on ? seg[L] : make_uint2(0, 0);
-    if (on && res_count[L] + sg.y <= (uint32_t)kappa) sg = make_uint2(0, 0);  // every example has a slot of its own
+    const uint32_t g = r < end ? list[k] : 0;
+    const uint32_t L = r < end ? ex_leaf[(size_t)t * P + g] : 0;
+    uint2 sg = r < end ? seg[L] : make_uint2(0, 0);
+    if (sg.y && res_count[L] + sg.y <= (uint32_t)kappa) sg = make_uint2(0, 0);  // every example has a slot of its own
     bool later = false;
+    wide_segments(sg, min(end - r0, (uint32_t)EX_THREADS), [&](uint2 e) {
+        for (int i = threadIdx.x; i < kappa; i += EX_THREADS) table[i] = 0;
+        __syncthreads();
+        for (uint32_t q = threadIdx.x; q < e.y; q += EX_THREADS) {
+            const uint32_t s = slot[e.x + q];
+            if (s != kNoSlot) atomicMax(&table[s], list[e.x + q] + 1);
+        }
+        __syncthreads();
+        if (on && sg.x == e.x && sg.y) later = table[mine] != g + 1;
+        __syncthreads();
+    });
     segment_tiles(
-        sg, [&](uint32_t q0, uint32_t n) {
+        on && sg.y < EX_WIDE ? sg : make_uint2(0, 0), [&](uint32_t q0, uint32_t n) {
             for (uint32_t q = threadIdx.x; q < n; q += EX_THREADS) s_gs[q] = make_uint2(list[q0 + q], slot[q0 + q]);
         },
         [&](uint32_t first, uint32_t last) {
@@ -553,7 +631,7 @@ rl_status adapt_frame(rl_forest *f, const float *depth, const uint8_t *rgb,
         RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees, &f->ex_leaf));
         RL_TRY(alloc_n(f->ctx, (uint64_t)P, &f->ex_pt));
         RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees, &f->ex_rank));
-        RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees + 16, &f->ex_list));  // then the entries in use per tree
+        RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees + EX_MAX_TREES, &f->ex_list));  // then the entries in use per tree
         RL_TRY(alloc_n(f->ctx, (uint64_t)f->n_leaves, &f->ex_seg));
         f->ex_capacity = P;
     }
@@ -561,11 +639,10 @@ rl_status adapt_frame(rl_forest *f, const float *depth, const uint8_t *rgb,
     for (int i = 0; i < 12; ++i) pose.m[i] = T[i];
     const uint32_t k0 = (uint32_t)f->seed, k1 = (uint32_t)(f->seed >> 32);
     uint32_t *used = f->ex_list + (size_t)P * p.n_trees;
-    RL_CK(cudaMemsetAsync(used, 0, 16 * sizeof(uint32_t), s));
     const dim3 grid((P + EX_THREADS - 1) / EX_THREADS, p.n_trees);
     k_adapt_examples<<<grid, EX_THREADS, 0, s>>>(f->nodes, f->n_branch, p.depth, f->leaves_per_tree, depth, rgb, K->width,
                                           K->height, K->fx, K->fy, K->cx, K->cy, pose, gw, gh, st, o, f->ex_leaf,
-                                          f->ex_rank, f->ex_pt, f->frame_cnt);
+                                          f->ex_rank, f->ex_pt, f->frame_cnt, used);
     RL_LAUNCH_CK();
     k_adapt_segments<<<(f->n_leaves + 255) / 256, 256, 0, s>>>(f->frame_cnt, f->n_leaves, f->leaves_per_tree, P,
                                                                f->ex_seg, used);

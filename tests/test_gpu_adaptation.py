@@ -32,6 +32,8 @@ CASES = {
     "two rows a thread": dict(trees=1, depth=1, kappa=1025, m_max=64, size=(101, 67), step=1, frames=2, min_size=2),
     "largest capacity": dict(trees=1, depth=1, kappa=4096, m_max=64, size=(160, 120), step=1, frames=1, min_size=5),
     "leaves of every size": dict(trees=3, depth=7, kappa=200, m_max=10, size=(160, 120), step=2, frames=6, min_size=1),
+    "more pixels than a table's": dict(trees=2, depth=2, kappa=50, m_max=4, size=(480, 360), step=1, frames=2,
+                                       min_size=2),
     "repeated frames": dict(trees=2, depth=3, kappa=300, m_max=12, size=(96, 72), step=3, frames=4, min_size=3,
                             repeat=True),
 }
