@@ -316,8 +316,12 @@ __global__ void __launch_bounds__(1024) k_select(SelectArgs a) {
 // to 250 modes; CT grows to 8 while the call's blocks still fit two per SM.
 // A large batch keeps CT = 1: the lanes that share a scan idle through the
 // accumulation, about a quarter more instructions.  Measured on four 640x480
-// frames, 64 hypotheses, up to 250 modes per pixel, six rounds: 4.5 ms with
-// CT = 8, 17.9 with one block per part.
+// frames, 64 hypotheses, up to 250 modes per pixel, six rounds: 4.2 ms with
+// CT = 8 (4.4 when a step's count and point were not loaded a step ahead),
+// 17.9 with one block per part.  What bounds it then is the latency of a
+// step's chain of loads with two warps per sub-partition, not the scan:
+// CT = 16 took as long, and so did rows read once for a warp's hypotheses
+// (4.8 ms) or eight modes at a time (5.2 ms).
 constexpr int LM3_THREADS = 256;
 constexpr int LM3_BPQ = 4;
 constexpr int LM3_HMAX = 64 / LM3_BPQ;  // hypotheses of a part (n_cull <= 64)
@@ -404,14 +408,24 @@ __global__ void __launch_bounds__(LM3_THREADS, 2) k_lm_spread(LmArgs a) {
             float P[12];
 #pragma unroll
             for (int k = 0; k < 12; ++k) P[k] = act ? (float)s_H[hl][k] : 0.f;
+            int next_cnt = 0;
+            float4 next_x = make_float4(0.f, 0.f, 0.f, 0.f);
+            auto fetch = [&](int st) {  // a step ahead: what its scan waits for
+                const int i = st * G + g;
+                const bool on = act && i < a.n_pix;
+                next_cnt = on ? (int)tcnt[i] : 0;
+                if (on) next_x = xcs[i];
+            };
+            fetch(0);
             for (int st = 0; st < steps; ++st) {
                 const int i = st * G + g;
                 const bool on = act && i < a.n_pix;
-                const int cnt = on ? (int)tcnt[i] : 0;
+                const int cnt = next_cnt;
+                const float4 x = next_x;
+                fetch(st + 1);
                 const size_t base = (size_t)i * stride;
                 float y0 = 0.f, y1 = 0.f, y2 = 0.f;
                 if (cnt > 0) {
-                    const float4 x = xcs[i];
                     y0 = fmaf(P[0], x.x, fmaf(P[1], x.y, fmaf(P[2], x.z, P[3])));
                     y1 = fmaf(P[4], x.x, fmaf(P[5], x.y, fmaf(P[6], x.z, P[7])));
                     y2 = fmaf(P[8], x.x, fmaf(P[9], x.y, fmaf(P[10], x.z, P[11])));
