@@ -115,3 +115,32 @@ def test_means_of_values_of_any_range(rg, offset):
     assert modes.size.max() > 50
     g.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("m_max,precision,chunk", [(1, 0, 1), (7, 1, 5), (50, 1, 11), (64, 0, 16), (33, 1, 40)])
+def test_streaming_store_catches_up(rg, m_max, precision, chunk):
+    """After every round-robin update the front store of a streaming forest
+    holds what the single store of another holds."""
+    fp = dict(workloads.FOREST_DEFAULT, n_trees=2, depth=3, kappa=120, m_max=m_max, min_cluster_size=2, tau_c=0.15,
+              grid_step=3, mode_precision=precision)
+    ctx = rg.Context(0, arena_bytes=1 << 28)
+    forests = [rg.Forest.random(ctx, fp, 8) for _ in range(2)]
+    forests[1].set_streaming(True)
+    room = rooms.Room((4.0, 3.0, 2.5), 5)
+    K = dataclasses.replace(rooms.intrinsics_for(640, 480), width=96, height=72, fx=120.0, fy=120.0, cx=48.0, cy=36.0)
+    for i, T in enumerate(rooms.training_trajectory(room, 5)):
+        d, rgb = rooms.render(room, K, T, noise_seed=40 + i)
+        stores = []
+        for f in forests:
+            f.adapt(d, rgb, K, T)
+            f.update_modes(chunk)
+            stores.append(f.export())
+        a, b = stores
+        np.testing.assert_array_equal(a["nmodes"], b["nmodes"])
+        held = np.arange(m_max)[None, :] < a["nmodes"][:, None]  # the others are not set before a leaf's first update
+        for k in ("mode_pos", "mode_rgb", "mode_U", "mode_size"):
+            np.testing.assert_array_equal(a[k][held], b[k][held], err_msg=k)
+    assert held.any()
+    for f in forests:
+        f.close()
+    ctx.close()
