@@ -14,8 +14,7 @@
 //    closer than 1e-6 relative are redone in FP64;
 //  - densities: term t = 2^(d2 c), c = -log2(e) / (2 sigma^2) rounded, its
 //    argument within 7 u relative, ex2.approx within 2^-22 relative; terms
-//    summed in groups of 8 whose sums are Kahan-added, then over at most 32
-//    lanes: within 14 u.  With x = -ln t the exact exponents,
+//    summed in groups of 8 whose sums are Kahan-added: within 14 u.  With x = -ln t the exact exponents,
 //    |rho32 - rho64| <= 8 u sum(t x) + (14 u + 2^-22) rho, and sum(t x) <=
 //    rho ln(n / rho) (the entropy bound, equality when all terms are equal).
 //    Terms below 2^-40 are left out where whole tiles of points are that far
@@ -43,11 +42,13 @@
 // lanes compute eight members' products at once, then carry a running sum
 // each (a warp per cluster took three FP64 instructions a member, a thread
 // per cluster 27).
-// Of 297 thousand cycles of a full leaf of 1024 points with the columns in
-// tiles of 32, the sort took 24, densities 44, parents 77, FP64 densities 54,
-// comparisons in FP64 29 and the sums 43 (training; 21, 52, 134, 20, 10 and
-// 93 online, where clusters are larger).  A cluster of four blocks on each
-// full leaf was slower: the full leaves fill the GPU.
+// Thousands of cycles of a leaf of more than 600 points, training / online
+// (where clusters are larger), before the means were summed in parallel: sort
+// 19 / 18, densities 49 / 61, parents 60 / 71, FP64 densities 13 / 8, FP64
+// comparisons 20 / 10, members 5 / 10, cluster sums 33 / 73, factors 11 / 10.
+// With the columns in groups of 32, every column of a group compared and a
+// warp per cluster it was 297 and 350 in all.  A cluster of four blocks on
+// each full leaf was slower: the full leaves fill the GPU.
 //
 // Measured on GB300: 10,240 leaves of 107 points on average, about 800 of
 // more than 600 (24 frames of 640x480, 5 trees of depth 11, capacity 1024):
