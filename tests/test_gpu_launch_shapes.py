@@ -107,3 +107,33 @@ def test_icp_does_not_depend_on_the_poses_in_the_call(rg, size):
         H.check_icp_one(whole[1][i], whole[2][i], whole[0][i], ok, frac, P, 0.5, f"pose {i}")
     scene.close()
     ctx.close()
+
+
+@pytest.mark.parametrize("inside,outside", [(1, 0), (3, 0), (4, 0), (17, 0), (3, 1), (15, 1), (16, 17), (1, 32)])
+def test_scores_do_not_depend_on_the_poses_beside(rg, inside, outside):
+    """Groups of four poses are reduced together while all of a chunk are
+    inside the box: a pose's score has the same bits alone, and the inside
+    poses' match the FP64 oracle (FP32 rays: 1e-4 relative)."""
+    w = workloads.small_case(n_trees=1, depth=3, n_train=1)
+    room, rng = w.room(), np.random.default_rng(inside * 64 + outside)
+    depth, _ = rooms.render(room, w.K, rooms.look_pose([2.0, 1.4, 1.3], 2.0, -0.1), noise_seed=2)
+    depth = rooms.mask_depth(depth, 0.25, seed=9)
+    lo, hi = np.asarray(room.lo, np.float64), np.asarray(room.hi, np.float64)
+    poses = []
+    for k in range(inside + outside):
+        at = lo + (hi - lo) * rng.uniform(0.2, 0.8, 3)
+        if k >= inside:
+            at[k % 3] = lo[k % 3] - rng.uniform(0.1, 1.0)
+        poses.append(rooms.look_pose(at, rng.uniform(-3, 3), rng.uniform(-0.3, 0.3)))
+    poses = np.stack(poses)[rng.permutation(inside + outside)]
+    ctx = rg.Context(0, arena_bytes=1 << 26)
+    scene = rg.Scene(ctx, lo, hi)
+    s, f = scene.score_poses(depth, w.K, poses)
+    for i, P in enumerate(poses):
+        s1, f1 = scene.score_poses(depth, w.K, poses[i:i + 1])
+        assert s[i] == s1[0] and f[i] == f1[0], i
+        o_s, _, _ = oracle.depth_score(P, depth, w.K, room.lo, room.hi)
+        if np.all(P[:3, 3] > lo) and np.all(P[:3, 3] < hi):
+            assert abs(s[i] - o_s) <= 1e-4 * o_s, (i, s[i], o_s)
+    scene.close()
+    ctx.close()
