@@ -556,6 +556,7 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
                             const bool adds = j < n && !(dist2f(p, pts[min(j, n - 1)]) * inv2s2 > 38.7f - logf((float)r));
                             if (adds) buf[lane] = exp(-(dist2(p, pts[j]) * a.inv2s2));
                             unsigned m = __ballot_sync(0xffffffffu, adds);
+                            __syncwarp();  // the lanes' terms are read by all (a vote orders no memory)
                             for (; m; m &= m - 1) r += buf[__ffs(m) - 1];
                             __syncwarp();
                         }
