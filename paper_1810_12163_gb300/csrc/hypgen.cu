@@ -354,8 +354,11 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) k_hypgen(HypArgs a) {
     constexpr int step = pairs ? 64 : 32;
     bool done = slot >= a.p.n_hyp;
     for (int base = mate * step; base < a.p.max_iter && !done; base += team * step) {
-        // a team mate's success comes first (what is pending may come before it)
-        if (*(volatile int *)&s_best[sl] < base) break;
+        // A team mate's success comes first (what is pending may come before it).
+        // The mates write s_best meanwhile, so lane 0's reading counts for the
+        // warp: all its lanes have to stop or go on together, ballots follow.
+        const int best = *(volatile int *)&s_best[sl];
+        if (__shfl_sync(0xffffffffu, best, 0) < base) break;
         if (pairs) {
             Draw dA, dB;
             bool sA, sB;
