@@ -324,13 +324,21 @@ __global__ void __launch_bounds__(ICP_THREADS, 3) k_icp(IcpArgs a) {
     }
 }
 
+// Where warps of different roles meet: __syncthreads() wants every thread of
+// the block at one place of the program, a named barrier (1: __syncthreads()
+// is 0) only THREADS of them at any.  Orders their memory accesses alike.
+template <int THREADS>
+__device__ __forceinline__ void role_barrier() {
+    asm volatile("barrier.cta.sync 1, %0;" ::"n"(THREADS) : "memory");
+}
+
 // The same by a cluster of C blocks per pose, for calls of few poses: the
 // sums of the one-block kernel are serial chains of a thread (1,200 pixels at
 // full resolution), so what they leave idle can only prepare their terms.
 // Block c owns the chains of the one-block kernel's warps c OW, ... (OW = 8 /
 // C streams, a lane per chain); its helper warps evaluate the streams'
 // pixels ahead, a chunk at a time, and hand (depth, gap, direction, axis)
-// over in shared memory, double-buffered with a block barrier per chunk.  The
+// over in shared memory, double-buffered with a barrier per chunk.  The
 // owners add the terms in the same order and the lanes and warps are reduced
 // in the same order, so the results do not depend on C.  Block 0 solves; the
 // pose goes back through distributed shared memory.
@@ -432,7 +440,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(IcpTeam<C, AX>::thre
                                 }
                             }
                         }
-                        __syncthreads();
+                        role_barrier<NT>();
                     }
                 };
                 if constexpr (AX == 1)
@@ -489,7 +497,7 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(IcpTeam<C, AX>::thre
                             s_b[ck & 1][stream][i][lane] = make_float2(dir[2], __int_as_float(ax));
                         }
                     }
-                    __syncthreads();
+                    role_barrier<NT>();
                 }
                 visited += (unsigned long long)n_valid;
                 n_in = __reduce_add_sync(0xffffffffu, n_in);
