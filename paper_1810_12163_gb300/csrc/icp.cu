@@ -37,12 +37,12 @@ constexpr int ICP_NS = 27;
 template <int O>
 __device__ __forceinline__ void icp_add(float acc[ICP_NS], float P1, float P2, float r) {
     acc[O] += 1.f;
-    acc[O + 1] += P1;
-    acc[O + 2] += P2;
+    acc[O + 1] = __fadd_rn(acc[O + 1], P1);
+    acc[O + 2] = __fadd_rn(acc[O + 2], P2);
     acc[O + 3] = fmaf(P1, P1, acc[O + 3]);
     acc[O + 4] = fmaf(P2, P2, acc[O + 4]);
     acc[O + 5] = fmaf(P1, P2, acc[O + 5]);
-    acc[O + 6] += r;
+    acc[O + 6] = __fadd_rn(acc[O + 6], r);
     acc[O + 7] = fmaf(P1, r, acc[O + 7]);
     acc[O + 8] = fmaf(P2, r, acc[O + 8]);
 }
@@ -54,7 +54,9 @@ __device__ __forceinline__ void icp_add(float acc[ICP_NS], float P1, float P2, f
 // the first face hit is the exit face, s = min over axes of the distance to
 // the face the ray heads for; otherwise the general slab test (exit from
 // inside, entry from outside).  exit_num[ax] = (hi - t, t - lo) for the two
-// ray directions.
+// ray directions.  Here and in the sums, products and additions that the
+// compiler may or may not fuse are rounded by name: the kernels below have to
+// agree to the bit whatever it would make of each of them.
 template <bool INSIDE>
 __device__ __forceinline__ int icp_gap(const IcpArgs &a, float d, int u, int v, float cx, float cy, float ifx,
                                        float ify, const float R[9], const float t[3], const float exit_hi[3],
@@ -64,7 +66,6 @@ __device__ __forceinline__ int icp_gap(const IcpArgs &a, float d, int u, int v, 
     const float c0 = ((float)u - cx) * ifx, c1 = ((float)v - cy) * ify;
 #pragma unroll
     for (int r = 0; r < 3; ++r) dir[r] = fmaf(R[3 * r], c0, fmaf(R[3 * r + 1], c1, R[3 * r + 2]));
-    float sh;
     int ax;
     if (INSIDE) {
         // exit distance along axis k: e_k / |dir_k| (e_k > 0); the smallest is
@@ -77,7 +78,7 @@ __device__ __forceinline__ int icp_gap(const IcpArgs &a, float d, int u, int v, 
             const float nk = dir[k] > 0.f ? exit_hi[k] : exit_lo[k], dk = fabsf(dir[k]);
             if (nk * da < na * dk) { na = nk; da = dk; ax = k; }
         }
-        sh = na * rcp_approx(da);
+        gap = fmaf(-na, rcp_approx(da), d);
     } else {
         float tn = -INFINITY, tf = INFINITY;
         int an = 0, af = 0;
@@ -89,16 +90,15 @@ __device__ __forceinline__ int icp_gap(const IcpArgs &a, float d, int u, int v, 
                 continue;
             }
             const float inv = rcp_approx(dir[k]);
-            const float t1 = (a.lo[k] - t[k]) * inv, t2 = (a.hi[k] - t[k]) * inv;
+            const float t1 = __fmul_rn(a.lo[k] - t[k], inv), t2 = __fmul_rn(a.hi[k] - t[k], inv);
             const float tmin = fminf(t1, t2), tmax = fmaxf(t1, t2);
             if (tmin > tn) { tn = tmin; an = k; }
             if (tmax < tf) { tf = tmax; af = k; }
         }
         if (!hit || tn > tf || !(tf > 0.f)) return -1;
-        sh = tn > 0.f ? tn : tf;
+        gap = __fsub_rn(d, tn > 0.f ? tn : tf);
         ax = tn > 0.f ? an : af;
     }
-    gap = d - sh;
     const float dd2 = fmaf(dir[0], dir[0], fmaf(dir[1], dir[1], dir[2] * dir[2]));
     return gap * gap * dd2 > dist2 ? -1 : ax;
 }
@@ -109,15 +109,15 @@ __device__ __forceinline__ void icp_terms(int ax, float d, float gap, float dir0
                                           float acc[ICP_NS]) {
     // q' = d dir (the camera point rotated into the world frame); residual
     // r = n . (q - p) = gap dir[ax]
-    const float q0 = d * dir0, q1 = d * dir1, q2 = d * dir2;
+    const float q0 = __fmul_rn(d, dir0), q1 = __fmul_rn(d, dir1), q2 = __fmul_rn(d, dir2);
     // neighbouring pixels of a warp mostly share a face, so the branch on
     // the axis rarely diverges; constant offsets keep acc in registers
     if (ax == 0)
-        icp_add<0>(acc, q2, -q1, gap * dir0);
+        icp_add<0>(acc, q2, -q1, __fmul_rn(gap, dir0));
     else if (ax == 1)
-        icp_add<9>(acc, q0, -q2, gap * dir1);
+        icp_add<9>(acc, q0, -q2, __fmul_rn(gap, dir1));
     else
-        icp_add<18>(acc, q1, -q0, gap * dir2);
+        icp_add<18>(acc, q1, -q0, __fmul_rn(gap, dir2));
 }
 
 // The same for the sums of one axis, given q' there (P1, P2) and the residual;
@@ -125,12 +125,12 @@ __device__ __forceinline__ void icp_terms(int ax, float d, float gap, float dir0
 __device__ __forceinline__ void icp_add_axis(float s[9], bool on, float P1, float P2, float r) {
     const float u = on ? P1 : 0.f, v = on ? P2 : 0.f, w = on ? r : 0.f;
     s[0] += on ? 1.f : 0.f;
-    s[1] += u;
-    s[2] += v;
+    s[1] = __fadd_rn(s[1], u);
+    s[2] = __fadd_rn(s[2], v);
     s[3] = fmaf(u, u, s[3]);
     s[4] = fmaf(v, v, s[4]);
     s[5] = fmaf(u, v, s[5]);
-    s[6] += w;
+    s[6] = __fadd_rn(s[6], w);
     s[7] = fmaf(u, w, s[7]);
     s[8] = fmaf(v, w, s[8]);
 }
@@ -435,8 +435,8 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(IcpTeam<C, AX>::thre
                                     if (ax >= 0) icp_terms(ax, va.x, va.y, va.z, va.w, vb.x, acc);
                                 } else {  // as icp_terms
                                     const float dir[3] = {va.z, va.w, vb.x};
-                                    icp_add_axis(acc, ax == AXIS, va.x * dir[(AXIS + 2) % 3],
-                                                 -(va.x * dir[(AXIS + 1) % 3]), va.y * dir[AXIS]);
+                                    icp_add_axis(acc, ax == AXIS, __fmul_rn(va.x, dir[(AXIS + 2) % 3]),
+                                                 -__fmul_rn(va.x, dir[(AXIS + 1) % 3]), __fmul_rn(va.y, dir[AXIS]));
                                 }
                             }
                         }
