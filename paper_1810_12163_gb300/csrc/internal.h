@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/relocgb.h"
+#include "lm_shape.h"
 
 // ---------------------------------------------------------------------------
 // Error plumbing: every ABI entry point returns rl_status; the message of the
@@ -304,6 +305,7 @@ struct rl_reloc {
     // sub-batches of a call (tune.streams): private streams and fork/join events
     cudaStream_t side[7] = {};
     cudaEvent_t fork_ev = nullptr, join_ev[7] = {};
+    rl::LmResident lm_resident;             // LM clusters that the GPU holds at once
     uint32_t lm_wait_limit = kLmWaitLimit;  // probes of the LM kernel's waits for staged tiles
     // streaming forests: recorded after the last launch that read mode store b
     cudaEvent_t read_done[2] = {nullptr, nullptr};

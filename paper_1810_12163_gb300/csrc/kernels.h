@@ -61,6 +61,7 @@ struct LmArgs {
     uint32_t wait_limit;       // probes of a wait for a staged tile before it gives up
     int n_active;              // frames at work on the GPU at once (shapes the launch, never the result)
     int sm_count;
+    LmResident resident;       // clusters that the GPU holds at once, by shape
 };
 
 rl_status prepare_kernels();
@@ -75,6 +76,8 @@ rl_status launch_lm_cluster(const LmArgs &a, int n, cudaStream_t s);
 // refined pose's Eq. 5 energy in q.cur_energy).
 bool lm_uses_cluster(const RParams &p);
 rl_status prepare_lm_cluster();
+// The current device's; after prepare_lm_cluster, outside any stream capture.
+LmResident lm_resident();
 
 // Ranking raycast tiles: 256 threads x RC_PIX pixels; one partial record
 // per (frame, pose, tile).

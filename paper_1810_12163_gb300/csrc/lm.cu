@@ -15,12 +15,13 @@
 // which order, depends on RANKS and on the hypotheses listed alone; SUBS only
 // spreads the hypotheses over more CTAs, whose lanes then share the mode scan
 // of a pair (S lanes of it each).  A call of few frames leaves most SMs idle
-// with SUBS = 1 (one frame: 4 of 152), so SUBS grows while the call's CTAs
-// fit the GPU.  Measured on 640x480 frames of up to 50 modes per pixel: first
-// round of 8 frames 1391 us with SUBS = 1, 941 with 4; of one frame 572 and
-// 439; a later round (RANKS = 8) of 8 frames 445 and, with 2, 365.  What
-// bounds it then is the issue of two warps per sub-partition (36% of cycles)
-// on the scans and the normal equations' serial chains.
+// with SUBS = 1 (one frame: 4 of 152), so SUBS grows with what the GPU holds
+// of the larger clusters (lm_sets).  Measured on 640x480 frames of up to 50
+// modes per pixel: first round of 8 frames 1391 us with SUBS = 1, 941 with 4;
+// of one frame 572 and 439; a later round (RANKS = 8) of 8 frames 445 and,
+// with 2, 365.  What bounds it then is the issue of two warps per
+// sub-partition (36% of cycles) on the scans and the normal equations' serial
+// chains.
 //
 // A pass streams the CTA's tiles of the mode table (rows of decoded M(u))
 // into shared memory with bulk asynchronous copies on an mbarrier pipeline.
@@ -1026,35 +1027,65 @@ static rl_status launch_lm_shape(const LmArgs &a, int n, cudaStream_t s) {
     return RL_OK;
 }
 
-// The cluster of a round with RANKS CTAs on the pixels.  SUBS > 1 while the
-// call's CTAs fit the SMs that whole clusters of 8 or 16 can fill (16 of the
-// 19 of a GPC), one per SM, and rows are long enough: the lanes that share a
-// scan idle through the normal equations, so with up to 9 modes per pixel
-// SUBS = 4 was slower (8 frames 3.43 ms a call against 2.99).  Rows too long
-// for the deeper pipeline's shared memory keep SUBS = 1.
-template <int RANKS, int MOST>
-static rl_status launch_lm_ranks(const LmArgs &a, int n, cudaStream_t s) {
-    const int ctas = a.n_active * RANKS, room = a.sm_count / 19 * 16;
-    if (a.p.maxm >= LMC_SPLIT_MODES && lmc_layout(a.p.mpad, a.p.use_cov, LMC_STAGES_SUB).total <= kLmClusterSmemMax) {
-        if (ctas * MOST <= room) return launch_lm_shape<RANKS, MOST>(a, n, s);
-        if (ctas * 2 <= room) return launch_lm_shape<RANKS, 2>(a, n, s);
-    }
-    return launch_lm_shape<RANKS, 1>(a, n, s);
-}
-
+// SUBS > 1 (lm_sets) where rows are long enough: the lanes that share a scan
+// idle through the normal equations, so with up to 9 modes per pixel SUBS = 4
+// was slower (8 frames 3.43 ms a call against 2.99).  Rows too long for the
+// deeper pipeline's shared memory keep SUBS = 1.
 rl_status launch_lm_cluster(const LmArgs &a, int n, cudaStream_t s) {
-    // round r refines on eta * (r + 2) pixels
-    return a.n_pix <= 2 * a.p.eta ? launch_lm_ranks<LMC_RANKS_FIRST, 4>(a, n, s)
-                                  : launch_lm_ranks<LMC_RANKS_LATER, 2>(a, n, s);
+    const bool first = a.n_pix <= 2 * a.p.eta;  // round r refines on eta * (r + 2) pixels
+    const bool split = a.p.maxm >= LMC_SPLIT_MODES &&
+                       lmc_layout(a.p.mpad, a.p.use_cov, LMC_STAGES_SUB).total <= kLmClusterSmemMax;
+    const int sets = split ? lm_sets(a.resident, first, a.n_active) : 1;
+    if (first) {
+        if (sets == 4) return launch_lm_shape<LMC_RANKS_FIRST, 4>(a, n, s);
+        if (sets == 2) return launch_lm_shape<LMC_RANKS_FIRST, 2>(a, n, s);
+        return launch_lm_shape<LMC_RANKS_FIRST, 1>(a, n, s);
+    }
+    if (sets == 2) return launch_lm_shape<LMC_RANKS_LATER, 2>(a, n, s);
+    return launch_lm_shape<LMC_RANKS_LATER, 1>(a, n, s);
 }
 
 template <int RANKS, int SUBS>
 static rl_status prepare_lm_shape() {
     RL_CK(cudaFuncSetAttribute(k_lm_cluster<RANKS, SUBS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kLmClusterSmemMax));
-    if (RANKS * SUBS > 8)  // clusters above 8 CTAs are not portable and must be allowed explicitly
-        RL_CK(cudaFuncSetAttribute(k_lm_cluster<RANKS, SUBS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    // clusters above 8 CTAs are not portable and must be allowed explicitly;
+    // where they are not, none is resident and the shape is never launched
+    if (RANKS * SUBS > 8 && cudaFuncSetAttribute(k_lm_cluster<RANKS, SUBS>,
+                                                 cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        cudaGetLastError();
     return RL_OK;
+}
+
+// With the most shared memory a launch may ask for, which leaves one CTA per
+// SM, so that the count holds for every relocaliser.
+template <int RANKS, int SUBS>
+static int resident_clusters() {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(RANKS * SUBS);
+    cfg.blockDim = dim3(LMC_THREADS);
+    cfg.dynamicSmemBytes = kLmClusterSmemMax;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = RANKS * SUBS;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_lm_cluster<RANKS, SUBS>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+LmResident lm_resident() {
+    LmResident r;
+    r.first4 = resident_clusters<LMC_RANKS_FIRST, 4>();
+    r.first2 = resident_clusters<LMC_RANKS_FIRST, 2>();
+    r.later2 = resident_clusters<LMC_RANKS_LATER, 2>();
+    return r;
 }
 
 rl_status prepare_lm_cluster() {

@@ -255,7 +255,8 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
         const int n_pix = p.eta * (round + 2);
         const bool lm = p.pose_update && p.lm_max_iter > 0;
         if (lm) {
-            LmArgs la{q, q.leaves, hw_max, mv, p, n_pix, work, maxm, maxm | 1, r->lm_wait_limit, n_active, f->ctx->sm_count};
+            LmArgs la{q, q.leaves, hw_max, mv, p, n_pix, work, maxm, maxm | 1, r->lm_wait_limit, n_active, f->ctx->sm_count,
+                      r->lm_resident};
             PROF(K_LM);
             RL_TRY(launch_lm(la, n, s));
         }
@@ -590,6 +591,7 @@ extern "C" rl_status rl_reloc_create(rl_forest *f, rl_scene *scene, const rl_ran
     r->max_w = max_w;
     r->max_h = max_h;
     r->max_batch = max_batch;
+    r->lm_resident = lm_resident();
     RParams &rp = r->rp;
     rp.n_hyp = p->n_hyp; rp.max_iter = p->max_iter; rp.n_cull = p->n_cull; rp.eta = p->eta;
     rp.k_out = p->k_out; rp.pose_update = p->pose_update; rp.use_cov = p->use_cov;
