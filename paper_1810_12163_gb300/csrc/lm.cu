@@ -686,6 +686,9 @@ __global__ void __cluster_dims__(RANKS *SUBS, 1, 1) __launch_bounds__(LMC_THREAD
         if (t == 0) s_nl[0] = s_nl[1] = 0;
         __syncthreads();
         if (dir_ok && !first) {
+            // a staged pass that gave up has left correspondences and anchors
+            // unwritten, whose indices are not to be followed
+            act = act && !*s_abort;
             // rows from global memory; chunks of Gp * LMC_KP of the CTA's
             // pixels (local pixel j is pixel j % 16 of tile crank + (j / 16) * RANKS)
             const int n_local = my_tiles * LMC_P;
