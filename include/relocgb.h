@@ -351,10 +351,10 @@ rl_status rl_reloc_set_graphs(rl_reloc *r, int32_t enable);
 rl_status rl_reloc_graph_kernels(rl_reloc *r, int32_t n, int32_t *out);
 /* Failure injection for tests of the device-side failure path (the paper
  * has no counterpart).  The LM kernel waits, with a bound, for the bulk
- * copies that stage its mode-table tiles; a wait that runs out marks the
- * frame, the kernel skips the rest of that frame's work, drains its copies
- * in flight (always with the full bound) and the call returns
- * RL_ERR_TIMEOUT.  `probes` sets how many times a tile wait probes before it
+ * copies that stage its mode-table tiles, and for a stage to be free for the
+ * next; a wait that runs out marks the frame, the kernel skips the rest of
+ * that frame's work, drains its copies in flight (always with the full
+ * bound) and the call returns RL_ERR_TIMEOUT.  `probes` sets how many times such a wait probes before it
  * gives up (0: at once); a negative value restores the default (2^22).
  * Synchronises the device and drops the relocaliser's captured graphs,
  * which hold the limit; a cascade's graphs keep the limit they were captured

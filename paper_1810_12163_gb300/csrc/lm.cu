@@ -50,10 +50,10 @@
 // values; each CTA solves every hypothesis's 6x6 system in FP64 and takes
 // the same decisions, with one cluster barrier per iteration.
 //
-// Every wait on a copy is bounded: a wait that gives up marks the frame in
-// dev_err, the CTA skips the rest of its work while keeping step with the
-// cluster barriers, and waits (bounded again) for its copies in flight
-// before it exits.
+// Every wait on a copy, or for a stage to be free, is bounded: one that gives
+// up marks the frame in dev_err, the CTA skips the rest of its work while
+// keeping step with the cluster barriers, and waits (bounded again) for its
+// copies in flight before it exits.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -346,7 +346,8 @@ __global__ void __cluster_dims__(RANKS *SUBS, 1, 1) __launch_bounds__(LMC_THREAD
     };
     auto issue = [&](int j) {  // the pass's j-th tile of this CTA
         const uint32_t q = q_pass + (uint32_t)j, s = q % STAGES;
-        if (SUBS > 1 && q >= STAGES && !mbar_wait_bounded(bar0 + 8 * (STAGES + s), (q / STAGES - 1) & 1u, kWaitLimit, s_abort)) {
+        if (SUBS > 1 && q >= STAGES &&
+            !mbar_wait_bounded(bar0 + 8 * (STAGES + s), (q / STAGES - 1) & 1u, a.wait_limit, s_abort)) {
             give_up();
             return;
         }

@@ -30,6 +30,15 @@ def test_lm_waits_run_out_then_recover(rg, model, n, n_cull):  # noqa: F811
         rel.relocalise_batch(depth, rgb, w.K, seeds)
     assert e.value.status == 5  # RL_ERR_TIMEOUT
     torch.cuda.synchronize()  # the context is still usable
+    for probes in (1, 2, 8):  # copies and stages late for some of the waits, for all or for none
+        rel.set_wait_limit(probes)
+        try:
+            got = rel.relocalise_batch(depth, rgb, w.K, seeds)
+        except rg.RelocError as e:
+            assert e.status == 5
+            continue
+        for a, b in zip(got, before):
+            np.testing.assert_array_equal(a["chosen_pose"], b["chosen_pose"], err_msg=f"{probes} probes")
     rel.set_wait_limit(-1)
     for graphs in (False, True):
         rel.set_graphs(graphs)
