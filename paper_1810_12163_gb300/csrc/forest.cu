@@ -88,9 +88,16 @@ __device__ __forceinline__ int walk_tree(const float4 *__restrict__ nodes, int d
     return n - ((1 << depth) - 1);
 }
 
+// A call's node (k_scale_nodes): offsets times fx / 585, and for the split
+// either kSplitDepth or the selector of a byte permute that makes the float
+// 2^23 + c of the channel's colour byte c; its low 4 bits are the channel.
+constexpr uint32_t kSplitDepth = 0x80000000u;
+constexpr uint32_t kSplitByte = 0x7540u;  // bytes c, 0x00, 0x00, 0x4B of (colours, 0x4B000000)
+
 // All T trees of one pixel walked level by level, interleaved: T
 // independent chains of dependent node and probe loads in flight at once.
-template <int T>
+// PRE: the nodes are a call's.
+template <int T, bool PRE>
 __device__ __forceinline__ void walk_trees(const float4 *__restrict__ nodes, int n_branch, int depth,
                                            const float *__restrict__ D, const uint8_t *__restrict__ C,
                                            int W, int H, float s, int x, int y, float d, float inv,
@@ -106,15 +113,15 @@ __device__ __forceinline__ void walk_trees(const float4 *__restrict__ nodes, int
 #pragma unroll
         for (int t = 0; t < T; ++t) {
             const uint32_t meta = __float_as_uint(nd[t].w);
-            const float ox = __fmul_rn(__fmul_rn(nd[t].x, s), inv);
-            const float oy = __fmul_rn(__fmul_rn(nd[t].y, s), inv);
+            const float ox = __fmul_rn(PRE ? nd[t].x : __fmul_rn(nd[t].x, s), inv);
+            const float oy = __fmul_rn(PRE ? nd[t].y : __fmul_rn(nd[t].y, s), inv);
             const int q = probe_coord(y, oy, H) * W + probe_coord(x, ox, W);
             float f;
-            if ((meta & 255u) == 0u) {
+            if (PRE ? meta == kSplitDepth : (meta & 255u) == 0u) {
                 const float dq = __ldg(&D[q]);
                 f = __fsub_rn(d, dq > 0.0f ? dq : 0.0f);
             } else {
-                const int c = (int)(meta >> 8);
+                const int c = (int)(PRE ? meta & 15u : meta >> 8);
                 f = __fsub_rn((float)__ldg(&C[p * 3 + c]), (float)__ldg(&C[q * 3 + c]));
             }
             n[t] = (f >= nd[t].z) ? 2 * n[t] + 2 : 2 * n[t] + 1;
@@ -124,13 +131,13 @@ __device__ __forceinline__ void walk_trees(const float4 *__restrict__ nodes, int
     for (int t = 0; t < T; ++t) leaf[t] = n[t] - ((1 << depth) - 1);
 }
 
-template <int T>
+template <int T, bool PRE>
 __device__ __forceinline__ int walk_and_store(const float4 *nodes, int n_branch, int depth, const Frame &fr,
                                               float s, int x, int y, float d, float inv, uint16_t *o,
                                               int hw_max, const uint8_t *nmodes, int lpt, int k_top,
                                               bool count, uint4 *rec) {
     int leaf[kRecTrees], cnt[kRecTrees];
-    walk_trees<T>(nodes, n_branch, depth, fr.depth, fr.rgb, fr.W, fr.H, s, x, y, d, inv, leaf);
+    walk_trees<T, PRE>(nodes, n_branch, depth, fr.depth, fr.rgb, fr.W, fr.H, s, x, y, d, inv, leaf);
     int total = 0;
 #pragma unroll
     for (int t = 0; t < T; ++t) {
@@ -147,10 +154,13 @@ __device__ __forceinline__ int walk_and_store(const float4 *nodes, int n_branch,
 // When `mcount` is given it also receives |M(u)| = sum over the trees of
 // min(modes of the reached leaf, k_top) per pixel (0 without depth); the
 // pixel records `prec` (at most kRecTrees trees) hold the per-tree counts.
+// nodes_s: the call's nodes for focal length fx_s, taken for the frames of
+// that focal length, or null.
 __global__ void k_leaves(const float4 *__restrict__ nodes, int n_branch, int depth, int n_trees,
                          const Frame *__restrict__ frames, int hw_max, uint16_t *__restrict__ out,
                          const uint8_t *__restrict__ nmodes, int leaves_per_tree, int k_top,
-                         uint16_t *__restrict__ mcount, uint4 *__restrict__ prec) {
+                         uint16_t *__restrict__ mcount, uint4 *__restrict__ prec,
+                         const float4 *__restrict__ nodes_s, float fx_s) {
     const Frame fr = frames[blockIdx.y];
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= fr.W * fr.H) return;
@@ -169,9 +179,12 @@ __global__ void k_leaves(const float4 *__restrict__ nodes, int n_branch, int dep
     const float inv = __frcp_rn(d);
     int total = 0;
     const bool cnt = mcount != nullptr || prec != nullptr;  // per-tree counts wanted
-#define RL_WALK(T)                                                                                            \
-    total = walk_and_store<T>(nodes, n_branch, depth, fr, s, x, y, d, inv, o, hw_max, nmodes, leaves_per_tree, \
-                              k_top, cnt, rec)
+    const bool pre = nodes_s != nullptr && fr.fx == fx_s;   // the same for the whole block (one frame)
+#define RL_WALK(T)                                                                                          \
+    total = pre ? walk_and_store<T, true>(nodes_s, n_branch, depth, fr, s, x, y, d, inv, o, hw_max, nmodes, \
+                                          leaves_per_tree, k_top, cnt, rec)                                  \
+                : walk_and_store<T, false>(nodes, n_branch, depth, fr, s, x, y, d, inv, o, hw_max, nmodes,  \
+                                           leaves_per_tree, k_top, cnt, rec)
     switch (n_trees) {
     case 1: RL_WALK(1); break;
     case 2: RL_WALK(2); break;
@@ -192,12 +205,13 @@ __global__ void k_leaves(const float4 *__restrict__ nodes, int n_branch, int dep
 
 rl_status launch_leaves(const rl_forest *f, const Frame *frames_dev, int n_frames, int n_trees,
                         int hw_max, uint16_t *out, int max_w, int max_h, cudaStream_t s,
-                        int k_top, uint16_t *mcount, uint4 *prec, int threads) {
+                        int k_top, uint16_t *mcount, uint4 *prec, int threads, const float4 *nodes_s,
+                        float fx_s) {
     const int npx = max_w * max_h;
     dim3 grid((npx + threads - 1) / threads, n_frames);
     k_leaves<<<grid, threads, 0, s>>>(f->nodes, f->n_branch, f->p.depth, n_trees, frames_dev, hw_max, out,
                                   f->nmodes, f->leaves_per_tree, k_top, mcount,
-                                  n_trees <= kRecTrees ? prec : nullptr);
+                                  n_trees <= kRecTrees ? prec : nullptr, nodes_s, fx_s);
     RL_LAUNCH_CK();
     return RL_OK;
 }
@@ -214,28 +228,27 @@ rl_status launch_leaves(const rl_forest *f, const Frame *frames_dev, int n_frame
 //    the difference of the colours;
 //  - the call's nodes carry the offsets times fx / 585 and the permute's
 //    selector, and a coordinate is clamped by one min-with-relu.
+// It needs 8 bytes per pixel that nothing else uses yet (run_relocalise);
+// k_leaves walks the frames as they are where there is no such place.
 // That is 33 instructions a test instead of 44.  Measured on 8 frames of
 // 640x480, 5 trees of depth 15: 208 us + 11 us of packing (was 267; 75% issue,
 // the gathers' latency next), one frame 38 + 4 us (51).
 // ---------------------------------------------------------------------------
-constexpr uint32_t kSplitDepth = 0x80000000u;  // packed node: Depth split; else the permute selector
-constexpr uint32_t kSplitByte = 0x7540u;       // bytes c, 0x00, 0x00, 0x4B of (colours, 0x4B000000)
-
 __device__ __forceinline__ float4 pack_node(float4 v, float s) {
     const uint32_t meta = __float_as_uint(v.w);
     const uint32_t sel = (meta & 255u) == 0u ? kSplitDepth : kSplitByte | (meta >> 8);
     return make_float4(__fmul_rn(v.x, s), __fmul_rn(v.y, s), v.z, __uint_as_float(sel));
 }
 
-// frame b's pixels at out + b * stride
+// frame b's pixels at out + b * hw_max
 __global__ void __launch_bounds__(256) k_pack_frames(const Frame *__restrict__ frames, uint2 *__restrict__ out,
-                                                     size_t stride) {
+                                                     int hw_max) {
     const Frame fr = frames[blockIdx.y];
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= fr.W * fr.H) return;
     const float d = fr.depth[p];
     const uint8_t *c = fr.rgb + (size_t)p * 3;
-    out[blockIdx.y * stride + p] = make_uint2(__float_as_uint(d > 0.0f ? d : 0.0f),
+    out[(size_t)blockIdx.y * hw_max + p] = make_uint2(__float_as_uint(d > 0.0f ? d : 0.0f),
                                               (uint32_t)c[0] | ((uint32_t)c[1] << 8) | ((uint32_t)c[2] << 16));
 }
 
@@ -280,12 +293,12 @@ __device__ __forceinline__ uint4 walk_packed(const float4 *__restrict__ nodes, i
 template <int T>
 __global__ void k_leaves_packed(const float4 *__restrict__ nodes, const float4 *__restrict__ nodes_s, float fx_s,
                                 int n_branch, int depth, const Frame *__restrict__ frames, int hw_max,
-                                const uint2 *__restrict__ packed, size_t stride, const uint8_t *__restrict__ nmodes,
+                                const uint2 *__restrict__ packed, const uint8_t *__restrict__ nmodes,
                                 int leaves_per_tree, int k_top, uint4 *__restrict__ prec) {
     const Frame fr = frames[blockIdx.y];
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= fr.W * fr.H) return;
-    const uint2 *px = packed + blockIdx.y * stride;
+    const uint2 *px = packed + (size_t)blockIdx.y * hw_max;
     const uint2 own = px[p];
     const float d = __uint_as_float(own.x);
     uint4 rec = make_uint4(0, 0, 0, 0);
@@ -304,13 +317,13 @@ __global__ void k_leaves_packed(const float4 *__restrict__ nodes, const float4 *
 
 rl_status launch_leaves_packed(const rl_forest *f, const Frame *frames_dev, int n_frames, int n_trees, int hw_max,
                                cudaStream_t s, int k_top, uint4 *prec, int threads, const float4 *nodes_s, float fx_s,
-                               uint2 *packed, size_t stride) {
-    k_pack_frames<<<dim3((hw_max + 255) / 256, n_frames), 256, 0, s>>>(frames_dev, packed, stride);
+                               uint2 *packed) {
+    k_pack_frames<<<dim3((hw_max + 255) / 256, n_frames), 256, 0, s>>>(frames_dev, packed, hw_max);
     RL_LAUNCH_CK();
     const dim3 grid((hw_max + threads - 1) / threads, n_frames);
 #define RL_WALK(T)                                                                                                 \
     k_leaves_packed<T><<<grid, threads, 0, s>>>(f->nodes, nodes_s, fx_s, f->n_branch, f->p.depth, frames_dev, hw_max, \
-                                                packed, stride, f->nmodes, f->leaves_per_tree, k_top, prec)
+                                                packed, f->nmodes, f->leaves_per_tree, k_top, prec)
     switch (n_trees) {
     case 1: RL_WALK(1); break;
     case 2: RL_WALK(2); break;

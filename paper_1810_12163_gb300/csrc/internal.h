@@ -396,14 +396,14 @@ rl_status launch_forest_random(rl_forest *f, cudaStream_t s);
 rl_status launch_leaves(const rl_forest *f, const Frame *frames_dev, int n_frames, int n_trees,
                         int hw_max, uint16_t *out, int max_w, int max_h, cudaStream_t s,
                         int k_top = 0, uint16_t *mcount = nullptr, uint4 *prec = nullptr,
-                        int threads = 128);
+                        int threads = 128, const float4 *nodes_s = nullptr, float fx_s = 0.f);
 // Pixel records of at most kRecTrees trees from frames packed into `packed`
-// (stride pixels per frame), nodes_s the call's nodes for focal length fx_s.
+// (hw_max pixels per frame), nodes_s the call's nodes for focal length fx_s.
 rl_status launch_leaves_packed(const rl_forest *f, const Frame *frames_dev, int n_frames, int n_trees, int hw_max,
                                cudaStream_t s, int k_top, uint4 *prec, int threads, const float4 *nodes_s, float fx_s,
-                               uint2 *packed, size_t stride);
+                               uint2 *packed);
 // The first n_trees trees' split nodes for the walk of a call at focal length
-// fx (read by launch_leaves_packed for frames of that focal length).
+// fx (read by both walks for frames of that focal length).
 rl_status launch_scale_nodes(const rl_forest *f, int n_trees, float4 *out, float fx, cudaStream_t s);
 rl_status adapt_frame(rl_forest *f, const float *depth, const uint8_t *rgb,
                       const rl_intrinsics *K, const double T[16], cudaStream_t s);

@@ -163,6 +163,18 @@ static void prof_resolve(rl_reloc *r) {
 
 #define PROF(kid) ProfScope prof_scope_##kid##__LINE__(r, kid, s)
 
+// Where the walk's packed frames go (n frames of hw pixels), with pixel
+// records: an array that nothing reads until the walk is done, the colour
+// masks', or without masks the leaf maps', which are not written with records
+// (at 2 bytes per tree large enough for 8 a pixel from four trees on, of
+// which the alignment takes up to 6 bytes).  Null: no place.
+static uint2 *packed_frames(const QueryState &q, int n_trees, int n, size_t hw) {
+    if (!q.prec || q.pcm) return q.pcm;
+    const uintptr_t at = ((uintptr_t)q.leaves + 7) / 8 * 8;
+    const uintptr_t end = (uintptr_t)q.leaves + sizeof(uint16_t) * n_trees * hw * n;
+    return at + sizeof(uint2) * hw * n <= end ? (uint2 *)at : nullptr;
+}
+
 rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, int level, cudaStream_t s) {
     rl_forest *f = r->forest;
     RParams p = r->rp;
@@ -180,21 +192,14 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
     // count map is written
     {
         PROF(K_LEAVES);
-        // packed frames go where nothing is live yet: the colour masks' array
-        // (written after the walk) or the leaf maps' (not written with records)
-        uint2 *packed = q.pcm;
-        size_t stride = hw_max;
-        if (!packed && (size_t)p.n_trees * hw_max * sizeof(uint16_t) % sizeof(uint2) == 0 &&
-            p.n_trees * sizeof(uint16_t) >= sizeof(uint2)) {
-            packed = (uint2 *)q.leaves;
-            stride = (size_t)p.n_trees * hw_max * sizeof(uint16_t) / sizeof(uint2);
-        }
-        if (q.prec && packed)
+        uint2 *packed = packed_frames(q, p.n_trees, n, hw_max);
+        const float fx = r->host_frames[0].fx;
+        if (packed)
             RL_TRY(launch_leaves_packed(f, q.frames, n, p.n_trees, hw_max, s, p.k_top, q.prec, r->tune.leaves_threads,
-                                        r->nodes_s, r->host_frames[0].fx, packed, stride));
+                                        r->nodes_s, fx, packed));
         else
             RL_TRY(launch_leaves(f, q.frames, n, p.n_trees, hw_max, q.prec ? nullptr : q.leaves, r->max_w, r->max_h, s,
-                                 p.k_top, q.prec ? nullptr : q.mcount, q.prec, r->tune.leaves_threads));
+                                 p.k_top, q.prec ? nullptr : q.mcount, q.prec, r->tune.leaves_threads, r->nodes_s, fx));
     }
     if (q.pcm) { PROF(K_CMASK); RL_TRY(launch_colour_mask(q.frames, q.mcount, q.prec, hw_max, mv, p, q.pcm, q.pbits, n, hw_max, s, r->tune.mask_threads)); }
     else if (q.pbits) { PROF(K_CMASK); RL_TRY(launch_mode_bits(q.frames, q.prec, hw_max, p.n_trees, q.pbits, n, s)); }
