@@ -183,7 +183,7 @@ constexpr uint32_t kLmWaitLimit = 1u << 22;
 // Device-resident per-query RANSAC state (arrays sized for max_batch).
 struct QueryState {
     uint16_t *leaves;        // [B][T][HWmax]
-    uint16_t *mcount;        // [B][HWmax] |M(u)| per pixel
+    uint16_t *mcount;        // [B][HWmax] |M(u)| per pixel, null with pixel records
     uint4 *prec;             // [B][HWmax] per-pixel leaves + counts (<= 5 trees), else null
     uint2 *pcm;              // [B][HWmax] colour-check bits of M(u) | |M(u)| << 56 (|M(u)| <= 56), else null
     uint32_t *pbits;         // [B][HWmax / 32 + 1] bit p: M(u) of pixel p is non-empty (with prec)

@@ -627,8 +627,8 @@ extern "C" rl_status rl_reloc_create(rl_forest *f, rl_scene *scene, const rl_ran
         r->q_layout.push_back({offsetof(QueryState, field), (size_t)((count) / B) * sizeof(*q.field)}); \
     }
     A(leaves, B * p->n_trees_used * hw);
-    A(mcount, B * hw);
     if (p->n_trees_used <= kRecTrees) A(prec, B * hw);
+    if (!q.prec) A(mcount, B * hw);  // the records hold the counts
     if (p->n_trees_used <= kRecTrees && maxm <= kMaskModes) A(pcm, B * hw);
     if (q.prec) A(pbits, B * (hw / 32 + 1));
     A(hyp_pose, B * N * 12);
