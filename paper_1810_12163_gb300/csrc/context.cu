@@ -258,8 +258,7 @@ static rl_status check_forest_params(const rl_forest_params *p) {
 static void forest_release(rl_forest *f) {
     rl_ctx *c = f->ctx;
     void *ptrs[] = {f->nodes, f->res, f->res_count, f->nmodes, f->centroid, f->mpos_h, f->mpos_f,
-                    f->mrgb, f->mU, f->msize, f->ex_leaf, f->ex_pt, f->ex_rank, f->ex_list, f->ex_seg, f->frame_cnt,
-                    f->stage_depth, f->stage_rgb};
+                    f->mrgb, f->mU, f->msize, f->ex_leaf, f->ex_pt, f->ex_list, f->frame_cnt, f->stage_depth, f->stage_rgb};
     for (void *p : ptrs) arena_free(c, p);
     free_store(c, f->alt);
     if (f->ready) cudaEventDestroy(f->ready);

@@ -4,6 +4,10 @@
 // Compiled with --fmad=false: the FP32 feature arithmetic and the FP64
 // back-projection are plain IEEE operations in a fixed order, so leaves and
 // reservoir contents are exactly reproducible.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "internal.h"
 #include "relocgb_dev.cuh"
 
@@ -355,16 +359,20 @@ rl_status launch_scale_nodes(const rl_forest *f, int n_trees, float4 *out, float
 // Reservoir adaptation (Sec. 3.2.2), deterministic Algorithm R.
 //
 // For one frame: (1) every grid pixel with depth is back-projected, moved to
-// world space and walked down every tree; each example takes an arrival
-// number in its leaf (in any order).  (2) Every leaf with arrivals gets a
-// segment of the frame's example list.  (3) The examples are scattered into
-// their leaf's segment.  (4) An example's rank
+// world space and walked down every tree, and its leaves count it.  (2) Every
+// leaf gets a segment of the frame's example list, in leaf order, and its
+// reservoir's count goes up by the segment's length.  (3) The examples are
+// scattered into their leaf's segment (in any order).  (4) An example's rank
 // among the frame's examples of its leaf, in pixel order, is the number of
 // smaller pixels in its segment; it gives the count c = count_before_frame +
 // rank and, with it, Algorithm R's slot, a pure function of (leaf, c).  (5)
 // An example writes its slot unless a later example of the same leaf in this
-// frame draws the same slot.  (6) The
-// counts are committed.
+// frame draws the same slot.
+//
+// Scratch is two words per example (list entry; leaf and slot of 16 bits) and
+// the points.  A segment needs no record of its own: step 3 advances a leaf's
+// count from where its segment starts to where it ends, and it starts where
+// the leaf before ends.
 //
 // Threads of steps 4 and 5 follow the list, so that the lanes of a warp
 // mostly look at one segment.  Segments shorter than EX_WIDE are staged in
@@ -372,16 +380,20 @@ rl_status launch_scale_nodes(const rl_forest *f, int n_trees, float4 *out, float
 // A longer one (a thousand or two in the fullest leaf of a room) gets a table
 // in every block that holds a part of it: a bitmap of its pixels, whose
 // running count is the rank, and the last pixel of each slot.
-// Measured on GB300 (640x480, 19,200 grid pixels, 5 trees of depth 11): 33 us
-// a frame (11 walk, 3 segments, 2 scatter, 8 slots, 8 insert, 2 commit).
-// Every entry against every other in long segments too: 18 us slots, 27 us
-// insert.  A thread per pixel walking all trees, ranks from all pairs of
+// Measured on GB300 (640x480, 19,200 grid pixels, 5 trees of depth 15): 33 us
+// a frame (clearing 1.5, walk 11, segments 5, scatter 2.5, slots 7, insert
+// 6.5), a call 47 us; of depth 11 a call is 43 us, of depth 6 43 (59 with an
+// atomic per example, whose leaves are then full).  With a record per segment
+// and words of their own for arrival numbers and slots, 4 bytes more per
+// example and 8 per leaf, the calls took 48, 47 and 59 us.  Every entry
+// against every other in long segments too: 18 us slots, 27 us insert.  A thread per pixel walking all trees, ranks from all pairs of
 // pixels and the slot of every later example drawn again: 620 us.
 // ---------------------------------------------------------------------------
 constexpr int EX_THREADS = 128, EX_TILE = 1024;
 constexpr int EX_WIDE = 256;      // entries from which a segment gets a table
 constexpr int EX_TABLE = 4096;    // its words: 131,072 pixels at a time, or the largest capacity
-constexpr int EX_MAX_TREES = 16;
+constexpr uint16_t kNoLeaf = 0xFFFFu, kNoSlot = 0xFFFFu;  // a tree has at most 2^15, capacities are at most 4096
+constexpr int EX_SCAN_THREADS = 1024, EX_SCAN_EACH = 4;  // eight blocks: 2^15 leaves, the most a tree has
 
 struct Pose12 {
     double m[12];
@@ -391,19 +403,17 @@ __global__ void k_adapt_examples(const float4 *__restrict__ nodes, int n_branch,
                                  int leaves_per_tree, const float *__restrict__ D,
                                  const uint8_t *__restrict__ C, int W, int H, float fx, float fy,
                                  float cx, float cy, Pose12 T, int gw, int gh, int step, int origin,
-                                 uint32_t *__restrict__ ex_leaf, uint32_t *__restrict__ ex_rank,
-                                 float4 *__restrict__ ex_pt, uint32_t *__restrict__ frame_cnt,
-                                 uint32_t *__restrict__ used) {
+                                 uint16_t *__restrict__ ex_leaf, float4 *__restrict__ ex_pt,
+                                 uint32_t *__restrict__ frame_cnt) {
     const int P = gw * gh;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < EX_MAX_TREES) used[threadIdx.x] = 0;
     const int g = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;  // a thread per (grid pixel, tree)
-    if (g >= P) return;
     const int x = origin + (g % gw) * step, y = origin + (g / gw) * step;
     const int p = y * W + x;
-    const float d = D[p];
+    const float d = g < P ? D[p] : 0.0f;
     const size_t e = (size_t)t * P + g;
+    const unsigned live = __ballot_sync(0xffffffffu, d > 0.0f);
     if (!(d > 0.0f)) {
-        ex_leaf[e] = 0xFFFFFFFFu;
+        if (g < P) ex_leaf[e] = kNoLeaf;
         return;
     }
     if (t == 0) {
@@ -423,32 +433,91 @@ __global__ void k_adapt_examples(const float4 *__restrict__ nodes, int n_branch,
     const float s = __fdiv_rn(fx, 585.0f);
     const float inv = __frcp_rn(d);
     const int leaf = walk_tree(nodes + (size_t)t * n_branch, depth, D, C, W, H, s, x, y, d, inv);
-    const uint32_t L = (uint32_t)(t * leaves_per_tree + leaf);
-    ex_leaf[e] = L;
-    ex_rank[e] = atomicAdd(&frame_cnt[L], 1u);
+    ex_leaf[e] = (uint16_t)leaf;
+    // one atomic for a warp's examples of a leaf: neighbours often share it,
+    // and those of a full leaf would queue at its count
+    const unsigned same = __match_any_sync(live, leaf);
+    if ((threadIdx.x & 31) == __ffs(same) - 1)
+        atomicAdd(&frame_cnt[t * leaves_per_tree + leaf], (uint32_t)__popc(same));
 }
 
-// Segments: a leaf's (first entry, length) in the list; tree t's segments lie
-// in [t P, t P + used[t]).
-__global__ void k_adapt_segments(const uint32_t *__restrict__ frame_cnt, int L, int leaves_per_tree, int P,
-                                 uint2 *__restrict__ seg, uint32_t *__restrict__ used) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= L) return;
-    const uint32_t n = frame_cnt[l];
-    if (!n) return;
-    const int t = l / leaves_per_tree;
-    seg[l] = make_uint2((uint32_t)t * (uint32_t)P + atomicAdd(&used[t], n), n);
+// Segments: each count of a tree's leaves becomes where the leaf's segment
+// starts, the sum of the counts before it (tree t's segments lie in [t P, (t +
+// 1) P)), and is added to the leaf's reservoir count.  A cluster of blocks per
+// tree (one block up to 4,096 leaves), so that any tree takes one step of it.
+__global__ void __launch_bounds__(EX_SCAN_THREADS)
+    k_adapt_segments(uint32_t *__restrict__ frame_cnt, uint32_t *__restrict__ res_count, int leaves_per_tree, int P) {
+    __shared__ uint32_t sums[32], total;
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, rank = blockIdx.x, t = blockIdx.y;
+    const int per = EX_SCAN_EACH * blockDim.x;  // a block's leaves
+    const int l0 = rank * per + EX_SCAN_EACH * tid, end = leaves_per_tree;
+    uint32_t *cnt = frame_cnt + (size_t)t * leaves_per_tree, *res = res_count + (size_t)t * leaves_per_tree;
+    uint32_t c[EX_SCAN_EACH], before[EX_SCAN_EACH], mine = 0;
+#pragma unroll
+    for (int k = 0; k < EX_SCAN_EACH; ++k) {
+        c[k] = l0 + k < end ? cnt[l0 + k] : 0;
+        before[k] = l0 + k < end ? res[l0 + k] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < EX_SCAN_EACH; ++k) mine += c[k];
+    auto sum_to = [&](uint32_t v) {  // over the warp's lanes up to this one
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += x;
+        }
+        return v;
+    };
+    const uint32_t upto = sum_to(mine);
+    if (lane == 31) sums[w] = upto;
+    __syncthreads();
+    if (w == 0) {
+        const uint32_t v = lane < (int)blockDim.x / 32 ? sums[lane] : 0, all = sum_to(v);
+        sums[lane] = all - v;
+        if (lane == 31) total = all;
+    }
+    __syncthreads();
+    if (gridDim.x > 1) cluster.sync();
+    uint32_t at = (uint32_t)t * (uint32_t)P + sums[w] + upto - mine;
+    // the blocks before, a lane each (at most eight blocks)
+    at += __reduce_add_sync(0xffffffffu, lane < rank ? *cluster.map_shared_rank(&total, lane) : 0u);
+#pragma unroll
+    for (int k = 0; k < EX_SCAN_EACH; ++k)
+        if (l0 + k < end) {
+            cnt[l0 + k] = at;
+            if (c[k]) res[l0 + k] = before[k] + c[k];
+            at += c[k];
+        }
+    if (gridDim.x > 1) cluster.sync();  // no block leaves while another may still read its sum
 }
 
-__global__ void k_adapt_scatter(const uint32_t *__restrict__ ex_leaf, const uint32_t *__restrict__ ex_rank, int P,
-                                const uint2 *__restrict__ seg, uint32_t *__restrict__ list) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= P) return;
-    const size_t e = (size_t)blockIdx.y * P + g;
-    const uint32_t L = ex_leaf[e];
-    if (L == 0xFFFFFFFFu) return;
-    list[seg[L].x + ex_rank[e]] = (uint32_t)g;
+__global__ void k_adapt_scatter(const uint16_t *__restrict__ ex_leaf, int P, int leaves_per_tree,
+                                uint32_t *__restrict__ frame_cnt, uint32_t *__restrict__ list) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y, lane = threadIdx.x & 31;
+    const uint32_t leaf = g < P ? ex_leaf[(size_t)t * P + g] : kNoLeaf;
+    const unsigned same = __match_any_sync(0xffffffffu, leaf);
+    const int first = __ffs(same) - 1;
+    uint32_t at = 0;
+    if (lane == first && leaf != kNoLeaf) at = atomicAdd(&frame_cnt[t * leaves_per_tree + leaf], (uint32_t)__popc(same));
+    at = __shfl_sync(0xffffffffu, at, first);
+    if (leaf != kNoLeaf) list[at + __popc(same & ((1u << lane) - 1u))] = (uint32_t)g;
 }
+
+// What a step reads of the list once it is filled.
+struct ExList {
+    const uint32_t *entry;  // grid pixels, tree t's from t P
+    const uint32_t *ends;   // [L] end of the leaf's segment
+    int P, leaves_per_tree;
+    // entries [t P, end(t)) are in use
+    __device__ uint32_t end(int t) const { return ends[(t + 1) * leaves_per_tree - 1]; }
+    // (first entry, length) of leaf `leaf` of tree t
+    __device__ uint2 segment(int t, uint32_t leaf) const {
+        const uint32_t l = (uint32_t)(t * leaves_per_tree) + leaf;
+        const uint32_t first = leaf ? ends[l - 1] : (uint32_t)t * (uint32_t)P;
+        return make_uint2(first, ends[l] - first);
+    }
+};
 
 __device__ __forceinline__ int64_t reservoir_slot(uint32_t L, uint32_t c, int kappa, uint32_t k0,
                                                   uint32_t k1) {
@@ -458,7 +527,6 @@ __device__ __forceinline__ int64_t reservoir_slot(uint32_t L, uint32_t c, int ka
     return j < (uint64_t)kappa ? (int64_t)j : -1;
 }
 
-constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 // Runs f(first, last) on every thread of a block for the part of its segment
 // [sg.x, sg.x + sg.y) in each tile of the block's segments (load(q0, n) stages
 // entries q0 .. q0 + n in shared memory); threads without a segment have
@@ -504,19 +572,18 @@ __device__ __forceinline__ void wide_segments(uint2 sg, uint32_t live, F f) {
     if (b.y >= EX_WIDE && b.x != a.x) f(b);
 }
 
-// slot[k]: the slot of entry k of the list, or kNoSlot.
-__global__ void __launch_bounds__(EX_THREADS) k_adapt_slots(
-    const uint32_t *__restrict__ ex_leaf, const uint32_t *__restrict__ list, int P, const uint2 *__restrict__ seg,
-    const uint32_t *__restrict__ used, const uint32_t *__restrict__ res_count, int kappa, uint32_t k0, uint32_t k1,
-    uint32_t *__restrict__ slot) {
+// slot[r]: the slot of entry r of the list, or kNoSlot.
+__global__ void __launch_bounds__(EX_THREADS) k_adapt_slots(const uint16_t *__restrict__ ex_leaf, ExList list,
+                                                            const uint32_t *__restrict__ res_count, int kappa,
+                                                            uint32_t k0, uint32_t k1, uint16_t *__restrict__ slot) {
     __shared__ uint32_t s_g[EX_TILE], table[EX_TABLE], chunk[EX_THREADS], sum[EX_THREADS / 32];
-    const uint32_t r0 = blockIdx.x * EX_THREADS, r = r0 + threadIdx.x, t = blockIdx.y, end = used[t];
+    const int P = list.P, t = blockIdx.y;
+    const uint32_t r0 = (uint32_t)t * P + blockIdx.x * EX_THREADS, r = r0 + threadIdx.x, end = list.end(t);
     if (r0 >= end) return;
     const bool on = r < end;
-    const size_t k = (size_t)t * P + r;
-    const uint32_t g = on ? list[k] : 0;
-    const uint32_t L = on ? ex_leaf[(size_t)t * P + g] : 0;
-    const uint2 sg = on ? seg[L] : make_uint2(0, 0);
+    const uint32_t g = on ? list.entry[r] : 0;
+    const uint32_t leaf = on ? ex_leaf[(size_t)t * P + g] : 0;
+    const uint2 sg = on ? list.segment(t, leaf) : make_uint2(0, 0);
     uint32_t rank = 0;
     wide_segments(sg, min(end - r0, (uint32_t)EX_THREADS), [&](uint2 e) {
         for (uint32_t w0 = 0; w0 < (uint32_t)P; w0 += EX_TABLE * 32) {  // the set bits below g
@@ -524,7 +591,7 @@ __global__ void __launch_bounds__(EX_THREADS) k_adapt_slots(
             for (uint32_t i = threadIdx.x; i < words; i += EX_THREADS) table[i] = 0;
             __syncthreads();
             for (uint32_t q = threadIdx.x; q < e.y; q += EX_THREADS) {
-                const uint32_t d = list[e.x + q] - w0;
+                const uint32_t d = list.entry[e.x + q] - w0;
                 if (d < words * 32) atomicOr(&table[d >> 5], 1u << (d & 31));
             }
             __syncthreads();
@@ -561,39 +628,40 @@ __global__ void __launch_bounds__(EX_THREADS) k_adapt_slots(
     });
     segment_tiles(
         sg.y < EX_WIDE ? sg : make_uint2(0, 0), [&](uint32_t q0, uint32_t n) {
-            for (uint32_t q = threadIdx.x; q < n; q += EX_THREADS) s_g[q] = list[q0 + q];
+            for (uint32_t q = threadIdx.x; q < n; q += EX_THREADS) s_g[q] = list.entry[q0 + q];
         },
         [&](uint32_t first, uint32_t last) {
 #pragma unroll 8
             for (uint32_t q = first; q < last; ++q) rank += s_g[q] < g;
         });
     if (!on) return;
-    const int64_t s = reservoir_slot(L, res_count[L] + rank, kappa, k0, k1);
-    slot[k] = s < 0 ? kNoSlot : (uint32_t)s;
+    const uint32_t L = (uint32_t)(t * list.leaves_per_tree) + leaf;
+    const int64_t s = reservoir_slot(L, res_count[L] - sg.y + rank, kappa, k0, k1);
+    slot[r] = s < 0 ? kNoSlot : (uint16_t)s;
 }
 
-__global__ void __launch_bounds__(EX_THREADS) k_adapt_insert(
-    const uint32_t *__restrict__ ex_leaf, const uint32_t *__restrict__ slot, const uint32_t *__restrict__ list,
-    const float4 *__restrict__ ex_pt, int P, const uint2 *__restrict__ seg, const uint32_t *__restrict__ used,
-    const uint32_t *__restrict__ res_count, int kappa, float4 *__restrict__ res) {
+__global__ void __launch_bounds__(EX_THREADS) k_adapt_insert(const uint16_t *__restrict__ ex_leaf,
+                                                             const uint16_t *__restrict__ slot, ExList list,
+                                                             const float4 *__restrict__ ex_pt,
+                                                             const uint32_t *__restrict__ res_count, int kappa,
+                                                             float4 *__restrict__ res) {
     __shared__ uint2 s_gs[EX_TILE];
     __shared__ uint32_t table[EX_TABLE];
-    const uint32_t r0 = blockIdx.x * EX_THREADS, r = r0 + threadIdx.x, t = blockIdx.y, end = used[t];
+    const int P = list.P, t = blockIdx.y;
+    const uint32_t r0 = (uint32_t)t * P + blockIdx.x * EX_THREADS, r = r0 + threadIdx.x, end = list.end(t);
     if (r0 >= end) return;
-    const size_t k = (size_t)t * P + r;
-    const uint32_t mine = r < end ? slot[k] : kNoSlot;
+    const uint32_t g = r < end ? list.entry[r] : 0, mine = r < end ? slot[r] : kNoSlot;
+    const uint32_t leaf = r < end ? ex_leaf[(size_t)t * P + g] : 0, L = (uint32_t)(t * list.leaves_per_tree) + leaf;
     const bool on = mine != kNoSlot;
-    const uint32_t g = r < end ? list[k] : 0;
-    const uint32_t L = r < end ? ex_leaf[(size_t)t * P + g] : 0;
-    uint2 sg = r < end ? seg[L] : make_uint2(0, 0);
-    if (sg.y && res_count[L] + sg.y <= (uint32_t)kappa) sg = make_uint2(0, 0);  // every example has a slot of its own
+    uint2 sg = r < end ? list.segment(t, leaf) : make_uint2(0, 0);
+    if (sg.y && res_count[L] <= (uint32_t)kappa) sg = make_uint2(0, 0);  // every example has a slot of its own
     bool later = false;
     wide_segments(sg, min(end - r0, (uint32_t)EX_THREADS), [&](uint2 e) {
         for (int i = threadIdx.x; i < kappa; i += EX_THREADS) table[i] = 0;
         __syncthreads();
         for (uint32_t q = threadIdx.x; q < e.y; q += EX_THREADS) {
             const uint32_t s = slot[e.x + q];
-            if (s != kNoSlot) atomicMax(&table[s], list[e.x + q] + 1);
+            if (s != kNoSlot) atomicMax(&table[s], list.entry[e.x + q] + 1);
         }
         __syncthreads();
         if (on && sg.x == e.x && sg.y) later = table[mine] != g + 1;
@@ -601,24 +669,14 @@ __global__ void __launch_bounds__(EX_THREADS) k_adapt_insert(
     });
     segment_tiles(
         on && sg.y < EX_WIDE ? sg : make_uint2(0, 0), [&](uint32_t q0, uint32_t n) {
-            for (uint32_t q = threadIdx.x; q < n; q += EX_THREADS) s_gs[q] = make_uint2(list[q0 + q], slot[q0 + q]);
+            for (uint32_t q = threadIdx.x; q < n; q += EX_THREADS)
+                s_gs[q] = make_uint2(list.entry[q0 + q], slot[q0 + q]);
         },
         [&](uint32_t first, uint32_t last) {
 #pragma unroll 8
             for (uint32_t q = first; q < last; ++q) later |= s_gs[q].x > g && s_gs[q].y == mine;
         });
     if (on && !later) res[(size_t)L * kappa + mine] = ex_pt[g];
-}
-
-__global__ void k_adapt_commit(uint32_t *__restrict__ res_count, uint32_t *__restrict__ frame_cnt,
-                               int L) {
-    const int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= L) return;
-    const uint32_t n = frame_cnt[l];
-    if (n) {
-        res_count[l] += n;
-        frame_cnt[l] = 0;
-    }
 }
 
 rl_status adapt_frame(rl_forest *f, const float *depth, const uint8_t *rgb,
@@ -632,43 +690,46 @@ rl_status adapt_frame(rl_forest *f, const float *depth, const uint8_t *rgb,
     if (f->ex_capacity < P) {
         arena_free(f->ctx, f->ex_leaf);
         arena_free(f->ctx, f->ex_pt);
-        arena_free(f->ctx, f->ex_rank);
         arena_free(f->ctx, f->ex_list);
-        arena_free(f->ctx, f->ex_seg);
         f->ex_leaf = nullptr;
         f->ex_pt = nullptr;
-        f->ex_rank = nullptr;
         f->ex_list = nullptr;
-        f->ex_seg = nullptr;
         f->ex_capacity = 0;
-        RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees, &f->ex_leaf));
+        RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees * 2, &f->ex_leaf));
         RL_TRY(alloc_n(f->ctx, (uint64_t)P, &f->ex_pt));
-        RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees, &f->ex_rank));
-        RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees + EX_MAX_TREES, &f->ex_list));  // then the entries in use per tree
-        RL_TRY(alloc_n(f->ctx, (uint64_t)f->n_leaves, &f->ex_seg));
+        RL_TRY(alloc_n(f->ctx, (uint64_t)P * p.n_trees, &f->ex_list));
         f->ex_capacity = P;
     }
     Pose12 pose;
     for (int i = 0; i < 12; ++i) pose.m[i] = T[i];
     const uint32_t k0 = (uint32_t)f->seed, k1 = (uint32_t)(f->seed >> 32);
-    uint32_t *used = f->ex_list + (size_t)P * p.n_trees;
     const dim3 grid((P + EX_THREADS - 1) / EX_THREADS, p.n_trees);
+    const ExList list{f->ex_list, f->frame_cnt, P, f->leaves_per_tree};
+    RL_CK(cudaMemsetAsync(f->frame_cnt, 0, sizeof(uint32_t) * f->n_leaves, s));
     k_adapt_examples<<<grid, EX_THREADS, 0, s>>>(f->nodes, f->n_branch, p.depth, f->leaves_per_tree, depth, rgb, K->width,
                                           K->height, K->fx, K->fy, K->cx, K->cy, pose, gw, gh, st, o, f->ex_leaf,
-                                          f->ex_rank, f->ex_pt, f->frame_cnt, used);
+                                          f->ex_pt, f->frame_cnt);
     RL_LAUNCH_CK();
-    k_adapt_segments<<<(f->n_leaves + 255) / 256, 256, 0, s>>>(f->frame_cnt, f->n_leaves, f->leaves_per_tree, P,
-                                                               f->ex_seg, used);
+    const int groups = (f->leaves_per_tree + EX_SCAN_EACH - 1) / EX_SCAN_EACH;  // leaves of a thread
+    const int scan = std::min(EX_SCAN_THREADS, (groups + 31) / 32 * 32);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((groups + scan - 1) / scan, p.n_trees);
+    cfg.blockDim = dim3(scan);
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = cfg.gridDim.x;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    RL_CK(cudaLaunchKernelEx(&cfg, k_adapt_segments, f->frame_cnt, f->res_count, f->leaves_per_tree, P));
+    k_adapt_scatter<<<grid, EX_THREADS, 0, s>>>(f->ex_leaf, P, f->leaves_per_tree, f->frame_cnt, f->ex_list);
     RL_LAUNCH_CK();
-    k_adapt_scatter<<<grid, EX_THREADS, 0, s>>>(f->ex_leaf, f->ex_rank, P, f->ex_seg, f->ex_list);
+    uint16_t *slot = f->ex_leaf + (size_t)P * p.n_trees;
+    k_adapt_slots<<<grid, EX_THREADS, 0, s>>>(f->ex_leaf, list, f->res_count, p.kappa, k0, k1, slot);
     RL_LAUNCH_CK();
-    k_adapt_slots<<<grid, EX_THREADS, 0, s>>>(f->ex_leaf, f->ex_list, P, f->ex_seg, used, f->res_count, p.kappa, k0, k1,
-                                       f->ex_rank);
-    RL_LAUNCH_CK();
-    k_adapt_insert<<<grid, EX_THREADS, 0, s>>>(f->ex_leaf, f->ex_rank, f->ex_list, f->ex_pt, P, f->ex_seg, used,
-                                        f->res_count, p.kappa, f->res);
-    RL_LAUNCH_CK();
-    k_adapt_commit<<<(f->n_leaves + 255) / 256, 256, 0, s>>>(f->res_count, f->frame_cnt, f->n_leaves);
+    k_adapt_insert<<<grid, EX_THREADS, 0, s>>>(f->ex_leaf, slot, list, f->ex_pt, f->res_count, p.kappa, f->res);
     RL_LAUNCH_CK();
     return RL_OK;
 }

@@ -99,12 +99,10 @@ struct rl_forest {
     float4 *mU = nullptr;           // [L][m_max][2]: U00 U01 U02 U11 | U12 U22 0 0
     int32_t *msize = nullptr;
     // adaptation scratch
-    uint32_t *ex_leaf = nullptr;    // [T][grid pixels]
+    uint16_t *ex_leaf = nullptr;    // [T][grid pixels] leaf in the tree; then as many slots by list entry
     float4 *ex_pt = nullptr;        // [grid pixels]
-    uint32_t *ex_rank = nullptr;    // [T][grid pixels] arrival number; then the slots by list entry
-    uint32_t *ex_list = nullptr;    // [T][grid pixels] examples by leaf; then [16] entries used per tree
-    uint2 *ex_seg = nullptr;        // [L] (first entry, length) of the leaf's examples in ex_list
-    uint32_t *frame_cnt = nullptr;  // [L]
+    uint32_t *ex_list = nullptr;    // [T][grid pixels] examples by leaf
+    uint32_t *frame_cnt = nullptr;  // [L] arrivals of the frame; then where the leaf's part of ex_list ends
     int ex_capacity = 0;
     float *stage_depth = nullptr;
     uint8_t *stage_rgb = nullptr;

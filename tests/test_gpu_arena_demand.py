@@ -1,5 +1,8 @@
 """What the library asks of the caller's arena does not grow: programs size it
 once, some to the byte."""
+import dataclasses
+
+import numpy as np
 import pytest
 
 from synth import workloads
@@ -41,4 +44,26 @@ def test_relocaliser(rg, case):
     rel.close()
     f.close()
     scene.close()
+    ctx.close()
+
+
+@pytest.mark.parametrize("trees,depth", [(1, 1), (5, 6), (3, 15), (16, 4)])
+def test_adaptation(rg, trees, depth):
+    """Two words per example and tree, and a point per grid pixel, whatever
+    the number of leaves; again only for a larger frame."""
+    import torch
+    w = workloads.small_case()
+    ctx = rg.Context(0, arena_bytes=1 << 28)
+    f = rg.Forest.random(ctx, dict(w.forest, n_trees=trees, depth=depth, m_max=2, kappa=8, grid_step=4), 3)
+    start = ctx.usage()[0]
+    most = 0
+    for size in ((4, 4), (96, 72), (160, 121), (95, 70), (640, 480)):
+        K = dataclasses.replace(w.K, width=size[0], height=size[1])
+        d = torch.full((size[1], size[0]), 2.0, device="cuda")
+        f.adapt(d, torch.zeros(size[1], size[0], 3, dtype=torch.uint8, device="cuda"), K, np.eye(4))
+        most = max(most, -(-size[0] // 4) * -(-size[1] // 4))
+        asked = sum(-(-b // 256) * 256 for b in (4 * most * trees, 16 * most, 4 * most * trees))
+        assert ctx.usage()[0] - start <= asked, size
+    assert f.export()["res_count"].sum() == trees * (1 + 24 * 18 + 40 * 31 + 24 * 18 + 160 * 120)
+    f.close()
     ctx.close()
