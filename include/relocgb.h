@@ -377,8 +377,12 @@ rl_status rl_reloc_debug(rl_reloc *r, int32_t q, double *hyp_pose /* n_hyp*12 */
  * (every kernel computes the same values in the same order for each of
  * them).  Defaults: {16, 128, 128, 256, 8}. */
 typedef struct {
-    int32_t hypgen_warps;     /* warps (slots) per block of generation: 2, 4, 8 or 16 */
-    int32_t energy_threads;   /* at most this many hypotheses per block of Eq. 5: 32, 64, 128 or 256 */
+    int32_t hypgen_warps;     /* warps per block of generation, a slot each: 2, 4, 8 or 16.  In a
+                               * call of few slots a team of up to 16 warps serves each, and a
+                               * block holds at least a team. */
+    int32_t energy_threads;   /* at most this many hypotheses per block of Eq. 5: 32, 64, 128 or 256.
+                               * A launch whose blocks hold all hypotheses of a frame and leave the
+                               * GPU idle takes up to 256 threads, several per hypothesis. */
     int32_t leaves_threads;   /* pixels per block of the forest walk: 64, 128, 256 or 512 */
     int32_t mask_threads;     /* pixels per block of the colour-check masks: 64, 128 or 256 */
     int32_t streams;          /* sub-batches of a call run concurrently on this many streams: 1, 2,

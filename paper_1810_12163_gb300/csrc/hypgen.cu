@@ -10,6 +10,8 @@
 // slot, is exactly reproducible.
 #include <limits.h>
 
+#include <algorithm>
+
 #include "hypgen_dev.cuh"
 #include "kernels.h"
 
@@ -585,8 +587,11 @@ rl_status launch_hypgen(const Frame *frames, const uint16_t *leaves, const uint1
     // the bitmap path needs the frame's bitmap in shared memory
     const size_t bits_smem = (size_t)(hw_max / 32 + 1) * 4;
     const bool bits = prec && pbits && bits_smem <= kHypBitsSmemMax;
+    // a team is warps of one block: the blocks of a call with few slots are as
+    // large as its teams, whatever suits the batches that `warps` was tuned on
     int team = 1;
-    while (2 * team <= warps && (int64_t)p.n_hyp * n_active * 2 * team <= (int64_t)sm_count * 32) team *= 2;
+    while (2 * team <= 16 && (int64_t)p.n_hyp * n_active * 2 * team <= (int64_t)sm_count * 32) team *= 2;
+    warps = std::max(warps, team);
     HypArgs a{frames, leaves, mcount, prec, pcm, hw_max, mv, p, hyp_pose, hyp_iter, work, bits ? pbits : nullptr, team};
     if (p.redraw)
         launch_hypgen_path<1>(a, warps, n, bits_smem, s);

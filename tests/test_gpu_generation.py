@@ -36,3 +36,19 @@ def test_a_team_stops_at_its_mates_success(rg, model, n_hyp, redraw):  # noqa: F
             found += [it for it in got if it >= 0]
         rel.close()
     assert max(found) > 64  # beyond the first warp's first group
+
+
+@pytest.mark.parametrize("warps", [2, 4, 8, 16])
+def test_block_size_does_not_change_a_small_call(rg, model, warps):  # noqa: F811
+    """Blocks tuned on batches: in a call of few slots they grow to its teams,
+    and in one of many slots hold this many slots."""
+    w, f, scene, nodes, modes, queries = model
+    for n_hyp, k_top in ((3, 10), (200, 10), (200, 40), (4096, 10)):  # colour masks and pixel records
+        p = dict(w.ransac, n_trees_used=5, k_top=k_top, n_hyp=n_hyp, n_cull=min(n_hyp, 24), max_iter=700)
+        rel = rg.Relocaliser(f, scene, p, w.width, w.height, 1)
+        rel.set_tuning(dict(rel.tuning, hypgen_warps=warps))
+        d, c, _, seed = queries[1]
+        rel.relocalise(d, c, w.K, seed)
+        np.testing.assert_array_equal(rel.debug(0)["hyp_iter"],
+                                      oracle_iterations(p, d, c, w, w.K, nodes, modes, seed))
+        rel.close()
