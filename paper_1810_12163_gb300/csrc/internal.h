@@ -409,10 +409,10 @@ rl_status update_modes(rl_forest *f, int64_t begin, int64_t count, cudaStream_t 
 rl_status reset_leaves(rl_forest *f, cudaStream_t s);
 ModeView mode_view(const rl_forest *f);
 // The launch sequence of n frames whose query state is q (r->q, or a slice
-// of it for a sub-batch: query_slice); n_active: frames at work on the GPU
-// at once, the call's other sub-batches included (it shapes launches, never
-// results).
-rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, int level, cudaStream_t s);
+// of it for a sub-batch: query_slice) in a call of n_call frames, its other
+// sub-batches included, of which about n_active are expected at work on the
+// GPU at once, the others being empty (both shape launches, never results).
+rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_call, int n_active, int level, cudaStream_t s);
 // q for the frames b0, b0 + 1, ... of r's batch.
 QueryState query_slice(const rl_reloc *r, int b0);
 // Batch of n frames whose descriptors (device pointers, per-frame sizes and

@@ -59,7 +59,7 @@ struct LmArgs {
     int maxm;                  // |M(u)| bound: trees x min(k_top, m_max)
     int maxm_pad;              // maxm rounded up to an odd count (shared-memory rows)
     uint32_t wait_limit;       // probes of a wait for a staged tile before it gives up
-    int n_active;              // frames at work on the GPU at once (shapes the launch, never the result)
+    int n_call, n_active;      // frames of the call, and those expected at work (they shape the launch, never the result)
     int sm_count;
     LmResident resident;       // clusters that the GPU holds at once, by shape
 };

@@ -1039,7 +1039,7 @@ rl_status launch_lm_cluster(const LmArgs &a, int n, cudaStream_t s) {
     const bool first = a.n_pix <= 2 * a.p.eta;  // round r refines on eta * (r + 2) pixels
     const bool split = a.p.maxm >= LMC_SPLIT_MODES &&
                        lmc_layout(a.p.mpad, a.p.use_cov, LMC_STAGES_SUB).total <= kLmClusterSmemMax;
-    const int sets = split ? lm_sets(a.resident, first, a.n_active) : 1;
+    const int sets = split ? lm_sets(a.resident, first, a.n_call, a.n_active < a.n_call) : 1;
     if (first) {
         if (sets == 4) return launch_lm_shape<LMC_RANKS_FIRST, 4>(a, n, s);
         if (sets == 2) return launch_lm_shape<LMC_RANKS_FIRST, 2>(a, n, s);

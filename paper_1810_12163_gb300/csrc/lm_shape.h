@@ -20,10 +20,18 @@ struct LmResident {
 // cluster that may wait starts as soon as the shortest of the others ends:
 // there a call of 8 frames of 640x480 takes 3.90 ms (4.32 with half the
 // sets), one of 16 frames 5.33 (5.60 with one set).
-inline int lm_sets(const LmResident &r, bool first_round, int frames) {
-    auto fits = [frames](int held) { return held > 0 && frames <= held + 1; };
-    if (first_round) return fits(r.first4) ? 4 : fits(r.first2) ? 2 : 1;
-    return fits(r.later2) ? 2 : 1;
+//
+// sparse: a later level of a cascade, where most frames are empty, but all may
+// be at work.  Clusters of 16 are then used up to two deep, of 8 up to three.
+// Cascades of 640x480 frames of which one in ten goes on, of 16, 32, 48 and 64
+// frames: 2.08, 2.35, 2.78 and 3.17 ms (2.24, 2.52, 2.88 and 3.21 with sets
+// for all frames alike, 2.08, 2.31, 2.79 and 3.08 with sets for a quarter);
+// with all going on 7.9, 10.4, 13.4 and 16.8 ms (7.5, 10.4, 12.8 and 16.9;
+// 7.9, 12.7, 13.3 and 18.4).
+inline int lm_sets(const LmResident &r, bool first_round, int frames, bool sparse) {
+    auto fits = [&](int held, int deep) { return held > 0 && frames <= (sparse ? deep : 1) * (held + 1); };
+    if (first_round) return fits(r.first4, 2) ? 4 : fits(r.first2, 3) ? 2 : 1;
+    return fits(r.later2, 2) ? 2 : 1;
 }
 
 }  // namespace rl

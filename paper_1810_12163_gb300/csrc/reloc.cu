@@ -175,7 +175,7 @@ static uint2 *packed_frames(const QueryState &q, int n_trees, int n, size_t hw) 
     return at + sizeof(uint2) * hw * n <= end ? (uint2 *)at : nullptr;
 }
 
-rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, int level, cudaStream_t s) {
+rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_call, int n_active, int level, cudaStream_t s) {
     rl_forest *f = r->forest;
     RParams p = r->rp;
     p.level = level;
@@ -260,8 +260,8 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_active, 
         const int n_pix = p.eta * (round + 2);
         const bool lm = p.pose_update && p.lm_max_iter > 0;
         if (lm) {
-            LmArgs la{q, q.leaves, hw_max, mv, p, n_pix, work, maxm, maxm | 1, r->lm_wait_limit, n_active, f->ctx->sm_count,
-                      r->lm_resident};
+            LmArgs la{q, q.leaves, hw_max, mv, p, n_pix, work, maxm, maxm | 1, r->lm_wait_limit, n_call, n_active,
+                      f->ctx->sm_count, r->lm_resident};
             PROF(K_LM);
             RL_TRY(launch_lm(la, n, s));
         }
@@ -395,7 +395,7 @@ static rl_status run_relocalise_parts(rl_reloc *r, int n, int level, cudaStream_
     // replayed graph, walk the unscaled nodes)
     RL_TRY(launch_scale_nodes(r->forest, r->rp.n_trees, r->nodes_s, r->host_frames[0].fx, s));
     const int parts = r->prof.on ? 1 : std::max(1, std::min(r->tune.streams, n / kMinPart));
-    if (parts <= 1) return run_relocalise(r, r->q, n, n, level, s);
+    if (parts <= 1) return run_relocalise(r, r->q, n, n, n, level, s);
     for (int i = 0; i < parts - 1; ++i) {
         if (!r->side[i]) RL_CK(cudaStreamCreateWithFlags(&r->side[i], cudaStreamNonBlocking));
         if (!r->join_ev[i]) RL_CK(cudaEventCreateWithFlags(&r->join_ev[i], cudaEventDisableTiming));
@@ -407,7 +407,7 @@ static rl_status run_relocalise_parts(rl_reloc *r, int n, int level, cudaStream_
         const int nb = n / parts + (i < n % parts ? 1 : 0);
         cudaStream_t si = i == 0 ? s : r->side[i - 1];
         if (i > 0) RL_CK(cudaStreamWaitEvent(si, r->fork_ev, 0));
-        RL_TRY(run_relocalise(r, query_slice(r, b0), nb, n, level, si));
+        RL_TRY(run_relocalise(r, query_slice(r, b0), nb, n, n, level, si));
         if (i > 0) RL_CK(cudaEventRecord(r->join_ev[i - 1], si));
         b0 += nb;
     }
@@ -859,7 +859,8 @@ static CascadeOut cascade_out_slice(const CascadeOut &o, int b0) {
 }
 
 // A later level shapes its launches for a quarter of the call's frames: most
-// were accepted before and are empty frames there.
+// were accepted before and are empty frames there.  (LM clusters, which can
+// queue, also look at what happens when none was: lm_sets.)
 constexpr int kLaterLevelShare = 4;
 
 // All levels for the nb frames b0, b0 + 1, ... of the call of n frames.
@@ -878,7 +879,7 @@ static rl_status cascade_enqueue_part(rl_cascade *c, int b0, int nb, int n, cuda
                                                  r->stage_rgb + (size_t)b0 * hw * 3, hw);
             RL_LAUNCH_CK();
         }
-        RL_TRY(run_relocalise(r, q, nb, l == 0 ? n : std::max(1, n / kLaterLevelShare), l, s));
+        RL_TRY(run_relocalise(r, q, nb, n, l == 0 ? n : std::max(1, n / kLaterLevelShare), l, s));
         LaterFrames later{};
         for (int k = l + 1; k < L && later.n < 8; ++k) later.f[later.n++] = c->levels[k]->q.frames + b0;
         const float tau = l < L - 1 ? (float)c->thresholds[l] : INFINITY;
