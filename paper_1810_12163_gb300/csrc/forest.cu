@@ -386,8 +386,9 @@ rl_status launch_scale_nodes(const rl_forest *f, int n_trees, float4 *out, float
 // atomic per example, whose leaves are then full).  With a record per segment
 // and words of their own for arrival numbers and slots, 4 bytes more per
 // example and 8 per leaf, the calls took 48, 47 and 59 us.  Every entry
-// against every other in long segments too: 18 us slots, 27 us insert.  A thread per pixel walking all trees, ranks from all pairs of
-// pixels and the slot of every later example drawn again: 620 us.
+// against every other in long segments too: 18 us slots, 27 us insert.  A
+// thread per pixel walking all trees, ranks from all pairs of pixels and the
+// slot of every later example drawn again: 620 us.
 // ---------------------------------------------------------------------------
 constexpr int EX_THREADS = 128, EX_TILE = 1024;
 constexpr int EX_WIDE = 256;      // entries from which a segment gets a table

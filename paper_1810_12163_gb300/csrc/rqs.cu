@@ -43,12 +43,13 @@
 // each (a warp per cluster took three FP64 instructions a member, a thread
 // per cluster 27).
 // Thousands of cycles of a leaf of more than 600 points, training / online
-// (where clusters are larger), before the means were summed in parallel: sort
-// 19 / 18, densities 49 / 61, parents 60 / 71, FP64 densities 13 / 8, FP64
-// comparisons 20 / 10, members 5 / 10, cluster sums 33 / 73, factors 11 / 10.
-// With the columns in groups of 32, every column of a group compared and a
-// warp per cluster it was 297 and 350 in all.  A cluster of four blocks on
-// each full leaf was slower: the full leaves fill the GPU.
+// (where clusters are larger), by clock stamps at the phases' barriers: sort
+// and boxes 22 / 19, densities 50 / 62, parents 62 / 71, FP64 densities 16 /
+// 10, FP64 comparisons 15 / 7, members 9 / 15, cluster sums 26 / 58, factors
+// 11 / 10.  With the columns in groups of 32, every column of a group compared
+// and a warp per cluster it was 297 and 350 in all.  A cluster of four blocks
+// on each full leaf was slower in training, where the full leaves fill the
+// GPU; online, where they do not, it was not tried.
 //
 // Measured on GB300: 10,240 leaves of 107 points on average, about 800 of
 // more than 600 (24 frames of 640x480, 5 trees of depth 11, capacity 1024):
@@ -270,14 +271,15 @@ __device__ __forceinline__ void rqs_row(const RqsPar &r, int i, RqsBest &o) {
     if (LEVEL != RQS_MARK) o = {-1, 0.f, INFINITY};
     for (int j = lane; j < r.n; j += 32)
         if (j != i && !(dist2f(p, r.pts[j]) > r.tau_hi)) rqs_candidate<LEVEL>(r, p, i, ri, ei, j, o);
-    if (LEVEL == RQS_MARK) return;
+    if constexpr (LEVEL != RQS_MARK) {
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int oj = __shfl_xor_sync(0xffffffffu, o.j, off);
-        const float od = __shfl_xor_sync(0xffffffffu, o.d2, off);
-        if (oj >= 0 && rqs_nearer(r.pts, p, oj, od, o.j, o.d2)) {
-            o.j = oj;
-            o.d2 = od;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int oj = __shfl_xor_sync(0xffffffffu, o.j, off);
+            const float od = __shfl_xor_sync(0xffffffffu, o.d2, off);
+            if (oj >= 0 && rqs_nearer(r.pts, p, oj, od, o.j, o.d2)) {
+                o.j = oj;
+                o.d2 = od;
+            }
         }
     }
 }
@@ -452,8 +454,8 @@ __global__ void __launch_bounds__(RQS_THREADS, 2) k_rqs(RqsArgs a) {
             });
             if (k < n) {
                 const int i = sorted[2 * k];
-                // the bound of the file comment (4.8e-7, 0.8e-6) with 2% for
-                // its own rounding and second-order terms
+                // the bound of the file comment (8 u = 4.77e-7, 14 u + 2^-22 =
+                // 1.07e-6) with 2% for its own rounding and second-order terms
                 const float ln = fmaxf(logf((float)n / sum), 0.f) + 0.01f;
                 const float e = sum * (4.9e-7f * ln + 1.1e-6f) + 1e-12f * (float)n;
                 rho[i] = sum;
