@@ -346,10 +346,10 @@ __device__ __forceinline__ void role_barrier() {
 // AX owner warps share a stream: one that branches on the face's axis, as the
 // one-block kernel does, or one per axis, each with its nine sums and no
 // branch.  Alone on an SM (C = 8) the owners are the critical path and three
-// of them are faster (16 poses of 640x480: 423 us, 589 with one; the
-// one-block kernel 919); with four blocks per SM (C = 4) instructions count
-// and one that branches is (128 poses: 877 us, 1010 without the branch; the
-// one-block kernel 1315).  About 150 us of either are the 11 FP64 solves.
+// of them are faster (16 poses of 640x480: 423 us, 589 with one); with four
+// blocks per SM (C = 4) instructions count and one that branches is (128
+// poses: 877 us, 1010 without the branch).  About 150 us of either are the 11
+// FP64 solves.  icp_blocks has when each pays.
 template <int C, int AX>
 struct IcpTeam {
     static constexpr int threads = C == 8 ? 32 * (AX + 9) : ICP_THREADS;
@@ -547,16 +547,47 @@ __global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(IcpTeam<C, AX>::thre
 
 rl_status launch_icp(const IcpArgs &a, int n, cudaStream_t s) {
     if (n <= 0 || a.cap <= 0) return RL_OK;
-    // blocks of a cluster while the call's blocks fit the GPU (three and four per SM)
-    const int64_t poses = (int64_t)a.cap * a.n_active, room = a.sm_count;
-    if (poses * 8 <= 3 * room)
-        k_icp_team<8, 3><<<dim3(a.cap * 8, n), IcpTeam<8, 3>::threads, 0, s>>>(a);
-    else if (poses * 4 <= 4 * room)
-        k_icp_team<4, 1><<<dim3(a.cap * 4, n), IcpTeam<4, 1>::threads, 0, s>>>(a);
-    else
-        k_icp<<<dim3(a.cap, n), ICP_THREADS, 0, s>>>(a);
+    double cells = 0.0;  // pixels of an iteration, on average
+    int iters = 0;
+    for (int l = 0; l < a.ip.levels; ++l) {
+        cells += (double)a.max_hw / (a.ip.stride[l] * a.ip.stride[l]) * a.ip.iters[l];
+        iters += a.ip.iters[l];
+    }
+    switch (icp_blocks(a.resident, a.sm_count, (int64_t)a.cap * a.n_active, cells / iters)) {
+    case 8: k_icp_team<8, 3><<<dim3(a.cap * 8, n), IcpTeam<8, 3>::threads, 0, s>>>(a); break;
+    case 4: k_icp_team<4, 1><<<dim3(a.cap * 4, n), IcpTeam<4, 1>::threads, 0, s>>>(a); break;
+    default: k_icp<<<dim3(a.cap, n), ICP_THREADS, 0, s>>>(a);
+    }
     RL_LAUNCH_CK();
     return RL_OK;
+}
+
+template <int C, int AX>
+static int resident_teams() {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(IcpTeam<C, AX>::threads);
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_icp_team<C, AX>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
+}
+
+const IcpResident &icp_resident(rl_scene *sc) {
+    std::call_once(sc->icp_once, [sc] {
+        sc->icp_resident.of8 = resident_teams<8, 3>();
+        sc->icp_resident.of4 = resident_teams<4, 1>();
+    });
+    return sc->icp_resident;
 }
 
 }  // namespace rl

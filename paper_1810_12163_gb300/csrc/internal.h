@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/relocgb.h"
+#include "icp_shape.h"
 #include "lm_shape.h"
 
 // ---------------------------------------------------------------------------
@@ -124,6 +125,9 @@ struct rl_forest {
 struct rl_scene {
     rl_ctx *ctx = nullptr;
     double lo[3], hi[3];
+    // ICP clusters that the GPU holds at once, asked at the first use of ICP
+    std::once_flag icp_once;
+    rl::IcpResident icp_resident;
 };
 
 // Relocalisers using at most this many trees keep a 16-byte per-pixel record

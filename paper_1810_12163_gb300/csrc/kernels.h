@@ -118,8 +118,12 @@ struct IcpArgs {
     unsigned long long *work;  // profiling counters or null
     int n_active;              // frames at work on the GPU at once (shapes the launch, never the result)
     int sm_count;
+    int max_hw;                // pixels of the largest frame (as n_active)
+    IcpResident resident;      // clusters that the GPU holds at once
 };
 rl_status launch_icp(const IcpArgs &a, int n, cudaStream_t s);
+// The scene's device's (the current one).
+const IcpResident &icp_resident(rl_scene *sc);
 
 size_t energy_smem(int chunk, int maxm);
 rl_status launch_energy(const EnergyArgs &a, int max_count, int n, cudaStream_t s, int max_threads = 128);

@@ -307,6 +307,8 @@ rl_status run_relocalise(rl_reloc *r, const QueryState &q, int n, int n_call, in
         ia.work = work;
         ia.n_active = n_active;
         ia.sm_count = f->ctx->sm_count;
+        ia.max_hw = hw_max;
+        ia.resident = icp_resident(r->scene);
         PROF(K_ICP);
         RL_TRY(launch_icp(ia, n, s));
     }
@@ -607,7 +609,10 @@ extern "C" rl_status rl_reloc_create(rl_forest *f, rl_scene *scene, const rl_ran
     rp.rank = p->rank; rp.halve_to_one = p->halve_to_one; rp.level = 0;
     rp.icp = p->icp;
     rp.redraw = p->redraw;
-    if (p->icp) rp.icp_p = icp_device_params(p->icp_p);
+    if (p->icp) {
+        rp.icp_p = icp_device_params(p->icp_p);
+        icp_resident(scene);  // asked here, before any stream capture
+    }
     rp.max_rounds = rounds_for(p->n_cull, p->k_out, p->halve_to_one);
     // rows of whole 16-pixel tiles: the LM kernel stages tiles with bulk copies
     rp.max_pix = (p->eta * (rp.max_rounds + 1) + 15) / 16 * 16;
@@ -1394,6 +1399,8 @@ extern "C" rl_status rl_icp_poses(rl_scene *sc, const float *depth, const rl_int
         ia.ip = icp_device_params(*ip);
         ia.n_active = 1;
         ia.sm_count = ctx->sm_count;
+        ia.max_hw = npx;
+        ia.resident = icp_resident(sc);
         st = launch_icp(ia, 1, s);
     }
     if (st == RL_OK && (cudaMemcpyAsync(p12.data(), pd, p12.size() * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
