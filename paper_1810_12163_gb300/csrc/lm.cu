@@ -73,6 +73,7 @@ constexpr int LMC_P = 16;        // pixels per tile (max_pix is a multiple)
 constexpr int LMC_STAGES = 2;      // tiles in flight with two CTAs per SM (SUBS = 1)
 constexpr int LMC_STAGES_SUB = 4;  // and with one (SUBS > 1)
 constexpr int LMC_SPLIT_MODES = 24;  // |M(u)| bound from which the CTAs of a set share scans
+constexpr int LMC_HEAVY_MODES = 48;  // and from which, at Mahalanobis distances, a cluster may wait for it
 constexpr int LMC_HMAX = 64;
 constexpr int LMC_NV = 31;       // 21 J^T J + 6 J^T r + cost, inlier count, trial cost, Eq. 5 energy
 constexpr int LMC_PS = 33;       // odd stride of the per-thread partials (no bank conflicts)
@@ -1039,7 +1040,8 @@ rl_status launch_lm_cluster(const LmArgs &a, int n, cudaStream_t s) {
     const bool first = a.n_pix <= 2 * a.p.eta;  // round r refines on eta * (r + 2) pixels
     const bool split = a.p.maxm >= LMC_SPLIT_MODES &&
                        lmc_layout(a.p.mpad, a.p.use_cov, LMC_STAGES_SUB).total <= kLmClusterSmemMax;
-    const int sets = split ? lm_sets(a.resident, first, a.n_call, a.n_active < a.n_call) : 1;
+    const bool heavy = a.p.use_cov && a.p.maxm >= LMC_HEAVY_MODES;
+    const int sets = split ? lm_sets(a.resident, first, a.n_call, a.n_active < a.n_call, heavy) : 1;
     if (first) {
         if (sets == 4) return launch_lm_shape<LMC_RANKS_FIRST, 4>(a, n, s);
         if (sets == 2) return launch_lm_shape<LMC_RANKS_FIRST, 2>(a, n, s);

@@ -14,11 +14,10 @@ PROGRAM = r"""
 int main() {
     const rl::LmResident devices[] = {{}, {0, 16, 0}, {8, 16, 8}, {3, 9, 0}};
     for (const rl::LmResident &r : devices)
-        for (int first = 0; first < 2; ++first)
-            for (int sparse = 0; sparse < 2; ++sparse)
-                for (int frames = 1; frames <= 70; ++frames)
-                    std::printf("%d %d %d %d %d %d %d\n", r.first4, r.first2, r.later2, first, sparse, frames,
-                                rl::lm_sets(r, first != 0, frames, sparse != 0));
+        for (int kind = 0; kind < 8; ++kind)
+            for (int frames = 1; frames <= 70; ++frames)
+                std::printf("%d %d %d %d %d %d %d %d\n", r.first4, r.first2, r.later2, kind & 1, kind >> 1 & 1, kind >> 2,
+                            frames, rl::lm_sets(r, kind & 1, frames, kind >> 1 & 1, kind >> 2));
 }
 """
 
@@ -31,10 +30,10 @@ def test_sets_follow_what_the_device_holds(tmp_path):
                     str(exe)], check=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
     rows = [tuple(map(int, ln.split())) for ln in out.splitlines()]
-    assert len(rows) == 4 * 2 * 2 * 70
-    for first4, first2, later2, first, sparse, frames, sets in rows:
+    assert len(rows) == 4 * 8 * 70
+    for first4, first2, later2, first, sparse, heavy, frames, sets in rows:
         held = {4: first4, 2: first2} if first else {2: later2}
-        # at most one waits; where most frames are empty, clusters of 16 (4 x 4, 8 x 2) two deep and of 8 three
+        # none waits; of heavy ones one; where most frames are empty, clusters of 16 (4 x 4, 8 x 2) two deep, of 8 three
         deep = {s: 1 if not sparse else 2 if s * (4 if first else 8) == 16 else 3 for s in held}
-        fits = [s for s, n in held.items() if n > 0 and frames <= deep[s] * (n + 1)]
-        assert sets == max(fits, default=1), (first4, first2, later2, first, sparse, frames)
+        fits = [s for s, n in held.items() if n > 0 and frames <= (deep[s] * (n + 1) if heavy else n)]
+        assert sets == max(fits, default=1), (first4, first2, later2, first, sparse, heavy, frames)
